@@ -34,6 +34,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "exact64.cuh"
 #include "internal.cuh"
 #include "mlp_layout.cuh"
 #include "tc05.cuh"
@@ -82,7 +83,7 @@ struct Zone {
     R r, u, p, t1, t2, c;
 };
 
-__device__ __forceinline__ double div6(double x) { return x / 6.0; }
+__device__ __forceinline__ double div6(double x) { return x64::div6(x); }
 __device__ __forceinline__ float div6(float x) { return x * (1.0f / 6.0f); }
 
 // Load of a field value by the march (and the update's read of a cell's old
@@ -115,16 +116,17 @@ __device__ __forceinline__ Zone<double> prim<double, true>(double rho, double mn
                                                            Counters &cnt)
 {
     Zone<double> z;
-    if (!(rho >= k.rho_floor)) { rho = k.rho_floor; cnt.rare(ENZO_ST_RHO_FLOOR); }
-    double ke = 0.5 * ((mn * mn + m1 * m1) + m2 * m2) / rho;
+    if (!x64::ge_pos(rho, k.rho_floor)) { rho = k.rho_floor; cnt.rare(ENZO_ST_RHO_FLOOR); }
+    const x64::Recip ir = x64::recip(rho);
+    const double ke = x64::div<-1>((mn * mn + m1 * m1) + m2 * m2, rho, ir);
     double p = k.gm1 * (E - ke);
-    if (!(p >= k.p_floor)) { p = k.p_floor; cnt.rare(ENZO_ST_P_FLOOR); }
+    if (!x64::ge_pos(p, k.p_floor)) { p = k.p_floor; cnt.rare(ENZO_ST_P_FLOOR); }
     z.r = rho;
-    z.u = mn / rho;
+    z.u = x64::div(mn, rho, ir);
     z.p = p;
-    z.t1 = m1 / rho;
-    z.t2 = m2 / rho;
-    z.c = sqrt(k.gamma * p / rho);
+    z.t1 = x64::div(m1, rho, ir);
+    z.t2 = x64::div(m2, rho, ir);
+    z.c = x64::sqrt_rn(x64::div(k.gamma * p, rho, ir));
     return z;
 }
 
@@ -194,8 +196,9 @@ __device__ __forceinline__ Zone<double> prim_dual(double rho, double mn, double 
                                                   double &eps)
 {
     Zone<double> z;
-    if (!(rho >= k.rho_floor)) { rho = k.rho_floor; if (COUNT) cnt.rare(ENZO_ST_RHO_FLOOR); }
-    const double ke = 0.5 * ((mn * mn + m1 * m1) + m2 * m2) / rho;
+    if (!x64::ge_pos(rho, k.rho_floor)) { rho = k.rho_floor; if (COUNT) cnt.rare(ENZO_ST_RHO_FLOOR); }
+    const x64::Recip ir = x64::recip(rho);
+    const double ke = x64::div<-1>((mn * mn + m1 * m1) + m2 * m2, rho, ir);
     double p;
     if (E - ke < 1e-3 * E) {
         p = k.gm1 * ge;
@@ -203,14 +206,14 @@ __device__ __forceinline__ Zone<double> prim_dual(double rho, double mn, double 
     } else {
         p = k.gm1 * (E - ke);
     }
-    if (!(p >= k.p_floor)) { p = k.p_floor; if (COUNT) cnt.rare(ENZO_ST_P_FLOOR); }
+    if (!x64::ge_pos(p, k.p_floor)) { p = k.p_floor; if (COUNT) cnt.rare(ENZO_ST_P_FLOOR); }
     z.r = rho;
-    z.u = mn / rho;
+    z.u = x64::div(mn, rho, ir);
     z.p = p;
-    z.t1 = m1 / rho;
-    z.t2 = m2 / rho;
-    z.c = sqrt(k.gamma * p / rho);
-    eps = ge / rho;
+    z.t1 = x64::div(m1, rho, ir);
+    z.t2 = x64::div(m2, rho, ir);
+    z.c = x64::sqrt_rn(x64::div(k.gamma * p, rho, ir));
+    eps = x64::div(ge, rho, ir);
     return z;
 }
 
@@ -274,6 +277,47 @@ __device__ __forceinline__ R limited_slope(R qm, R q0, R qp)
     return r;
 }
 
+// FP64: the same values with the comparisons and the exact scalings by 2 on
+// the integer pipe.  With both one-sided differences of middle magnitude their
+// product is normal, so its sign is theirs, and the centred difference, no
+// smaller than either, is of the same sign.
+template <>
+__device__ __forceinline__ double limited_slope<double>(double qm, double q0, double qp)
+{
+    const double dl = q0 - qm;
+    const double dr = qp - q0;
+    if (x64::middle(dl) && x64::middle(dr)) {
+        if ((int)(x64::hi32(dl) ^ x64::hi32(dr)) < 0) return 0.0;
+        const double dc = qp - qm;
+        const uint64_t l = x64::mag(dl), r = x64::mag(dr);
+        const uint64_t a = x64::mag(dc) - 0x0010000000000000ull;
+        const uint64_t b = (l < r ? l : r) + 0x0010000000000000ull;
+        return x64::from_bits((a < b ? a : b) | (x64::bits(dl) & 0x8000000000000000ull));
+    }
+    double r = 0.0;
+    if (dl * dr > 0.0) {
+        const double dc = 0.5 * (qp - qm);
+        const double a = fabs(dc), b = 2.0 * fabs(dl), e = 2.0 * fabs(dr);
+        double m = a < b ? a : b;
+        m = m < e ? m : e;
+        r = dc >= 0.0 ? m : -m;
+    }
+    return r;
+}
+
+// Value at the interface between zones a and b with limited slopes da, db.
+template <class R>
+__device__ __forceinline__ R face_value(R a, R b, R da, R db)
+{
+    return (R)0.5 * (a + b) - div6(db - da);
+}
+// FP64: the half is exact, so one fused operation rounds as the two do.
+template <>
+__device__ __forceinline__ double face_value<double>(double a, double b, double da, double db)
+{
+    return __fma_rn(0.5, a + b, -div6(db - da));
+}
+
 // Monotone parabola of a zone (CW84 1.10): edges ql, qr in, (qL, Delta q, q6) out.
 template <class R>
 __device__ __forceinline__ void parabola(R qs, R ql, R qr, R &oL, R &oR, R &d, R &q6)
@@ -291,6 +335,52 @@ __device__ __forceinline__ void parabola(R qs, R ql, R qr, R &oL, R &oR, R &d, R
     oR = qr;
     d = qr - ql;
     q6 = (R)6 * (qs - (R)0.5 * (ql + qr));
+}
+
+// FP64: the same values.  The sign of the first product is its factors', and
+// the overshoot tests compare |q6| with |Delta q|: the products order as they
+// do unless they are within 16 ulp, where the products themselves decide.
+template <>
+__device__ __forceinline__ void parabola<double>(double qs, double ql, double qr, double &oL, double &oR, double &d,
+                                                 double &q6)
+{
+    const double er = qr - qs, el = qs - ql;
+    bool flat;
+    if (x64::middle(er) && x64::middle(el)) flat = (int)(x64::hi32(er) ^ x64::hi32(el)) < 0;
+    else flat = er * el <= 0.0;
+    double dd = qr - ql;
+    double qq = 6.0 * __fma_rn(-0.5, ql + qr, qs);
+    bool fl = false, fr = false;
+    if (flat) {
+        ql = qs;
+        qr = qs;
+    } else {
+        const long long diff = (long long)(x64::mag(qq) - x64::mag(dd));
+        if (x64::middle(dd) && x64::middle(qq) && (diff > 16 || diff < -16)) {
+            const bool same = (int)(x64::hi32(dd) ^ x64::hi32(qq)) >= 0;
+            fl = diff > 0 && same;
+            fr = diff > 0 && !same;
+        } else {
+            fl = dd * qq > dd * dd;
+            fr = !fl && -(dd * dd) > dd * qq;
+        }
+        const double e = fl ? qr : ql;
+        if (fl || fr) {
+            const double v = __fma_rn(-2.0, e, 3.0 * qs);
+            if (fl) ql = v;
+            else qr = v;
+        }
+    }
+    oL = ql;
+    oR = qr;
+    if (fl || fr) {
+        dd = qr - ql;
+        qq = 6.0 * __fma_rn(-0.5, ql + qr, qs);
+    } else if (flat) {
+        dd = qq = x64::finite(qs) ? 0.0 : qs - qs;
+    }
+    d = dd;
+    q6 = qq;
 }
 
 // Averages of the zone parabola over the fraction sig of the zone adjacent to
@@ -313,50 +403,134 @@ __device__ __forceinline__ R avg_left(R qL, R d, R q6, R sig)
 // moving toward the edge (u+c or u-c) averaged over its domain, else the edge
 // value; the others enter through beta corrections of the linearised
 // Lagrangian characteristic relations dp +- C du = 0, dp + C^2 d(1/rho) = 0.
-template <class R, int SIDE>
-__device__ __forceinline__ void trace_exact(const R qL[5], const R qR[5], const R d[5], const R q6[5],
-                                            R u, R c, R dtdx, const Consts<R> &k, R out[5])
+// SIDE = +1 / -1 together in FP64, every operation in the order of these
+// formulas (the reference's):
+//   C^2 = gamma p_ref rho_ref; beta of a wave that reaches the edge, with
+//   averages I over its domain: beta_+ = -(1/2C) ((u_ref - I u) + (p_ref - I p) / C),
+//   beta_- = (1/2C) ((u_ref - I u) - (p_ref - I p) / C),
+//   beta_0 = (p_ref - I p) / C^2 + 1/rho_ref - 1/(I rho);
+//   p = p_ref + C^2 (beta_+ + beta_-), u = u_ref + C (beta_+ - beta_-),
+//   1/rho = 1/rho_ref - ((beta_+ + beta_-) + beta_0).
+// What the FP64 pipe is spared: the reference wave's own beta is a zero (it
+// measures the reference against itself) unless the pressure floor cut the
+// reference; the entropy wave reaches one edge, the right one for u > 0, the
+// left one for u < 0, so its averages are formed once, for that edge (a left
+// edge through the mirrored Delta q), and neighbouring threads with opposite
+// velocities do not take two branches; the slow acoustic wave likewise, where
+// |u| > c.
+struct Edge64 {
+    double r, u, p;       // reference state
+    double bp, bm;        // beta_+, beta_-
+    bool plain;           // both are zeros that change nothing
+};
+
+__device__ __forceinline__ double avg64(double edge, double d, double q6, double s, double w)
 {
-    const R lam0 = u - c, lam1 = u, lam2 = u + c;
-    const bool r0 = SIDE > 0 ? lam0 > (R)0 : lam0 < (R)0;
-    const bool r1 = SIDE > 0 ? lam1 > (R)0 : lam1 < (R)0;
-    const bool r2 = SIDE > 0 ? lam2 > (R)0 : lam2 < (R)0;
-    const R s0 = SIDE > 0 ? lam0 * dtdx : -lam0 * dtdx;
-    const R s1 = SIDE > 0 ? lam1 * dtdx : -lam1 * dtdx;
-    const R s2 = SIDE > 0 ? lam2 * dtdx : -lam2 * dtdx;
-#define ENZO_I(SIG, V) (SIDE > 0 ? avg_right<R>(qR[V], d[V], q6[V], SIG) : avg_left<R>(qL[V], d[V], q6[V], SIG))
-    const bool rref = SIDE > 0 ? r2 : r0;
-    const R sref = SIDE > 0 ? s2 : s0;
-    const R *edge = SIDE > 0 ? qR : qL;
-    R rho_ref, u_ref, p_ref;
-    if (rref) {
-        rho_ref = ENZO_I(sref, 0);
-        u_ref = ENZO_I(sref, 1);
-        p_ref = ENZO_I(sref, 2);
-    } else {
-        rho_ref = edge[0];
-        u_ref = edge[1];
-        p_ref = edge[2];
+    return __fma_rn(-0.5, s * (d - w * q6), edge);
+}
+
+template <int SIDE>
+__device__ __forceinline__ Edge64 trace_ref64(const double e[5], const double d[5], const double q6[5], double lam,
+                                              double slam, const Consts<double> &k)
+{
+    // lam: the fast wave's speed toward this edge; slam: |lam| dt/dx
+    Edge64 o;
+    const bool reach = x64::gt0(lam);
+    double pa = e[2];
+    o.r = e[0];
+    o.u = e[1];
+    if (reach) {
+        const double w = 1.0 - slam * (2.0 / 3.0);
+        o.r = avg64(e[0], SIDE > 0 ? d[0] : -d[0], q6[0], slam, w);
+        o.u = avg64(e[1], SIDE > 0 ? d[1] : -d[1], q6[1], slam, w);
+        pa = avg64(e[2], SIDE > 0 ? d[2] : -d[2], q6[2], slam, w);
     }
-    if (!(rho_ref > k.rho_floor)) rho_ref = k.rho_floor;
-    if (!(p_ref > k.p_floor)) p_ref = k.p_floor;
-    const R C = sqrt(k.gamma * p_ref * rho_ref);
-    R bp = (R)0, bm = (R)0, b0 = (R)0;
-    if (r2) bp = -((R)0.5 / C) * ((u_ref - ENZO_I(s2, 1)) + (p_ref - ENZO_I(s2, 2)) / C);
-    if (r0) bm = ((R)0.5 / C) * ((u_ref - ENZO_I(s0, 1)) - (p_ref - ENZO_I(s0, 2)) / C);
-    if (r1) b0 = (p_ref - ENZO_I(s1, 2)) / (C * C) + (R)1 / rho_ref - (R)1 / ENZO_I(s1, 0);
-    R p = p_ref + (C * C) * (bp + bm);
-    const R un = u_ref + C * (bp - bm);
-    const R tau = (R)1 / rho_ref - ((bp + bm) + b0);
-    R rho = (R)1 / tau;
-    if (!(rho > k.rho_floor)) rho = k.rho_floor;
-    if (!(p > k.p_floor)) p = k.p_floor;
-    out[0] = rho;
-    out[1] = un;
-    out[2] = p;
-    out[3] = r1 ? ENZO_I(s1, 3) : edge[3];
-    out[4] = r1 ? ENZO_I(s1, 4) : edge[4];
-#undef ENZO_I
+    o.p = pa;
+    if (!x64::gt_pos(o.r, k.rho_floor)) o.r = k.rho_floor;
+    const bool cut = !x64::gt_pos(o.p, k.p_floor);
+    if (cut) o.p = k.p_floor;
+    o.bp = SIDE > 0 && reach ? -0.0 : 0.0;
+    o.bm = 0.0;
+    o.plain = true;
+    if (reach && (cut || !x64::finite(o.u) || !x64::finite(o.p))) {
+        const double C = sqrt(k.gamma * o.p * o.r), h = 0.5 / C, t = (o.p - pa) / C;
+        if (SIDE > 0) o.bp = -(h * ((o.u - o.u) + t));
+        else o.bm = h * ((o.u - o.u) - t);
+        o.plain = false;
+    }
+    return o;
+}
+
+__device__ __forceinline__ void trace_exact(const double qL[5], const double qR[5], const double d[5],
+                                            const double q6[5], double u, double c, double dtdx,
+                                            const Consts<double> &k, double outR[5], double outL[5])
+{
+    // outR: the right state of the left edge (SIDE = -1); outL: the left state of the right edge
+    const double lm = u - c, lp = u + c;
+    const double sm = lm * dtdx, s1 = fabs(u * dtdx), sp = lp * dtdx;
+    Edge64 er = trace_ref64<+1>(qR, d, q6, lp, sp, k);
+    Edge64 el = trace_ref64<-1>(qL, d, q6, -lm, -sm, k);
+    const bool right = x64::gt0(u), left = x64::lt0(u);
+    // entropy wave and slow acoustic wave: the edge they reach
+    double b0 = 0.0, t1 = 0.0, t2 = 0.0;
+    const double C2r = k.gamma * er.p * er.r, C2l = k.gamma * el.p * el.r;
+    const double Cr = x64::sqrt_rn(C2r), Cl = x64::sqrt_rn(C2l);
+    er.plain = er.plain && x64::finite(Cr);
+    el.plain = el.plain && x64::finite(Cl);
+    const double ir = x64::div(1.0, er.r), il = x64::div(1.0, el.r);
+    if (right || left) {
+        const double w = 1.0 - s1 * (2.0 / 3.0);
+        const double C = right ? Cr : Cl, p = right ? er.p : el.p;
+        const double ar = avg64(right ? qR[0] : qL[0], x64::neg_if(left, d[0]), q6[0], s1, w);
+        const double ap = avg64(right ? qR[2] : qL[2], x64::neg_if(left, d[2]), q6[2], s1, w);
+        t1 = avg64(right ? qR[3] : qL[3], x64::neg_if(left, d[3]), q6[3], s1, w);
+        t2 = avg64(right ? qR[4] : qL[4], x64::neg_if(left, d[4]), q6[4], s1, w);
+        b0 = x64::div(p - ap, C * C) + (right ? ir : il) - x64::div(1.0, ar);
+        const bool slow = right ? x64::gt0(lm) : x64::lt0(lp);
+        if (slow) {
+            const double ss = fabs(right ? sm : sp), ws = 1.0 - ss * (2.0 / 3.0);
+            const double au = avg64(right ? qR[1] : qL[1], x64::neg_if(left, d[1]), q6[1], ss, ws);
+            const double as = avg64(right ? qR[2] : qL[2], x64::neg_if(left, d[2]), q6[2], ss, ws);
+            const x64::Recip iC = x64::recip(C);
+            const double h = x64::div(0.5, C, iC), t = x64::div(p - as, C, iC);
+            const double du = (right ? er.u : el.u) - au;
+            const double b = h * (right ? du - t : du + t);
+            if (right) {
+                er.bm = b;
+                er.plain = false;
+            } else {
+                el.bp = -b;
+                el.plain = false;
+            }
+        }
+    }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+        const Edge64 &e = side ? er : el;
+        const double C = side ? Cr : Cl, i = side ? ir : il;
+        const bool here = side ? right : left;
+        double *out = side ? outL : outR;
+        double p = e.p, un, tau;
+        const double b = here ? b0 : 0.0;
+        if (e.plain) {
+            // adding +0 turns -0 into +0; adding -0 changes nothing
+            un = x64::bits(e.u) == 0x8000000000000000ull && x64::bits(e.bp) == 0 ? 0.0 : e.u;
+            tau = i - b;
+        } else {
+            const double sum = e.bp + e.bm;
+            p = e.p + (C * C) * sum;
+            un = e.u + C * (e.bp - e.bm);
+            tau = i - (sum + b);
+        }
+        double rho = x64::div(1.0, tau);
+        if (!x64::gt_pos(rho, k.rho_floor)) rho = k.rho_floor;
+        if (!x64::gt_pos(p, k.p_floor)) p = k.p_floor;
+        out[0] = rho;
+        out[1] = un;
+        out[2] = p;
+        out[3] = here ? t1 : (side ? qR[3] : qL[3]);
+        out[4] = here ? t2 : (side ? qR[4] : qL[4]);
+    }
 }
 
 // The same characteristic state in FP32, arranged for fewer operations (the
@@ -419,12 +593,17 @@ __device__ __forceinline__ void trace_f(const float qL[5], const float qR[5], co
 #undef ENZO_AVG
 }
 
-template <class R, int SIDE>
-__device__ __forceinline__ void trace(const R qL[5], const R qR[5], const R d[5], const R q6[5],
-                                      R u, R c, R dtdx, const Consts<R> &k, R out[5])
+// Right state of the zone's left edge (sR) and left state of its right edge (sL).
+template <class R>
+__device__ __forceinline__ void trace(const R qL[5], const R qR[5], const R d[5], const R q6[5], R u, R c, R dtdx,
+                                      const Consts<R> &k, R sR[5], R sL[5])
 {
-    if constexpr (std::is_same<R, float>::value) trace_f<SIDE>(qL, qR, d, q6, u, c, dtdx, k, out);
-    else trace_exact<R, SIDE>(qL, qR, d, q6, u, c, dtdx, k, out);
+    if constexpr (std::is_same<R, float>::value) {
+        trace_f<-1>(qL, qR, d, q6, u, c, dtdx, k, sR);
+        trace_f<+1>(qL, qR, d, q6, u, c, dtdx, k, sL);
+    } else {
+        trace_exact(qL, qR, d, q6, u, c, dtdx, k, sR, sL);
+    }
 }
 
 // A passive variable (eps of the dual-energy option) traced to one edge of its
@@ -437,56 +616,6 @@ __device__ __forceinline__ R trace_passive(R qL, R qR, R d, R q6, R u, R dtdx)
     const R s1 = SIDE > 0 ? u * dtdx : -u * dtdx;
     if (!r1) return SIDE > 0 ? qR : qL;
     return SIDE > 0 ? avg_right<R>(qR, d, q6, s1) : avg_left<R>(qL, d, q6, s1);
-}
-
-// Lagrangian shock speed W and |dp/du| of the shock curve Z = 2W^3/(W^2+C^2).
-template <class R>
-__device__ __forceinline__ void shock_side(R ps, R p, R C, const Consts<R> &k, R &W, R &Z)
-{
-    R rad = (R)1 + k.gp1o2g * (ps / p - (R)1);
-    if (rad < (R)1e-6) rad = (R)1e-6;
-    W = C * sqrt(rad);
-    Z = (R)2 * W * W * W / (W * W + C * C);
-}
-
-template <class R>
-__device__ __forceinline__ R plain_guess(R rl, R ul, R pl, R rr, R ur, R pr, const Consts<R> &k)
-{
-    const R CL = sqrt(k.gamma * pl * rl);
-    const R CR = sqrt(k.gamma * pr * rr);
-    const R p0 = (CR * pl + CL * pr + CL * CR * (ul - ur)) / (CL + CR);
-    return p0 > k.p_floor ? p0 : k.p_floor;
-}
-
-// Newton iteration on f(p*) = u*_R - u*_L = 0 (two-shock, Sec. 4.1.2).  Stops
-// when |f| <= tol (|u_L| + |u_R| + c_L + c_R), when the update no longer moves
-// p*, or (FP32 only) when the update is below a few ulp of p*.
-template <class R>
-__device__ __forceinline__ int newton(R rl, R ul, R pl, R rr, R ur, R pr, R p0,
-                                      const Consts<R> &k, R &pstar, bool &conv)
-{
-    const R CL = sqrt(k.gamma * pl * rl);
-    const R CR = sqrt(k.gamma * pr * rr);
-    const R uscale = (fabs(ul) + fabs(ur)) + (sqrt(k.gamma * pl / rl) + sqrt(k.gamma * pr / rr));
-    R ps = p0 > k.p_floor ? p0 : k.p_floor;
-    conv = false;
-    int it;
-    for (it = 0; it < k.nmax; ++it) {
-        R WL, ZL, WR, ZR;
-        shock_side(ps, pl, CL, k, WL, ZL);
-        shock_side(ps, pr, CR, k, WR, ZR);
-        const R usL = ul - (ps - pl) / WL;
-        const R usR = ur + (ps - pr) / WR;
-        const R f = usR - usL;
-        if (fabs(f) <= k.tol * uscale) { conv = true; break; }
-        R pn = ps - ZL * ZR * f / (ZL + ZR);
-        if (!(pn > k.p_floor)) pn = k.p_floor;
-        if (pn == ps) { conv = true; break; }
-        if (sizeof(R) == 4 && fabs(pn - ps) <= k.step_tol * pn) { ps = pn; conv = true; ++it; break; }
-        ps = pn;
-    }
-    pstar = ps;
-    return it;
 }
 
 template <class R>
@@ -616,83 +745,127 @@ __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float
     return o;
 }
 
-// Two-shock solve and sampling of the self-similar solution at x/t = 0.
-template <class R>
-__device__ __forceinline__ RiemannOut<R> riemann_exact(R rl, R ul, R pl, R rr, R ur, R pr, R pguess,
-                                                       const Consts<R> &k, Counters &cnt)
+// One side of the two-shock problem (Sec. 4.1.2) at pressure ps: Lagrangian
+// shock speed W = C sqrt(rad), rad = 1 + (gamma+1)/(2 gamma) (ps/p - 1) (at
+// least 1e-6), W^2, |dp/du| of the shock curve Z = 2 W^3 / (W^2 + C^2), and
+// (ps - p) / W.
+struct Side64 {
+    double W, W2, Z, du;
+};
+
+__device__ __forceinline__ Side64 shock_side64(double ps, double p, double C, double CC, const x64::Recip &ip,
+                                               const Consts<double> &k)
 {
-    RiemannOut<R> o;
-    R ps;
-    bool conv;
-    int it;
-    if (pguess > (R)0) {
-        it = newton(rl, ul, pl, rr, ur, pr, pguess, k, ps, conv);
-        if (!conv) {
-            cnt.restarts++;
-            it += newton(rl, ul, pl, rr, ur, pr, plain_guess(rl, ul, pl, rr, ur, pr, k), k, ps, conv);
+    Side64 o;
+    double rad = 1.0 + k.gp1o2g * (x64::div(ps, p, ip) - 1.0);
+    if (x64::lt_pos(rad, 1e-6)) rad = 1e-6;
+    o.W = C * x64::sqrt_rn(rad);
+    o.W2 = o.W * o.W;
+    const double den = o.W2 + CC;
+    o.Z = x64::div<1>(o.W2 * o.W, den, x64::recip(den));
+    o.du = x64::div(ps - p, o.W);
+    return o;
+}
+
+// Two-shock solve and sampling of the self-similar solution at x/t = 0, FP64.
+// Newton iteration on f(p*) = u*_R - u*_L = 0 stops when |f| <= tol (|u_L| +
+// |u_R| + c_L + c_R) or when the update no longer moves p*; a given guess that
+// reaches the cap restarts once from the plain guess.  Every value that
+// reaches the results is formed in the order of these formulas.  What the FP64
+// pipe is spared: the accepted iterate's side quantities serve the star state
+// without a second evaluation; the stopping bound is first tested in FP32, and
+// formed in FP64 only where |f| is within 1e-4 of it; the upwind side alone is
+// sampled, with velocities mirrored for the right one, so that a warp takes at
+// most two branches (shock, rarefaction) instead of four.
+__device__ __forceinline__ RiemannOut<double> riemann_exact(double rl, double ul, double pl, double rr, double ur,
+                                                            double pr, double pguess, const Consts<double> &k,
+                                                            Counters &cnt)
+{
+    RiemannOut<double> o;
+    const double gpl = k.gamma * pl, gpr = k.gamma * pr;
+    const double CL = x64::sqrt_rn(gpl * rl), CR = x64::sqrt_rn(gpr * rr);
+    const double CCL = CL * CL, CCR = CR * CR;
+    const x64::Recip ipl = x64::recip(pl), ipr = x64::recip(pr);
+    // the stopping bound in FP32, as an interval; empty (0, inf) out of FP32's
+    // comfortable range
+    double tlo, thi;
+    {
+        const float us = (fabsf(d2f_rz(ul)) + fabsf(d2f_rz(ur))) +
+                         (sqrtf(d2f_rz(gpl) / d2f_rz(rl)) + sqrtf(d2f_rz(gpr) / d2f_rz(rr)));
+        const float t = us * d2f_rz(k.tol);
+        const bool ok = us > 1e-12f && us < 1e30f && t > 1e-30f;
+        tlo = ok ? f2d_exact(t * 0.9999f) : 0.0;
+        thi = ok ? f2d_exact(t * 1.0001f) : __longlong_as_double(0x7ff0000000000000ll);
+    }
+    double ps = pguess;
+    bool restarted = !(pguess > 0.0);
+    if (!restarted) ps = x64::gt_pos(pguess, k.p_floor) ? pguess : k.p_floor;
+    bool conv = false, plain = restarted;
+    int it = 0, base = 0;
+    Side64 L, R;
+    double usL, usR, ZZ;
+    for (;;) {
+        if (plain) {
+            const double p0 = x64::div((CR * pl + CL * pr) + (CL * CR) * (ul - ur), CL + CR);
+            ps = x64::gt_pos(p0, k.p_floor) ? p0 : k.p_floor;
+            plain = false;
         }
-    } else {
-        it = newton(rl, ul, pl, rr, ur, pr, plain_guess(rl, ul, pl, rr, ur, pr, k), k, ps, conv);
+        L = shock_side64(ps, pl, CL, CCL, ipl, k);
+        R = shock_side64(ps, pr, CR, CCR, ipr, k);
+        usL = ul - L.du;
+        usR = ur + R.du;
+        ZZ = L.Z + R.Z;
+        if (it - base >= k.nmax) {
+            if (restarted) break;
+            restarted = plain = true;
+            cnt.restarts++;
+            base = it;
+            continue;
+        }
+        const double f = usR - usL;
+        const uint64_t af = x64::mag(f);
+        bool stop = af <= x64::bits(tlo);
+        if (!stop && !(af > x64::bits(thi))) {
+            const double uscale = (fabs(ul) + fabs(ur)) + (sqrt(gpl / rl) + sqrt(gpr / rr));
+            stop = fabs(f) <= k.tol * uscale;
+        }
+        if (stop) { conv = true; break; }
+        double pn = ps - x64::div((L.Z * R.Z) * f, ZZ);
+        if (!x64::gt_pos(pn, k.p_floor)) pn = k.p_floor;
+        if (x64::bits(pn) == x64::bits(ps)) { conv = true; break; }
+        ps = pn;
+        ++it;
     }
     o.iters = it;
     o.conv = conv;
-    const R CL = sqrt(k.gamma * pl * rl);
-    const R CR = sqrt(k.gamma * pr * rr);
-    R WL, ZL, WR, ZR;
-    shock_side(ps, pl, CL, k, WL, ZL);
-    shock_side(ps, pr, CR, k, WR, ZR);
-    const R usL = ul - (ps - pl) / WL;
-    const R usR = ur + (ps - pr) / WR;
-    const R us = (ZL * usL + ZR * usR) / (ZL + ZR);
-    R rsL = (R)1 / ((R)1 / rl - (ps - pl) / (WL * WL));
-    R rsR = (R)1 / ((R)1 / rr - (ps - pr) / (WR * WR));
-    if (!(rsL > k.rho_floor)) rsL = k.rho_floor;
-    if (!(rsR > k.rho_floor)) rsR = k.rho_floor;
+    const double us = x64::div(L.Z * usL + R.Z * usR, ZZ);
     o.ustar = us;
     o.pstar = ps;
-    R rho, u, p;
-    if (us >= (R)0) {
-        if (ps > pl) {
-            const R S = ul - WL / rl;
-            if (S >= (R)0) { rho = rl; u = ul; p = pl; }
-            else { rho = rsL; u = us; p = ps; }
-        } else {
-            const R cl = sqrt(k.gamma * pl / rl);
-            const R cs = sqrt(k.gamma * ps / rsL);
-            const R Sh = ul - cl;
-            const R St = us - cs;
-            if (Sh >= (R)0) { rho = rl; u = ul; p = pl; }
-            else if (St <= (R)0) { rho = rsL; u = us; p = ps; }
-            else {
-                const R f = -Sh / (St - Sh);
-                rho = rl + f * (rsL - rl);
-                u = ul + f * (us - ul);
-                p = pl + f * (ps - pl);
-            }
-        }
+    const bool left = x64::ge0(us);
+    const double r = left ? rl : rr, u = left ? ul : ur, p = left ? pl : pr;
+    const double W = left ? L.W : R.W, W2 = left ? L.W2 : R.W2;
+    const x64::Recip ir = x64::recip(r);
+    double rs = x64::div(1.0, x64::div(1.0, r, ir) - x64::div(ps - p, W2));
+    if (!x64::gt_pos(rs, k.rho_floor)) rs = k.rho_floor;
+    const double um = x64::neg_if(!left, u), usm = x64::neg_if(!left, us);
+    bool inside;                                   // the star state, else the side state
+    if (ps > p) {
+        inside = !x64::ge0(um - x64::div(W, r, ir));
     } else {
-        if (ps > pr) {
-            const R S = ur + WR / rr;
-            if (S <= (R)0) { rho = rr; u = ur; p = pr; }
-            else { rho = rsR; u = us; p = ps; }
-        } else {
-            const R cr = sqrt(k.gamma * pr / rr);
-            const R cs = sqrt(k.gamma * ps / rsR);
-            const R Sh = ur + cr;
-            const R St = us + cs;
-            if (Sh <= (R)0) { rho = rr; u = ur; p = pr; }
-            else if (St >= (R)0) { rho = rsR; u = us; p = ps; }
-            else {
-                const R f = Sh / (Sh - St);
-                rho = rr + f * (rsR - rr);
-                u = ur + f * (us - ur);
-                p = pr + f * (ps - pr);
-            }
+        const double Sh = um - x64::sqrt_rn(x64::div(left ? gpl : gpr, r, ir));
+        const double St = usm - x64::sqrt_rn(x64::div(k.gamma * ps, rs));
+        inside = !x64::ge0(Sh);
+        if (inside && !x64::le0(St)) {
+            const double f = x64::div(-Sh, St - Sh);
+            o.rho = r + f * (rs - r);
+            o.u = u + f * (us - u);
+            o.p = p + f * (ps - p);
+            return o;
         }
     }
-    o.rho = rho;
-    o.u = u;
-    o.p = p;
+    o.rho = inside ? rs : r;
+    o.u = inside ? us : u;
+    o.p = inside ? ps : p;
     return o;
 }
 
@@ -701,7 +874,7 @@ __device__ __forceinline__ RiemannOut<R> riemann(R rl, R ul, R pl, R rr, R ur, R
                                                  const Consts<R> &k, Counters &cnt)
 {
     if constexpr (std::is_same<R, float>::value) return riemann_f(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
-    else return riemann_exact<R>(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
+    else return riemann_exact(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
 }
 
 // Physical flux of the split 1-D equations (Sec. 4.1): mass, normal momentum,
@@ -717,6 +890,19 @@ __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Con
     const R eint = p * k.gm1inv;
     const R ke = (R)0.5 * rho * ((u * u + t1 * t1) + t2 * t2);
     F[4] = u * ((eint + ke) + p);
+}
+
+// FP64: the half is exact, so one fused operation adds the kinetic energy.
+template <>
+__device__ __forceinline__ void phys_flux<double>(double rho, double u, double p, double t1, double t2,
+                                                  const Consts<double> &k, double F[5])
+{
+    const double mflux = rho * u;
+    F[0] = mflux;
+    F[1] = mflux * u + p;
+    F[2] = mflux * t1;
+    F[3] = mflux * t2;
+    F[4] = u * (__fma_rn(0.5, rho * ((u * u + t1 * t1) + t2 * t2), p * k.gm1inv) + p);
 }
 
 // HLL flux with Davis wave-speed bounds from first-order zone states (fallback).
@@ -1399,8 +1585,8 @@ struct Marcher {
             gpend.ok = ok;
         }
         if (!active) return;
-        if (fb && (EXT && a.mp.fallback == 2 ? fails_state(u) : !(u[0] > 0.0))) cnt.rare(ENZO_ST_NEG_AFTER);
-        if (u[0] != u[0] || u[4] != u[4]) cnt.rare(ENZO_ST_NAN);
+        if (fb && (EXT && a.mp.fallback == 2 ? fails_state(u) : !x64::gt0(u[0]))) cnt.rare(ENZO_ST_NEG_AFTER);
+        if (x64::is_nan(u[0]) || x64::is_nan(u[4])) cnt.rare(ENZO_ST_NAN);
         _Pragma("unroll") for (int v = 0; v < 5; ++v) const_cast<double *>(a.U[map[v]])[idx] = u[v];
     }
 
@@ -1611,8 +1797,8 @@ struct Marcher {
             if (kk >= 3) {
                 R qfcur[5];
                 _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                    qfcur[v] = (R)0.5 * (zv(zm2, v) + zv(zm1, v)) - div6(dcur[v] - dprev[v]);
-                const R qfce = dual ? (R)0.5 * (e2 + e1) - div6(dce - dep) : (R)0;
+                    qfcur[v] = face_value<R>(zv(zm2, v), zv(zm1, v), dprev[v], dcur[v]);
+                const R qfce = dual ? face_value<R>(e2, e1, dep, dce) : (R)0;
                 if (kk >= 4) {
                     R sRe = (R)0, sLen = (R)0;   // eps traced to the left / right edge of zone kk-2
                     // parabola of zone kk-2 (its edges: qfprev on the left, qfcur on the right)
@@ -1638,8 +1824,7 @@ struct Marcher {
                         _Pragma("unroll") for (int v = 0; v < 5; ++v) parabola<R>(zv(zm2, v), qfprev[v], qfcur[v], pL[v], pR[v], pd[v], p6[v]);
                     }
                     R sR[5], sLnew[5];
-                    trace<R, -1>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sR);
-                    trace<R, +1>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sLnew);
+                    trace<R>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sR, sLnew);
                     if (kk >= 5) {
                         // Riemann problem at interface (kk-3)+1/2
                         if (a.log) log_states(kk, sLprev, sR);
@@ -1682,7 +1867,7 @@ struct Marcher {
                                     bad = (sizeof(R) == 8 || dual || !clearly_ok(zm3, Fgprev, Fg, dtdx))
                                               ? fails_full(c, Fgprev, Fg, dtdx, dtdx64) : false;
                                 } else if (sizeof(R) == 8) {
-                                    bad = !(cell_update(rho_old<RING>(c), dtdx64, (double)Fgprev[0], (double)Fg[0]) > 0.0);
+                                    bad = !x64::gt0(cell_update(rho_old<RING>(c), dtdx64, (double)Fgprev[0], (double)Fg[0]));
                                 } else {
                                     // FP32 screen; cells near zero are decided in FP64
                                     const R rt = rho3 + dtdx * (Fgprev[0] - Fg[0]);
@@ -1831,14 +2016,13 @@ struct Marcher {
                 if (kk >= 3) {
                     R qfcur[5];
                     _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                        qfcur[v] = (R)0.5 * (zv(zm2, v) + zv(zm1, v)) - div6(dcur[v] - dprev[v]);
+                        qfcur[v] = face_value<R>(zv(zm2, v), zv(zm1, v), dprev[v], dcur[v]);
                     if (kk >= 4) {
                         // parabola of zone kk-2 (its edges: qfprev on the left, qfcur on the right)
                         R pL[5], pR[5], pd[5], p6[5];
                         _Pragma("unroll") for (int v = 0; v < 5; ++v) parabola<R>(zv(zm2, v), qfprev[v], qfcur[v], pL[v], pR[v], pd[v], p6[v]);
                         R sR[5], sLnew[5];
-                        trace<R, -1>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sR);
-                        trace<R, +1>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sLnew);
+                        trace<R>(pL, pR, pd, p6, zm2.u, zm2.c, dtdx, k, sR, sLnew);
                         if (kk >= 5) {
                             // interface (kk-3)+1/2: left state from zone kk-3, right from kk-2
                             if (a.log) log_states(kk, sLprev, sR);
@@ -2116,7 +2300,8 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
         const int64_t ncell = (int64_t)nx * ny * P.n[2];
         const int64_t first = (int64_t)(tile - a.prefix[pi]) * kCflTile;
         const int64_t N0 = nx + 2 * P.ng, N1 = ny + 2 * P.ng;
-        const double idx0 = 1.0 / P.dx[0], idx1 = 1.0 / P.dx[1], idx2 = 1.0 / P.dx[2];
+        const float idx0 = (float)(1.0 / P.dx[0]), idx1 = (float)(1.0 / P.dx[1]), idx2 = (float)(1.0 / P.dx[2]);
+        const x64::Recip id0 = x64::recip(P.dx[0]), id1 = x64::recip(P.dx[1]), id2 = x64::recip(P.dx[2]);
         for (int t = threadIdx.x; t < kCflTile; t += blockDim.x) {
             const int64_t cell = first + t;
             if (cell >= ncell) break;
@@ -2127,14 +2312,16 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
             const int64_t idx = P.off + (i + P.ng) + N0 * ((j + P.ng) + N1 * (int64_t)(kz + P.ng));
             if (sizeof(R) == 8) {
                 double rho = a.U[0][idx];
-                if (!(rho >= a.rho_floor)) rho = a.rho_floor;
+                if (!x64::ge_pos(rho, a.rho_floor)) rho = a.rho_floor;
                 const double mx = a.U[1][idx], my = a.U[2][idx], mz = a.U[3][idx];
-                const double ke = 0.5 * ((mx * mx + my * my) + mz * mz) / rho;
+                const x64::Recip ir = x64::recip(rho);
+                const double ke = x64::div<-1>((mx * mx + my * my) + mz * mz, rho, ir);
                 double p = (a.gamma - 1.0) * (a.U[4][idx] - ke);
-                if (!(p >= a.p_floor)) p = a.p_floor;
-                const double c = sqrt(a.gamma * p / rho);
-                const double r = ((c + fabs(mx / rho)) / P.dx[0] + (c + fabs(my / rho)) / P.dx[1]) +
-                                 (c + fabs(mz / rho)) / P.dx[2];
+                if (!x64::ge_pos(p, a.p_floor)) p = a.p_floor;
+                const double c = x64::sqrt_rn(x64::div(a.gamma * p, rho, ir));
+                const double r = (x64::div(c + fabs(x64::div(mx, rho, ir)), P.dx[0], id0) +
+                                  x64::div(c + fabs(x64::div(my, rho, ir)), P.dx[1], id1)) +
+                                 x64::div(c + fabs(x64::div(mz, rho, ir)), P.dx[2], id2);
                 best = r > best ? r : best;
             } else {
                 Counters quiet;
@@ -2146,8 +2333,8 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
                 k.eta_eke = 0.05f;
                 const Zone<float> z = prim_f<false>(a.U[0][idx], a.U[1][idx], a.U[2][idx], a.U[3][idx],
                                                     a.U[4][idx], k, quiet);
-                const float r = ((z.c + fabsf(z.u)) * (float)idx0 + (z.c + fabsf(z.t1)) * (float)idx1) +
-                                (z.c + fabsf(z.t2)) * (float)idx2;
+                const float r = ((z.c + fabsf(z.u)) * idx0 + (z.c + fabsf(z.t1)) * idx1) +
+                                (z.c + fabsf(z.t2)) * idx2;
                 best = (double)r > best ? (double)r : best;
             }
         }

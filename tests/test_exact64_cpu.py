@@ -1,0 +1,108 @@
+"""The integer-pipe division, square root and comparisons of exact64.cuh against
+the host's IEEE operations, bit for bit: operands at the edges of the
+significand (all zeros, all ones, one bit from either), exponents over the whole
+range and around the scaled results, squares and their neighbours, zeros,
+subnormals, infinities and NaN, with the FP32 seeds pushed to both ends of the
+hardware's error bound."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <limits>
+#include <random>
+#include "exact64.cuh"
+using namespace enzo::x64;
+static long bad = 0;
+static void same(const char *op, double a, double b, double ref, double got)
+{
+    if (bits(ref) == bits(got) || (ref != ref && got != got)) return;
+    if (bad++ < 5) printf("%s %a %a: %a, not %a\n", op, a, b, got, ref);
+}
+static void truth(const char *op, double a, double b, bool ref, bool got)
+{
+    if (ref != got && bad++ < 5) printf("%s %a %a\n", op, a, b);
+}
+int main(int argc, char **argv)
+{
+    seed_noise() = (float)atof(argv[1]);
+    std::mt19937_64 g(7);
+    const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+    const double special[] = {0.0, -0.0, 1.0, -1.0, 4.9e-324, 2.2250738585072014e-308, 1.7976931348623157e308, inf,
+                              -inf, nan, -nan, 1e-30, 6.0, 3.0};
+    auto draw = [&](bool wide) {
+        if (wide && g() % 32 == 0) return special[g() % 14];
+        uint64_t m = g() & 0xfffffffffffffull;
+        switch (g() % 8) {
+        case 0: m = 0; break;
+        case 1: m = 0xfffffffffffffull; break;
+        case 2: m &= ~0ull << (g() % 52); break;
+        case 3: m |= (1ull << (g() % 52)) - 1; break;
+        case 4: m = g() & 0xff; break;
+        case 5: m = 0xfffffffffffffull - (g() & 0xff); break;
+        default: break;
+        }
+        const uint64_t e = wide ? g() % 2048 : 1020 + g() % 7;
+        return from_bits((g() & (1ull << 63)) | (e << 52) | m);
+    };
+    for (long i = 0; i < 1500000; ++i) {
+        const bool wide = i % 3 == 0;
+        volatile double va = draw(wide), vb = draw(wide);
+        const double a = va, b = vb;
+        same("div", a, b, va / vb, div(a, b));
+        const Recip r = recip(b);
+        const double ha = 0.5 * a, da = a + a;
+        if (bits(ha + ha) == bits(a) || a != a) same("half div", a, b, ha / vb, div<-1>(a, b, r));
+        if (std::isfinite(da) || !std::isfinite(a)) same("double div", a, b, da / vb, div<1>(a, b, r));
+        same("div6", a, 6.0, va / 6.0, div6(a));
+        volatile double x = std::fabs(a);
+        same("sqrt", x, 0.0, std::sqrt(x), sqrt_rn(x));
+        volatile double y = from_bits(bits(a) & 0xfffffffff8000000ull);
+        const double sq = y * y;
+        for (int d = -1; d <= 1; ++d) {
+            volatile double z = from_bits(bits(sq) + d);
+            same("sqrt", z, 0.0, std::sqrt(z), sqrt_rn(z));
+        }
+        const double f = b > 0.0 && b < inf ? b : 1e-30;
+        truth(">=", a, f, a >= f, ge_pos(a, f));
+        truth(">", a, f, a > f, gt_pos(a, f));
+        truth("> self", f, f, false, gt_pos(f, f));
+        truth("<", a, f, a < f, lt_pos(a, f));
+        truth("> 0", a, 0, a > 0.0, gt0(a));
+        truth(">= 0", a, 0, a >= 0.0, ge0(a));
+        truth("< 0", a, 0, a < 0.0, lt0(a));
+        truth("<= 0", a, 0, a <= 0.0, le0(a));
+        truth("nan", a, 0, a != a, is_nan(a));
+    }
+    for (double a : special)
+        for (double b : special) {
+            volatile double va = a, vb = b;
+            same("div", a, b, va / vb, div(a, b));
+            same("sqrt", a, 0.0, std::sqrt(va), sqrt_rn(a));
+            same("div6", a, 6.0, va / 6.0, div6(a));
+        }
+    printf("%ld differ\n", bad);
+    return bad != 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def program(tmp_path_factory):
+    d = tmp_path_factory.mktemp("exact64")
+    (d / "t.cpp").write_text(SRC)
+    exe = str(d / "t")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-I",
+                    os.path.join(ROOT, "paper_1307_2265_gb300", "csrc"), str(d / "t.cpp"), "-o", exe], check=True)
+    return exe
+
+
+# rcp.approx.ftz.f32 is within 2^-23, rsqrt.approx.ftz.f32 within 2^-22.9
+@pytest.mark.parametrize("noise", [0.0, 1.3e-7, -1.3e-7])
+def test_exact64_matches_ieee(program, noise):
+    r = subprocess.run([program, repr(noise)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
