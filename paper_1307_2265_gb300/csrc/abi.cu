@@ -14,7 +14,7 @@ void note_launch(unsigned n) { g_launches += n; }
 
 
 __device__ __forceinline__ int tiles_of(const enzo_patch &P, int64_t field_len, int kind, int dir,
-                                        int cover, int tile_pencils, bool &bad)
+                                        int cover, int tile_pencils, int zones, bool &bad)
 {
     if (!patch_ok(P, field_len)) {
         bad = true;
@@ -25,6 +25,10 @@ __device__ __forceinline__ int tiles_of(const enzo_patch &P, int64_t field_len, 
         sweep_ranges(P, dir, cover, lo, hi);
         const int a1 = dir == 0 ? 1 : 0, a2 = dir == 2 ? 1 : 2;
         const int64_t pen = (int64_t)(hi[a1] - lo[a1]) * (hi[a2] - lo[a2]);
+        if (zones) {
+            int window;
+            staged_shape(P.n[dir] + 2 * P.ng, zones, tile_pencils, window);
+        }
         return (int)((pen + tile_pencils - 1) / tile_pencils);
     }
     if (kind == kKindFill) {
@@ -49,7 +53,7 @@ __device__ __forceinline__ int tiles_of(const enzo_patch &P, int64_t field_len, 
 // and of the CFL accumulator.
 __global__ void __launch_bounds__(1024) prefix_kernel(const enzo_patch *patches, int npatch,
                                                       int64_t field_len, int kind, int dir, int cover,
-                                                      int tile_pencils, int *prefix, unsigned *counter,
+                                                      int tile_pencils, int zones, int *prefix, unsigned *counter,
                                                       unsigned long long *rate_bits,
                                                       unsigned long long *status)
 {
@@ -62,7 +66,7 @@ __global__ void __launch_bounds__(1024) prefix_kernel(const enzo_patch *patches,
     unsigned nbad = 0;
     for (int i = beg; i < end; ++i) {
         bool b = false;
-        sum += tiles_of(patches[i], field_len, kind, dir, cover, tile_pencils, b);
+        sum += tiles_of(patches[i], field_len, kind, dir, cover, tile_pencils, zones, b);
         nbad += b;
     }
     s_sum[t] = sum;
@@ -76,7 +80,7 @@ __global__ void __launch_bounds__(1024) prefix_kernel(const enzo_patch *patches,
     int run = s_sum[t] - sum;
     for (int i = beg; i < end; ++i) {
         prefix[i] = run;
-        run += tiles_of(patches[i], field_len, kind, dir, cover, tile_pencils, bad);
+        run += tiles_of(patches[i], field_len, kind, dir, cover, tile_pencils, zones, bad);
     }
     if (t == T - 1) {
         prefix[npatch] = s_sum[T - 1];
@@ -242,16 +246,16 @@ static char *ws(const enzo_patch_batch *b) { return static_cast<char *>(b->works
 
 void launch_tile_prefix(const enzo_patch *patches, int npatch, int64_t field_len, int kind, int dir,
                         int cover, int *prefix, unsigned *counter, unsigned long long *rate_bits,
-                        unsigned long long *status, cudaStream_t s, int tile_pencils)
+                        unsigned long long *status, cudaStream_t s, int tile_pencils, int zones)
 {
-    prefix_kernel<<<1, 1024, 0, s>>>(patches, npatch, field_len, kind, dir, cover, tile_pencils, prefix,
+    prefix_kernel<<<1, 1024, 0, s>>>(patches, npatch, field_len, kind, dir, cover, tile_pencils, zones, prefix,
                                      counter, rate_bits, status);
 }
 
 static int launch_prefix(const enzo_patch_batch *b, int kind, int dir, int cover, bool reset_rate,
                          cudaStream_t s, int tile_pencils = kSweepThreads)
 {
-    prefix_kernel<<<1, 1024, 0, s>>>(b->patches, b->npatch, b->field_len, kind, dir, cover, tile_pencils,
+    prefix_kernel<<<1, 1024, 0, s>>>(b->patches, b->npatch, b->field_len, kind, dir, cover, tile_pencils, 0,
                                      reinterpret_cast<int *>(ws(b) + kWsPrefix),
                                      reinterpret_cast<unsigned *>(ws(b) + kWsCounter),
                                      reset_rate ? reinterpret_cast<unsigned long long *>(ws(b) + kWsRateBits)
@@ -269,6 +273,19 @@ static int device_sms()
     return sms > 0 ? sms : 1;
 }
 
+// FP32 batches too small for the marching sweep, which takes about 3 us per
+// position of its longest pencil however few pencils there are; the staged
+// sweep's time goes with the zones, 0.065 to 0.08 ns each, against 0.05 ns of a
+// march with every SM full.  The lines cross near 45000 pencils (the patches,
+// as far as the host knows them, taken as cubes): a 160^3 step took 1350 us
+// staged and 1610 marching, 40 patches of 8..64 580 and 670, 80 patches 1100
+// and 920.
+static bool few_pencils(const enzo_patch_batch *b)
+{
+    const double F = (double)b->field_len;
+    return F <= 45000.0 * std::cbrt(F / b->npatch);
+}
+
 int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double dt, const double *dt_dev,
                        int cover, const MethodParams &m, int precision, int tile_pencils, float *log,
                        unsigned long long *log_count, long long log_cap, int log_stride)
@@ -281,13 +298,18 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     int tile = tile_pencils > 0 ? tile_pencils : kSweepThreads;
     if (precision == ENZO_FP64 || m.guess == ENZO_GUESS_MLP || b->freg || m.options || m.fallback == 2)
         tile = kSweepThreads;
+    const int zones = m.options || m.fallback == 2 || m.guess == ENZO_GUESS_MLP ? 0
+                      : precision == ENZO_FP64                                  ? kStagedZones64
+                      : tile_pencils == 0 && few_pencils(b)                     ? kStagedZones32
+                                                                                : 0;
     launch_tile_prefix(b->patches, b->npatch, b->field_len, kKindSweep, dir, cover,
                        reinterpret_cast<int *>(scratch + kWsPrefix), reinterpret_cast<unsigned *>(scratch + kWsCounter),
-                       nullptr, b->status, s, tile);
+                       nullptr, b->status, s, tile, zones);
     note_launch();
     if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
     SweepArgs a;
     a.tile = tile;
+    a.zones = zones;
     a.patches = b->patches;
     a.npatch = b->npatch;
     a.dir = dir;

@@ -2,11 +2,13 @@
 // (fast reciprocal and square root), conserved variables accumulated in FP64
 // and E - KE recovered in FP64 in high-Mach cells.
 #include "ppm_device.cuh"
+#include "ppm_staged.cuh"
 
 namespace enzo {
 
 cudaError_t launch_sweep_fp32(const SweepArgs &a, int grid, cudaStream_t s)
 {
+    if (a.zones) return launch_staged<float, kStagedZones32, 3>(a, s);
     return launch_sweep_dir<float>(a, grid, s);
 }
 

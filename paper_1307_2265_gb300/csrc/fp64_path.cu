@@ -2,11 +2,13 @@
 // solver in double precision.  Built with --fmad=false and IEEE division and
 // square root so each operation rounds exactly once, in the written order.
 #include "ppm_device.cuh"
+#include "ppm_staged.cuh"
 
 namespace enzo {
 
 cudaError_t launch_sweep_fp64(const SweepArgs &a, int grid, cudaStream_t s)
 {
+    if (a.zones) return launch_staged<double, kStagedZones64, 2>(a, s);
     return launch_sweep_dir<double>(a, grid, s);
 }
 

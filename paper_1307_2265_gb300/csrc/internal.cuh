@@ -56,6 +56,7 @@ struct SweepArgs {
     const double *dt_ptr;      // device dt (enzo_step)
     MethodParams mp;
     int tile = kSweepThreads;  // pencils per CTA tile (= threads per CTA)
+    int zones = 0;             // staged sweep: zones per CTA tile (0: marching sweep)
     const int *prefix;         // [npatch + 1]
     unsigned *tile_counter;
     unsigned long long *status;
@@ -91,6 +92,38 @@ __host__ __device__ inline bool patch_ok(const enzo_patch &P, int64_t field_len)
     }
     const int64_t vol = (int64_t)(P.n[0] + 6) * (P.n[1] + 6) * (P.n[2] + 6);
     return P.off >= 0 && P.off + vol <= field_len;
+}
+
+// Staged sweep (ppm_staged.cuh): zones, and threads, per CTA tile.  FP64: 256
+// zones, two CTAs per SM (128 registers): a 400-patch level step took 84 ms
+// against 89 (192 zones), 99 (128 zones, four CTAs) and 85 (512 zones, one).
+// FP32: 256 zones, three CTAs per SM (80 registers): a 32^3 step took 102 us
+// against 108 (four CTAs, 64 registers), 104 and 115 (512 zones, one and two).
+constexpr int kStagedZones64 = 256, kStagedZones32 = 256;
+constexpr int kStagedMaxPencils = 8;   // windowed pencils per tile
+
+// Pencils per tile and positions per window for pencils of L positions in
+// tiles of `zones` zones: k windows of W positions (eight of each shared with
+// the one before), the k that leaves the fewest lanes idle, a window counted
+// 6% dearer than its lanes for what it repeats.  (A 128^3 FP32 step in whole
+// pencils of 134 positions, one per tile, took 816 us.)
+__host__ __device__ inline void staged_shape(int L, int zones, int &pencils, int &window)
+{
+    float best = 1e30f;
+    for (int k = 1; k <= 4096; ++k) {
+        const int W = (L + 8 * (k - 1) + k - 1) / k;
+        if (k > 1 && W < 32) break;
+        if (W > zones) continue;
+        int P = zones / W;
+        if (k > 1 && P > kStagedMaxPencils) P = kStagedMaxPencils;
+        const float cost = (float)k * (1.0f + 0.06f * (float)(k - 1) / (float)k) / (float)P;
+        if (cost < best * 0.999f) {
+            best = cost;
+            pencils = P;
+            window = W;
+        }
+        if (k > 8 && best < 1e30f) break;
+    }
 }
 
 // Launch helpers implemented in the precision translation units.
@@ -147,7 +180,8 @@ constexpr int kFlagTile = 8;            // flag kernel: 8^3 active cells per CTA
 // Launch of the per-patch tile prefix kernel (kind: kKind*) on stream s.
 void launch_tile_prefix(const enzo_patch *patches, int npatch, int64_t field_len, int kind, int dir,
                         int cover, int *prefix, unsigned *counter, unsigned long long *rate_bits,
-                        unsigned long long *status, cudaStream_t s, int tile_pencils = kSweepThreads);
+                        unsigned long long *status, cudaStream_t s, int tile_pencils = kSweepThreads,
+                        int zones = 0);
 
 #ifdef __CUDACC__
 // float <-> double conversions on the integer pipe.  On GB300 the FP64 pipe

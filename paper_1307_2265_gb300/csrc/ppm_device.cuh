@@ -55,6 +55,28 @@
 
 namespace enzo {
 
+// FP32 expressions whose rounding the compiler may choose (which product of a
+// sum it fuses) can differ from kernel to kernel.  The functions below that
+// take PIN state the choice when it is true: the one the marching kernels are
+// compiled to, found by comparing results, so that the staged kernels give
+// the march's values bit for bit.
+//
+// a b + c d: OPT 0 rounds c d, 1 rounds a b, 2 rounds both products.
+template <int OPT>
+__device__ __forceinline__ float mad2(float a, float b, float c, float d)
+{
+    if (OPT == 0) return __fmaf_rn(a, b, __fmul_rn(c, d));
+    if (OPT == 1) return __fmaf_rn(c, d, __fmul_rn(a, b));
+    return __fadd_rn(__fmul_rn(a, b), __fmul_rn(c, d));
+}
+
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 template <class R>
 struct Consts {
     R gamma, gm1, gm1inv, gp1o2g, rho_floor, p_floor, tol, step_tol, eta_eke;
@@ -140,7 +162,7 @@ __device__ __forceinline__ Zone<double> prim<double, false>(double rho, double m
     return prim<double, true>(rho, mn, m1, m2, E, k, quiet);
 }
 
-template <bool COUNT>
+template <bool COUNT, bool PIN = false>
 __device__ __forceinline__ Zone<float> prim_f(double rho64, double mn64, double m164,
                                               double m264, double E64, const Consts<float> &k,
                                               Counters &cnt)
@@ -150,8 +172,13 @@ __device__ __forceinline__ Zone<float> prim_f(double rho64, double mn64, double 
     if (!(rho >= k.rho_floor)) { rho = k.rho_floor; rho64 = f2d_exact(rho); if (COUNT) cnt.rare(ENZO_ST_RHO_FLOOR); }
     const float inv = 1.0f / rho;
     const float mn = d2f_rz(mn64), m1 = d2f_rz(m164), m2 = d2f_rz(m264), E = d2f_rz(E64);
-    const float ke = 0.5f * ((mn * mn + m1 * m1) + m2 * m2) * inv;
-    float e = E - ke;
+    float e;
+    if constexpr (PIN) {
+        e = __fmaf_rn(-__fmul_rn(0.5f, __fmaf_rn(m2, m2, mad2<0>(mn, mn, m1, m1))), inv, E);
+    } else {
+        const float ke = 0.5f * ((mn * mn + m1 * m1) + m2 * m2) * inv;
+        e = E - ke;
+    }
     if (e < k.eta_eke * E) {
         // high-Mach cell: the internal energy is a small difference of two
         // large numbers, so it is recovered in FP64
@@ -306,30 +333,33 @@ __device__ __forceinline__ double limited_slope<double>(double qm, double q0, do
 }
 
 // Value at the interface between zones a and b with limited slopes da, db.
-template <class R>
+// (FP64: the half is exact, so one fused operation rounds as the two do.)
+template <class R, bool PIN = false>
 __device__ __forceinline__ R face_value(R a, R b, R da, R db)
 {
-    return (R)0.5 * (a + b) - div6(db - da);
-}
-// FP64: the half is exact, so one fused operation rounds as the two do.
-template <>
-__device__ __forceinline__ double face_value<double>(double a, double b, double da, double db)
-{
-    return __fma_rn(0.5, a + b, -div6(db - da));
+    if constexpr (sizeof(R) == 8) return __fma_rn(0.5, a + b, -div6(db - da));
+    else if constexpr (PIN) return __fmaf_rn(0.5f, a + b, -__fmul_rn(db - da, 1.0f / 6.0f));
+    else return (R)0.5 * (a + b) - div6(db - da);
 }
 
 // Monotone parabola of a zone (CW84 1.10): edges ql, qr in, (qL, Delta q, q6) out.
-template <class R>
+__device__ __forceinline__ void parabola64(double qs, double ql, double qr, double &oL, double &oR, double &d, double &q6);
+
+template <class R, bool PIN = false>
 __device__ __forceinline__ void parabola(R qs, R ql, R qr, R &oL, R &oR, R &d, R &q6)
 {
+    if constexpr (sizeof(R) == 8) {
+        parabola64(qs, ql, qr, oL, oR, d, q6);
+        return;
+    }
     if ((qr - qs) * (qs - ql) <= (R)0) {
         ql = qs;
         qr = qs;
     } else {
         const R dd = qr - ql;
         const R qq6 = (R)6 * (qs - (R)0.5 * (ql + qr));
-        if (dd * qq6 > dd * dd) ql = (R)3 * qs - (R)2 * qr;
-        else if (-(dd * dd) > dd * qq6) qr = (R)3 * qs - (R)2 * ql;
+        if (dd * qq6 > dd * dd) ql = PIN ? (R)__fmaf_rn(3.0f, qs, -2.0f * qr) : (R)3 * qs - (R)2 * qr;
+        else if (-(dd * dd) > dd * qq6) qr = PIN ? (R)__fmaf_rn(3.0f, qs, -2.0f * ql) : (R)3 * qs - (R)2 * ql;
     }
     oL = ql;
     oR = qr;
@@ -340,9 +370,8 @@ __device__ __forceinline__ void parabola(R qs, R ql, R qr, R &oL, R &oR, R &d, R
 // FP64: the same values.  The sign of the first product is its factors', and
 // the overshoot tests compare |q6| with |Delta q|: the products order as they
 // do unless they are within 16 ulp, where the products themselves decide.
-template <>
-__device__ __forceinline__ void parabola<double>(double qs, double ql, double qr, double &oL, double &oR, double &d,
-                                                 double &q6)
+__device__ __forceinline__ void parabola64(double qs, double ql, double qr, double &oL, double &oR, double &d,
+                                           double &q6)
 {
     const double er = qr - qs, el = qs - ql;
     bool flat;
@@ -548,7 +577,7 @@ __device__ __forceinline__ void trace_exact(const double qL[5], const double qR[
 //   * p = p_ref + C^2 beta_s, u = u_ref - sg C beta_s,
 //     1/rho = 1/rho_ref - (beta_s + beta_0), with 1/C from one reciprocal
 //     square root of C^2 = gamma p_ref rho_ref.
-template <int SIDE>
+template <int SIDE, bool PIN = false>
 __device__ __forceinline__ void trace_f(const float qL[5], const float qR[5], const float d[5],
                                         const float q6[5], float u, float c, float dtdx,
                                         const Consts<float> &k, float out[5])
@@ -576,7 +605,7 @@ __device__ __forceinline__ void trace_f(const float qL[5], const float qR[5], co
     float bsl = 0.0f, b0 = 0.0f;
     if (ss > 0.0f) {
         const float du = u_ref - ENZO_AVG(as, bs, 1), dp = p_ref - ENZO_AVG(as, bs, 2);
-        bsl = (sg * 0.5f * iC) * fmaf(-sg * dp, iC, du);
+        bsl = PIN ? __fmul_rn(sg * 0.5f * iC, fmaf(-sg * dp, iC, du)) : (sg * 0.5f * iC) * fmaf(-sg * dp, iC, du);
     }
     if (s0 > 0.0f) {
         const float dp = p_ref - ENZO_AVG(a0, b0c, 2);
@@ -584,7 +613,7 @@ __device__ __forceinline__ void trace_f(const float qL[5], const float qR[5], co
     }
     float p = fmaf(C2, bsl, p_ref);
     const float un = fmaf(-sg * C, bsl, u_ref);
-    float rho = 1.0f / (irho - (bsl + b0));
+    float rho = 1.0f / (irho - (PIN ? __fadd_rn(bsl, b0) : bsl + b0));
     out[0] = rho > k.rho_floor ? rho : k.rho_floor;
     out[1] = un;
     out[2] = p > k.p_floor ? p : k.p_floor;
@@ -594,13 +623,13 @@ __device__ __forceinline__ void trace_f(const float qL[5], const float qR[5], co
 }
 
 // Right state of the zone's left edge (sR) and left state of its right edge (sL).
-template <class R>
+template <class R, bool PIN = false>
 __device__ __forceinline__ void trace(const R qL[5], const R qR[5], const R d[5], const R q6[5], R u, R c, R dtdx,
                                       const Consts<R> &k, R sR[5], R sL[5])
 {
     if constexpr (std::is_same<R, float>::value) {
-        trace_f<-1>(qL, qR, d, q6, u, c, dtdx, k, sR);
-        trace_f<+1>(qL, qR, d, q6, u, c, dtdx, k, sL);
+        trace_f<-1, PIN>(qL, qR, d, q6, u, c, dtdx, k, sR);
+        trace_f<+1, PIN>(qL, qR, d, q6, u, c, dtdx, k, sL);
     } else {
         trace_exact(qL, qR, d, q6, u, c, dtdx, k, sR, sL);
     }
@@ -639,6 +668,7 @@ struct RiemannOut {
 // step of the root).  A learned start that reaches the iteration cap restarts
 // once from the plain guess inside the same loop.  The upwind side alone is
 // sampled.
+template <bool PIN = false>
 __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float pl, float rr, float ur, float pr,
                                                       float pguess, const Consts<float> &k, Counters &cnt)
 {
@@ -650,7 +680,8 @@ __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float
         const float CL = C2L * iCL, CR = C2R * iCR;
         // |u*_R - u*_L| <= tol (|u_L| + |u_R| + c_L + c_R), c = C / rho
         ftol = k.tol * ((fabsf(ul) + fabsf(ur)) + (CL / rl + CR / rr));
-        plain = (CR * pl + CL * pr + CL * CR * (ul - ur)) / (CL + CR);
+        if constexpr (PIN) plain = __fmaf_rn(__fmul_rn(CL, CR), ul - ur, mad2<0>(CR, pl, CL, pr)) / __fadd_rn(CL, CR);
+        else plain = (CR * pl + CL * pr + CL * CR * (ul - ur)) / (CL + CR);
         plain = plain > k.p_floor ? plain : k.p_floor;
     }
     float ps = pguess > 0.0f ? (pguess > k.p_floor ? pguess : k.p_floor) : plain;
@@ -670,10 +701,14 @@ __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float
         const float iWL = rsL * iCL, iWR = rsR * iCR;
         usL = fmaf(pl - ps, iWL, ul);
         usR = fmaf(ps - pr, iWR, ur);
-        izL = iWL * fmaf(0.5f * rsL, rsL, 0.5f);
-        izR = iWR * fmaf(0.5f * rsR, rsR, 0.5f);
+        const float xL = fmaf(0.5f * rsL, rsL, 0.5f), xR = fmaf(0.5f * rsR, rsR, 0.5f);
+        izL = PIN ? __fmul_rn(iWL, xL) : iWL * xL;
+        izR = PIN ? __fmul_rn(iWR, xR) : iWR * xR;
         const float f = usR - usL;
-        float pn = ps - f / (izL + izR);
+        float pn;
+        if constexpr (PIN)
+            pn = __fmaf_rn(-f, rcp_approx(h < ENZO_NEWTON_HEAD - 1 ? __fmaf_rn(iWL, xL, izR) : __fadd_rn(izL, izR)), ps);
+        else pn = ps - f / (izL + izR);
         pn = pn > k.p_floor ? pn : k.p_floor;
         const bool fconv = fabsf(f) <= ftol;
         const bool sconv = fabsf(pn - ps) <= k.step_tol * pn;
@@ -704,11 +739,14 @@ __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float
         const float iWL = rsL * iCL, iWR = rsR * iCR;
         usL = fmaf(pl - ps, iWL, ul);
         usR = fmaf(ps - pr, iWR, ur);
-        izL = iWL * fmaf(0.5f * rsL, rsL, 0.5f);
-        izR = iWR * fmaf(0.5f * rsR, rsR, 0.5f);
+        const float xL = fmaf(0.5f * rsL, rsL, 0.5f), xR = fmaf(0.5f * rsR, rsR, 0.5f);
+        izL = PIN ? __fmul_rn(iWL, xL) : iWL * xL;
+        izR = PIN ? __fmul_rn(iWR, xR) : iWR * xR;
         const float f = usR - usL;
         if (fabsf(f) <= ftol) { conv = true; break; }
-        float pn = ps - f / (izL + izR);
+        float pn;
+        if constexpr (PIN) pn = __fmaf_rn(-f, rcp_approx(__fadd_rn(izL, izR)), ps);
+        else pn = ps - f / (izL + izR);
         pn = pn > k.p_floor ? pn : k.p_floor;
         ++it;
         if (fabsf(pn - ps) <= k.step_tol * pn) { conv = true; break; }
@@ -717,7 +755,9 @@ __device__ __forceinline__ RiemannOut<float> riemann_f(float rl, float ul, float
     RiemannOut<float> o;
     o.iters = it;
     o.conv = conv;
-    const float us = (usL * izR + usR * izL) / (izL + izR);
+    float us;
+    if constexpr (PIN) us = mad2<1>(usL, izR, usR, izL) / __fadd_rn(izL, izR);
+    else us = (usL * izR + usR * izL) / (izL + izR);
     o.ustar = us;
     o.pstar = ps;
     // sample x/t = 0 on the side upwind of the contact: sg = +1 left, -1 right;
@@ -869,17 +909,18 @@ __device__ __forceinline__ RiemannOut<double> riemann_exact(double rl, double ul
     return o;
 }
 
-template <class R>
+template <class R, bool PIN = false>
 __device__ __forceinline__ RiemannOut<R> riemann(R rl, R ul, R pl, R rr, R ur, R pr, R pguess,
                                                  const Consts<R> &k, Counters &cnt)
 {
-    if constexpr (std::is_same<R, float>::value) return riemann_f(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
+    if constexpr (std::is_same<R, float>::value) return riemann_f<PIN>(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
     else return riemann_exact(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
 }
 
 // Physical flux of the split 1-D equations (Sec. 4.1): mass, normal momentum,
 // transverse momenta, total energy.
-template <class R>
+// (FP64: the half is exact, so one fused operation adds the kinetic energy.)
+template <class R, bool PIN = false>
 __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Consts<R> &k, R F[5])
 {
     const R mflux = rho * u;
@@ -887,22 +928,16 @@ __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Con
     F[1] = mflux * u + p;
     F[2] = mflux * t1;
     F[3] = mflux * t2;
-    const R eint = p * k.gm1inv;
-    const R ke = (R)0.5 * rho * ((u * u + t1 * t1) + t2 * t2);
-    F[4] = u * ((eint + ke) + p);
-}
-
-// FP64: the half is exact, so one fused operation adds the kinetic energy.
-template <>
-__device__ __forceinline__ void phys_flux<double>(double rho, double u, double p, double t1, double t2,
-                                                  const Consts<double> &k, double F[5])
-{
-    const double mflux = rho * u;
-    F[0] = mflux;
-    F[1] = mflux * u + p;
-    F[2] = mflux * t1;
-    F[3] = mflux * t2;
-    F[4] = u * (__fma_rn(0.5, rho * ((u * u + t1 * t1) + t2 * t2), p * k.gm1inv) + p);
+    if constexpr (sizeof(R) == 8) {
+        F[4] = u * (__fma_rn(0.5, rho * ((u * u + t1 * t1) + t2 * t2), p * k.gm1inv) + p);
+    } else if constexpr (PIN) {
+        const float X = __fmaf_rn(t2, t2, mad2<0>(u, u, t1, t1));
+        F[4] = __fmul_rn(u, __fadd_rn(__fmaf_rn(p, k.gm1inv, __fmul_rn(__fmul_rn(0.5f, rho), X)), p));
+    } else {
+        const R eint = p * k.gm1inv;
+        const R ke = (R)0.5 * rho * ((u * u + t1 * t1) + t2 * t2);
+        F[4] = u * ((eint + ke) + p);
+    }
 }
 
 // HLL flux with Davis wave-speed bounds from first-order zone states (fallback).
@@ -2225,7 +2260,7 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (sizeof
         pc.L = P.n[DIR] + 2 * P.ng;
         pc.ng = P.ng;
         pc.n = P.n[DIR];
-        const double dtdx64 = dt / P.dx[DIR];
+        const double dtdx64 = x64::div(dt, P.dx[DIR]);   // off the FP64 pipe
         const R dtdx = (R)dtdx64;
         if (valid) interfaces += (unsigned long long)(P.n[DIR] + 1);
         const unsigned key = (unsigned)lo * 7919u + (unsigned)pe;
@@ -2396,10 +2431,15 @@ int sweep_grid_for(int device)
     if (cached[device]) return cached[device];
     int sms = 0, per = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    ring_prepare<R, 0, kSweepThreads, false>(device);
-    ring_prepare<R, 1, kSweepThreads, false>(device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false>, kSweepThreads,
-                                                  ring_bytes<R, kSweepThreads, 0, 1>());
+    if constexpr (sizeof(R) == 8) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, kSweepThreads, false, 1>,
+                                                      kSweepThreads, 0);
+    } else {
+        ring_prepare<R, 0, kSweepThreads, false>(device);
+        ring_prepare<R, 1, kSweepThreads, false>(device);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false>, kSweepThreads,
+                                                      ring_bytes<R, kSweepThreads, 0, 1>());
+    }
     if (sms < 1) sms = 1;
     if (per < 1) per = 1;
     cached[device] = sms * per;
@@ -2506,36 +2546,40 @@ cudaError_t launch_sweep_dir(const SweepArgs &a, int grid, cudaStream_t s)
         }
         return cudaGetLastError();
     }
-    constexpr int sx = ring_bytes<R, kSweepThreads, 0, 0>(), syz = ring_bytes<R, kSweepThreads, 0, 1>();
-    {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaError_t e = cudaSuccess;
-        if (a.freg) {
-            if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, true>(dev);
-            if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, true>(dev);
-            if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, true>(dev);
-        } else {
-            if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, false>(dev);
-            if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, false>(dev);
-            if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, false>(dev);
+    if constexpr (sizeof(R) == 8) {
+        return cudaErrorInvalidValue;   // the default FP64 sweep is the staged one
+    } else {
+        constexpr int sx = ring_bytes<R, kSweepThreads, 0, 0>(), syz = ring_bytes<R, kSweepThreads, 0, 1>();
+        {
+            int dev = 0;
+            cudaGetDevice(&dev);
+            cudaError_t e = cudaSuccess;
+            if (a.freg) {
+                if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, true>(dev);
+                if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, true>(dev);
+                if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, true>(dev);
+            } else {
+                if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, false>(dev);
+                if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, false>(dev);
+                if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, false>(dev);
+            }
+            if (e != cudaSuccess) return e;
         }
-        if (e != cudaSuccess) return e;
-    }
-    if (a.freg) {
+        if (a.freg) {
+            switch (a.dir) {
+            case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, true><<<grid, kSweepThreads, sx, s>>>(a); break;
+            case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
+            default: ppm_sweep_kernel<R, 2, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
+            }
+            return cudaGetLastError();
+        }
         switch (a.dir) {
-        case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, true><<<grid, kSweepThreads, sx, s>>>(a); break;
-        case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
-        default: ppm_sweep_kernel<R, 2, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
+        case 0: ppm_sweep_kernel<R, 0, false><<<grid, kSweepThreads, sx, s>>>(a); break;
+        case 1: ppm_sweep_kernel<R, 1, false><<<grid, kSweepThreads, syz, s>>>(a); break;
+        default: ppm_sweep_kernel<R, 2, false><<<grid, kSweepThreads, syz, s>>>(a); break;
         }
         return cudaGetLastError();
     }
-    switch (a.dir) {
-    case 0: ppm_sweep_kernel<R, 0, false><<<grid, kSweepThreads, sx, s>>>(a); break;
-    case 1: ppm_sweep_kernel<R, 1, false><<<grid, kSweepThreads, syz, s>>>(a); break;
-    default: ppm_sweep_kernel<R, 2, false><<<grid, kSweepThreads, syz, s>>>(a); break;
-    }
-    return cudaGetLastError();
 }
 
 }  // namespace enzo

@@ -1,0 +1,452 @@
+// The split PPM sweep by stages: one thread per zone, then per face, then per
+// cell, of a tile of whole pencils held in shared memory.
+//
+// The marching kernel (ppm_device.cuh) keeps one pencil per thread: its
+// parallelism is the number of pencils, its time the length of one, and its
+// loop body is longer than the instruction cache, which every warp walks on its
+// own.  Here a tile of at most THREADS zones goes through the steps of the
+// method together: primitives; slopes; interface values; parabolas and traced
+// states; Riemann problems; update.  Each step reads its neighbours from shared
+// memory, and its zones, faces or cells are dealt out to consecutive threads,
+// so no lane of a warp idles in a ghost zone where ghosts have no part.  Every
+// value is formed by the same functions as in the march, so results agree bit
+// for bit (FP64).
+//
+// A pencil longer than the tile goes in windows of W positions.  A window
+// updates cells [lo, hi), reads the four positions on either side (the
+// fallback test of the neighbouring cell needs its two faces), and hands the
+// last eight positions, as they were before any update, to the next window
+// through shared memory.
+#pragma once
+#include "ppm_device.cuh"
+
+namespace enzo {
+
+template <class R, int THREADS>
+struct StagedSmem {
+    double U[5][THREADS];      // raw conserved values (rho, m_n, m_t1, m_t2, E)
+    R q[6][THREADS];           // zone primitives r, u, p, t1, t2, c
+    R A[5][THREADS];           // slopes, then right states of the zones' left edges
+    R B[5][THREADS];           // interface values at s+1/2, then fluxes
+    R C[5][THREADS];           // left states of the zones' right edges
+    R save[6][3][kStagedMaxPencils];   // windowed wrapped pencils: the first three active zones
+    unsigned char bad[THREADS];
+};
+
+template <class R, int DIR, int THREADS, bool REG>
+struct Staged {
+    static constexpr int A1 = DIR == 0 ? 1 : 0;
+    static constexpr int A2 = DIR == 2 ? 1 : 2;
+    using Smem = StagedSmem<R, THREADS>;
+    const SweepArgs &a;
+    const enzo_patch &P;
+    Smem &S;
+    const Consts<R> &k;
+    Counters &cnt;
+    R dtdx;
+    double dtdx64, dt64;
+    int np, W, L, n, ng;       // pencils of this tile, window, pencil length, active cells, ghosts
+    int pen0, cnt1, r1, r2;    // first pencil, pencils per row of the cross-section, its origin
+    int64_t st1, st2, sd;
+    bool wrap;
+    int patch;
+
+    // Storage index of position 0 of pencil p of the tile.
+    __device__ __forceinline__ int64_t base(int p) const
+    {
+        const int pe = pen0 + p;
+        const int i2 = pe / cnt1, i1 = pe - i2 * cnt1;
+        return P.off + (int64_t)(r1 + i1) * st1 + (int64_t)(r2 + i2) * st2;
+    }
+    // Deal item t of m per pencil: pencil p and item j; x pencils item-fastest,
+    // y and z pencils pencil-fastest (neighbouring x), so global accesses run
+    // along x.
+    __device__ __forceinline__ void deal(int t, int m, int &p, int &j) const
+    {
+        if (DIR == 0) {
+            p = (int)((unsigned)t / (unsigned)m);
+            j = t - p * m;
+        } else {
+            j = (int)((unsigned)t / (unsigned)np);
+            p = t - j * np;
+        }
+    }
+    // Slot of window position w of pencil p; the slot one position on.
+    __device__ __forceinline__ int slot(int p, int w) const { return DIR == 0 ? p * W + w : w * np + p; }
+    __device__ __forceinline__ int next() const { return DIR == 0 ? 1 : np; }
+
+    __device__ __forceinline__ Zone<R> zone(int z) const
+    {
+        return Zone<R>{S.q[0][z], S.q[1][z], S.q[2][z], S.q[3][z], S.q[4][z], S.q[5][z]};
+    }
+
+    // Final flux of the face right of slot z: the Godunov flux, or HLL from the
+    // zone states beside a cell that failed (Sec. 4.1.2).
+    __device__ __forceinline__ void final_flux(int z, bool hll, R F[5]) const
+    {
+        if (hll) {
+            hll_flux<R>(zone(z), zone(z + next()), k, F);
+        } else {
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = S.B[v][z];
+        }
+    }
+
+    __device__ __forceinline__ void widen(const R F[5], double G[5]) const
+    {
+        _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            G[v] = sizeof(R) == 8 ? (double)F[v] : f2d_exact((float)(dtdx * F[v]));
+    }
+
+    // Flux registers of face f (left of active cell f) of pencil p, as the
+    // march records them.
+    __device__ __forceinline__ void record(int p, int f, const double G[5]) const
+    {
+        if (!REG || !a.freg) return;
+        const int pe = pen0 + p, i2 = pe / cnt1, i1 = pe - i2 * cnt1;
+        const int j1 = r1 + i1 - ng, j2 = r2 + i2 - ng;
+        const int na1 = P.n[A1], na2 = P.n[A2];
+        if (j1 < 0 || j1 >= na1 || j2 < 0 || j2 >= na2) return;
+        int64_t oall = 0, obnd = 0;
+        for (int d = 0; d < DIR; ++d) {
+            const int b1 = d == 0 ? 1 : 0, b2 = d == 2 ? 1 : 2;
+            oall += (int64_t)(P.n[d] + 1) * P.n[b1] * P.n[b2] * 5;
+            obnd += (int64_t)2 * P.n[b1] * P.n[b2] * 5;
+        }
+        const int64_t row = (int64_t)j2 * na1 + j1;
+        if (P.freg_all >= 0) {
+            double *o = a.freg + P.freg_all + oall + (row * (n + 1) + f) * 5;
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = G[v];
+        }
+        if (P.freg_bnd >= 0 && (f == 0 || f == n)) {
+            double *o = a.freg + P.freg_bnd + obnd + (row * 2 + (f == 0 ? 0 : 1)) * 5;
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = o[v] + (sizeof(R) == 8 ? dt64 * G[v] : G[v]);
+        }
+    }
+
+    __device__ __forceinline__ void log_states(int p, int s, const R l[3], const R r[3]) const
+    {
+        // the march's key and step: pencil identity, and the step that solves
+        // the interface right of position s
+        const int kk = s + 3;
+        const unsigned key = (unsigned)patch * 7919u + (unsigned)(pen0 + p);
+        const unsigned h = (key * 2654435761u) ^ ((unsigned)kk * 40503u);
+        if ((h % (unsigned)a.log_stride) != 0u) return;
+        const unsigned long long i = atomicAdd(a.log_count, 1ull);
+        if ((long long)i >= a.log_cap) return;
+        float *o = a.log + 6 * i;
+        _Pragma("unroll") for (int v = 0; v < 3; ++v)
+        {
+            o[v] = (float)l[v];
+            o[3 + v] = (float)r[v];
+        }
+    }
+
+    // One window: positions [w0, w0 + m), cells [lo, hi) updated.  fresh: first
+    // window position not handed over by the window before.
+    __device__ __forceinline__ void window(int w0, int m, int lo, int hi, int fresh)
+    {
+        const int t = threadIdx.x;
+        const bool first = w0 == 0, last = hi == L - ng;
+        const bool windowed = W < L;
+        const int map[5] = {0, 1 + DIR, 1 + A1, 1 + A2, 4};
+        int p, j;
+        // zones: load and primitives
+        deal(t, m - fresh, p, j);
+        if (p < np && j < m - fresh) {
+            const int w = fresh + j, s = w0 + w, z = slot(p, w);
+            const int64_t b = base(p);
+            bool count = true, saved = false;
+            int64_t idx = b + (int64_t)s * sd;
+            if (wrap) {
+                const int c = s - ng;
+                if (c < 0 || c >= n) idx = b + (int64_t)(ng + (c % n + n) % n) * sd;
+                count = c < n;
+                saved = windowed && c >= n;
+            }
+            Zone<R> q;
+            if (saved) {
+                const int i = s - ng - n;
+                q = Zone<R>{S.save[0][i][p], S.save[1][i][p], S.save[2][i][p],
+                            S.save[3][i][p], S.save[4][i][p], S.save[5][i][p]};
+            } else {
+                double u[5];
+                _Pragma("unroll") for (int v = 0; v < 5; ++v) u[v] = a.U[map[v]][idx];
+                Counters c;
+                c.st = count ? cnt.st : nullptr;
+                if constexpr (sizeof(R) == 4) q = prim_f<true, true>(u[0], u[1], u[2], u[3], u[4], k, c);
+                else q = prim<R, true>(u[0], u[1], u[2], u[3], u[4], k, c);
+                _Pragma("unroll") for (int v = 0; v < 5; ++v) S.U[v][z] = u[v];
+                if (windowed && wrap && s >= ng && s < ng + 3) {
+                    const int i = s - ng;
+                    S.save[0][i][p] = q.r;
+                    S.save[1][i][p] = q.u;
+                    S.save[2][i][p] = q.p;
+                    S.save[3][i][p] = q.t1;
+                    S.save[4][i][p] = q.t2;
+                    S.save[5][i][p] = q.c;
+                }
+            }
+            S.q[0][z] = q.r;
+            S.q[1][z] = q.u;
+            S.q[2][z] = q.p;
+            S.q[3][z] = q.t1;
+            S.q[4][z] = q.t2;
+            S.q[5][z] = q.c;
+        }
+        __syncthreads();
+        const int e = next();
+        // slopes of positions 1 .. m-2
+        deal(t, m - 2, p, j);
+        if (p < np && j < m - 2) {
+            const int z = slot(p, 1 + j);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                S.A[v][z] = limited_slope<R>(S.q[v][z - e], S.q[v][z], S.q[v][z + e]);
+        }
+        __syncthreads();
+        // interface values right of positions 1 .. m-3
+        deal(t, m - 3, p, j);
+        if (p < np && j < m - 3) {
+            const int z = slot(p, 1 + j);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                S.B[v][z] = face_value<R, true>(S.q[v][z], S.q[v][z + e], S.A[v][z], S.A[v][z + e]);
+        }
+        __syncthreads();
+        // parabolas and traced states of positions 2 .. m-3
+        deal(t, m - 4, p, j);
+        if (p < np && j < m - 4) {
+            const int z = slot(p, 2 + j);
+            R pL[5], pR[5], pd[5], p6[5], sR[5], sL[5];
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                parabola<R, true>(S.q[v][z], S.B[v][z - e], S.B[v][z], pL[v], pR[v], pd[v], p6[v]);
+            trace<R, true>(pL, pR, pd, p6, S.q[1][z], S.q[5][z], dtdx, k, sR, sL);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            {
+                S.A[v][z] = sR[v];
+                S.C[v][z] = sL[v];
+            }
+        }
+        __syncthreads();
+        // Riemann problems right of positions 2 .. m-4; this window answers for
+        // the faces left of its cells and, at the pencil's end, the last one
+        deal(t, m - 5, p, j);
+        if (p < np && j < m - 5) {
+            const int w = 2 + j, s = w0 + w, z = slot(p, w);
+            const bool own = s >= lo - 1 && (s < hi - 1 || last);
+            R l[5], r[5], F[5];
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            {
+                l[v] = S.C[v][z];
+                r[v] = S.A[v][z + e];
+            }
+            if (a.log && own) log_states(p, s, l, r);
+            if (a.mp.solver == ENZO_SOLVER_TWOSHOCK) {
+                const RiemannOut<R> o = riemann<R, true>(l[0], l[1], l[2], r[0], r[1], r[2], (R)-1, k, cnt);
+                if (own) {
+                    cnt.iters += (unsigned)o.iters;
+                    if (!o.conv) cnt.rare(ENZO_ST_NEWTON_NONCONV);
+                }
+                const bool up = o.ustar >= (R)0;
+                phys_flux<R, true>(o.rho, o.u, o.p, up ? l[3] : r[3], up ? l[4] : r[4], k, F);
+            } else if (a.mp.solver == ENZO_SOLVER_HLLC) {
+                hllc_states<R>(l, r, k, F);
+            } else {
+                hll_states<R>(l, r, k, F);
+            }
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) S.B[v][z] = F[v];
+        }
+        __syncthreads();
+        // does the Godunov update leave rho > 0?  Cells [lo - 1, hi] of the
+        // pencil's active ones (the neighbours' answers decide shared faces)
+        const bool fb = a.mp.fallback != 0;
+        bool any = false;
+        if (fb) {
+            const int c0 = first ? lo : lo - 1, c1 = last ? hi : hi + 1;
+            deal(t, c1 - c0, p, j);
+            if (p < np && j < c1 - c0) {
+                const int s = c0 + j, z = slot(p, s - w0);
+                const R fm = S.B[0][z - e], fp = S.B[0][z];
+                bool bad = false;
+                if (sizeof(R) == 8) {
+                    bad = !x64::gt0(cell_update(S.U[0][z], dtdx64, (double)fm, (double)fp));
+                } else {
+                    // FP32 screen; cells near zero are decided in FP64
+                    const R r0 = S.q[0][z];
+                    if (!(r0 + dtdx * (fm - fp) > (R)1e-3 * r0))
+                        bad = !((S.U[0][z] + f2d_exact((float)(dtdx * fm))) - f2d_exact((float)(dtdx * fp)) > 0.0);
+                }
+                if (bad && s >= lo && s < hi) cnt.rare(ENZO_ST_HLL_CELLS);
+                S.bad[z] = bad;
+                any = bad;
+            }
+            any = __syncthreads_or(any) != 0;
+        }
+        // update of cells [lo, hi)
+        deal(t, hi - lo, p, j);
+        if (p < np && j < hi - lo) {
+            const int s = lo + j, z = slot(p, s - w0);
+            bool hm = false, hp = false;
+            if (any) {
+                const bool b0 = S.bad[z];
+                hm = b0 || (s > ng && S.bad[z - e]);
+                hp = b0 || (s < L - ng - 1 && S.bad[z + e]);
+            }
+            R Fm[5], Fp[5];
+            double Gm[5], Gp[5], u[5];
+            final_flux(z - e, hm, Fm);
+            final_flux(z, hp, Fp);
+            widen(Fm, Gm);
+            widen(Fp, Gp);
+            if (REG) {
+                record(p, s - ng, Gm);
+                if (s == L - ng - 1) record(p, n, Gp);
+            }
+            const int64_t idx = base(p) + (int64_t)s * sd;
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            {
+                const double U = S.U[v][z];
+                u[v] = sizeof(R) == 8 ? cell_update(U, dtdx64, Gm[v], Gp[v]) : (U + Gm[v]) - Gp[v];
+            }
+            if (fb && !x64::gt0(u[0])) cnt.rare(ENZO_ST_NEG_AFTER);
+            if (x64::is_nan(u[0]) || x64::is_nan(u[4])) cnt.rare(ENZO_ST_NAN);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) a.U[map[v]][idx] = u[v];
+        }
+    }
+
+    __device__ void run()
+    {
+        if (W >= L) {
+            window(0, L, ng, L - ng, 0);
+            return;
+        }
+        int w0 = 0, lo = ng, fresh = 0;
+        for (;;) {
+            const bool last = w0 + W >= L;
+            const int m = last ? L - w0 : W, hi = last ? L - ng : w0 + W - 4;
+            window(w0, m, lo, hi, fresh);
+            if (last) return;
+            // the next window starts four positions left of its first cell
+            const int nw = hi - 4;
+            int p, j;
+            deal(threadIdx.x, 8, p, j);
+            const bool mine = p < np && j < 8;
+            R q[6];
+            double u[5];
+            if (mine) {
+                const int z = slot(p, nw - w0 + j);
+                _Pragma("unroll") for (int v = 0; v < 6; ++v) q[v] = S.q[v][z];
+                _Pragma("unroll") for (int v = 0; v < 5; ++v) u[v] = S.U[v][z];
+            }
+            __syncthreads();
+            if (mine) {
+                const int z = slot(p, j);
+                _Pragma("unroll") for (int v = 0; v < 6; ++v) S.q[v][z] = q[v];
+                _Pragma("unroll") for (int v = 0; v < 5; ++v) S.U[v][z] = u[v];
+            }
+            w0 = nw;
+            lo = hi;
+            fresh = 8;
+        }
+    }
+};
+
+// Persistent kernel: CTAs take (patch, tile) items from a device counter.
+template <class R, int DIR, int THREADS, bool REG, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) ppm_staged_kernel(const __grid_constant__ SweepArgs a)
+{
+    extern __shared__ __align__(16) unsigned char dsmem[];
+    // the tile at hand, found by one thread: its patch, dt/dx (a division each
+    // thread made for itself cost FP32 sweeps more of the FP64 pipe than their
+    // updates)
+    __shared__ enzo_patch s_patch;
+    __shared__ double s_dtdx;
+    __shared__ int s_tile, s_index;
+    StagedSmem<R, THREADS> &S = *reinterpret_cast<StagedSmem<R, THREADS> *>(dsmem);
+    constexpr int A1 = DIR == 0 ? 1 : 0, A2 = DIR == 2 ? 1 : 2;
+    Counters cnt;
+    cnt.st = a.status;
+    const Consts<R> k = make_consts<R>(a.mp);
+    const double dt = a.dt_ptr ? *a.dt_ptr : a.dt;
+    unsigned long long interfaces = 0;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            int tile = (int)atomicAdd(a.tile_counter, 1u);
+            if (tile >= a.prefix[a.npatch]) tile = -1;
+            else {
+                int lo = 0, hi = a.npatch;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if (a.prefix[mid] <= tile) lo = mid; else hi = mid;
+                }
+                s_patch = a.patches[lo];
+                s_index = lo;
+                s_dtdx = x64::div(dt, a.patches[lo].dx[DIR]);
+                tile -= a.prefix[lo];
+            }
+            s_tile = tile;
+        }
+        __syncthreads();
+        const int tile = s_tile;
+        if (tile < 0) break;
+        const enzo_patch &P = s_patch;
+        int rlo[3], rhi[3];
+        sweep_ranges(P, DIR, a.cover_mask, rlo, rhi);
+        const int cnt1 = rhi[A1] - rlo[A1], cnt2 = rhi[A2] - rlo[A2];
+        const int64_t N0 = P.n[0] + 2 * P.ng, N1 = P.n[1] + 2 * P.ng;
+        const int64_t stride[3] = {1, N0, N0 * N1};
+        const int L = P.n[DIR] + 2 * P.ng;
+        int per, W;
+        staged_shape(L, THREADS, per, W);
+        const int pen0 = tile * per;
+        const int np = min(per, cnt1 * cnt2 - pen0);
+        const double dtdx64 = s_dtdx;
+        if (threadIdx.x == 0) interfaces += (unsigned long long)np * (P.n[DIR] + 1);
+        Staged<R, DIR, THREADS, REG> t{a,  P,    S,  k,  cnt,  (R)dtdx64, dtdx64, dt, np, W, L, P.n[DIR], P.ng, pen0,
+                                       cnt1, rlo[A1], rlo[A2], stride[A1], stride[A2], stride[DIR],
+                                       (P.flags & ENZO_PATCH_PERIODIC) != 0, s_index};
+        t.run();
+        __syncthreads();
+    }
+    warp_flush(a.status, interfaces, ENZO_ST_INTERFACES);
+    warp_flush(a.status, cnt.iters, ENZO_ST_NEWTON_ITERS);
+    warp_flush(a.status, cnt.restarts, ENZO_ST_GUESS_RESTARTS);
+}
+
+template <class R, int DIR, int THREADS, bool REG, int MINB>
+cudaError_t launch_staged_one(const SweepArgs &a, cudaStream_t s)
+{
+    auto kern = ppm_staged_kernel<R, DIR, THREADS, REG, MINB>;
+    constexpr int bytes = (int)sizeof(StagedSmem<R, THREADS>);
+    static int cached[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    if (!cached[dev]) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        int sms = 0, per = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, THREADS, bytes);
+        cached[dev] = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+    }
+    kern<<<cached[dev], THREADS, bytes, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <class R, int THREADS, int MINB>
+cudaError_t launch_staged(const SweepArgs &a, cudaStream_t s)
+{
+    if (a.freg) {
+        switch (a.dir) {
+        case 0: return launch_staged_one<R, 0, THREADS, true, MINB>(a, s);
+        case 1: return launch_staged_one<R, 1, THREADS, true, MINB>(a, s);
+        default: return launch_staged_one<R, 2, THREADS, true, MINB>(a, s);
+        }
+    }
+    switch (a.dir) {
+    case 0: return launch_staged_one<R, 0, THREADS, false, MINB>(a, s);
+    case 1: return launch_staged_one<R, 1, THREADS, false, MINB>(a, s);
+    default: return launch_staged_one<R, 2, THREADS, false, MINB>(a, s);
+    }
+}
+
+}  // namespace enzo

@@ -1,0 +1,56 @@
+"""The staged sweep (one tile of whole pencils, or of windows of long ones, in
+shared memory) at its edges: one-cell axes, pencils of exactly one tile, one
+position more, many windows, ragged batches, wrapped and ghosted patches.  FP64
+equals the oracle bit for bit; FP32 equals the marching sweep (chosen by naming
+a tile) bit for bit, counters included."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1307_2265_gb300 as ez
+from gpu_helpers import active, batch_from_patches, gpu_evolve, gpu_patches, oracle_evolve_batch, white_patch
+
+pytestmark = pytest.mark.gpu
+
+BATCHES = {
+    "cells": [(1, 1, 1), (2, 1, 3), (1, 5, 1)],
+    "tile": [(250, 2, 3), (2, 250, 1), (1, 3, 250)],
+    "over": [(251, 3, 2), (3, 251, 2), (2, 1, 251)],
+    "windows": [(700, 1, 2), (2, 333, 3), (1, 2, 520)],
+    "ragged": [(38, 33, 17), (8, 64, 9), (129, 5, 6), (7, 7, 7)],
+}
+
+
+def _patches(sizes, mach):
+    return [white_patch(n, seed=40 + i, mach=mach) for i, n in enumerate(sizes)]
+
+
+@pytest.mark.parametrize("flags", [0, ez.PATCH_PERIODIC])
+@pytest.mark.parametrize("mach", [1.0, 12.0])
+@pytest.mark.parametrize("name", sorted(BATCHES))
+def test_fp64_equals_oracle(name, mach, flags):
+    dx = [1.0 / 64] * 3
+    patches = _patches(BATCHES[name], mach)
+    ora = [[f.copy() for f in U] for U in patches]
+    oracle_evolve_batch(ora, dx, 2, oracle.Params())
+    b = batch_from_patches(patches, dx, flags=flags)
+    gpu_evolve(b, ez.Params(precision=ez.FP64), 2)
+    for G, O in zip(gpu_patches(b), ora):
+        for g, o in zip(G, O):
+            assert np.array_equal(active(g), active(o))
+
+
+@pytest.mark.parametrize("flags", [0, ez.PATCH_PERIODIC])
+@pytest.mark.parametrize("mach", [1.0, 12.0])
+@pytest.mark.parametrize("name", sorted(BATCHES))
+def test_fp32_equals_march(name, mach, flags):
+    dx = [1.0 / 64] * 3
+    out = []
+    for tile in ((0, 0, 0), (128, 128, 128)):
+        b = batch_from_patches(_patches(BATCHES[name], mach), dx, flags=flags)
+        gpu_evolve(b, ez.Params(precision=ez.FP32, tile=tile), 2)
+        out.append((gpu_patches(b), b.read_status()))
+    assert out[0][1] == out[1][1]
+    for G, M in zip(out[0][0], out[1][0]):
+        for g, m in zip(G, M):
+            assert np.array_equal(active(g), active(m), equal_nan=True)
