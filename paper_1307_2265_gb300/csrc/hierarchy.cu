@@ -7,22 +7,16 @@
 // the order written.
 #include <cstdint>
 
+#include "exact64.cuh"
 #include "internal.cuh"
 
 namespace enzo {
 
 constexpr double kEps = 1e-300;
 
-__device__ __forceinline__ double minmod(double a, double b)
-{
-    const double aa = fabs(a), ab = fabs(b);
-    const double m = aa < ab ? aa : ab;
-    const double out = a > 0.0 ? m : (a < 0.0 ? -m : 0.0);
-    return a * b < 0.0 ? 0.0 : out;
-}
-
-// SecondOrderA value of child (kz, ky, kx) of the centre of a 3x3x3 parent
-// neighbourhood Q[z][y][x] (r = 2).  T = double: the FP64 arithmetic (the oracle's order);
+// SecondOrderA slopes (fx, fy, fz) of the centre of a 3x3x3 parent
+// neighbourhood Q[z][y][x] (r = 2); a child's value is the centre plus a quarter
+// of each, signed by its half.  T = double: the FP64 arithmetic (the oracle's order);
 // T = float: the same steps for the FP32 path (ghost values only feed the
 // FP32 reconstruction; conservation is kept by flux correction).
 template <class T>
@@ -34,8 +28,12 @@ __device__ __forceinline__ T minmod_t(T a, T b)
     return a * b < (T)0 ? (T)0 : out;
 }
 
+// Division: IEEE in both precisions; FP64 on the integer pipe (exact64.cuh).
+__device__ __forceinline__ double div_t(double a, double b) { return x64::div(a, b); }
+__device__ __forceinline__ float div_t(float a, float b) { return a / b; }
+
 template <class T>
-__device__ __forceinline__ T second_order_a(const T Q[3][3][3], int kz, int ky, int kx)
+__device__ __forceinline__ void second_order_a(const T Q[3][3][3], T &fx, T &fy, T &fz)
 {
     const T Q0 = Q[1][1][1];
     T C[2][2][2];
@@ -63,23 +61,23 @@ __device__ __forceinline__ T second_order_a(const T Q[3][3][3], int kz, int ky, 
     if (d0 == (T)0) {
         a1 = a2 = a3 = (T)0;
     } else {
-        const T s = ((d1 + d2) + d3) / d0;
+        const T s = div_t((d1 + d2) + d3, d0);
         if (s < (T)0 || s > (T)1) {
             const T sp = s < (T)0 ? (T)0 : (T)1;
-            const T c1 = s < (T)0 ? (d1 / d0 < (T)0 ? (T)1 : (T)0) : (d1 / d0 > (T)0 ? (T)1 : (T)0);
-            const T c2 = s < (T)0 ? (d2 / d0 < (T)0 ? (T)1 : (T)0) : (d2 / d0 > (T)0 ? (T)1 : (T)0);
-            const T c3 = s < (T)0 ? (d3 / d0 < (T)0 ? (T)1 : (T)0) : (d3 / d0 > (T)0 ? (T)1 : (T)0);
+            const T e1 = div_t(d1, d0), c1 = (s < (T)0 ? e1 < (T)0 : e1 > (T)0) ? (T)1 : (T)0;
+            const T e2 = div_t(d2, d0), c2 = (s < (T)0 ? e2 < (T)0 : e2 > (T)0) ? (T)1 : (T)0;
+            const T e3 = div_t(d3, d0), c3 = (s < (T)0 ? e3 < (T)0 : e3 > (T)0) ? (T)1 : (T)0;
             const T num = sp * d0 - ((((T)1 - c1) * d1 + ((T)1 - c2) * d2) + ((T)1 - c3) * d3);
             const T den = ((c1 * d1 + c2 * d2) + c3 * d3) + (sizeof(T) == 8 ? (T)kEps : (T)1e-37f);
-            const T f = num / den;
+            const T f = div_t(num, den);
             a1 = f * c1 * d1 + ((T)1 - c1) * d1;
             a2 = f * c2 * d2 + ((T)1 - c2) * d2;
             a3 = f * c3 * d3 + ((T)1 - c3) * d3;
         }
     }
-    const T fx = a2 + a3, fy = a1 + a3, fz = a1 + a2;
-    const T cx = kx ? (T)0.25 : (T)-0.25, cy = ky ? (T)0.25 : (T)-0.25, cz = kz ? (T)0.25 : (T)-0.25;
-    return ((Q0 + cx * fx) + cy * fy) + cz * fz;
+    fx = a2 + a3;
+    fy = a1 + a3;
+    fz = a1 + a2;
 }
 
 // float <-> double on the integer pipe (d2f_rz, f2d_exact: internal.cuh)
@@ -109,56 +107,75 @@ struct InterpArgs {
     int nbox;
 };
 
-// Ghost cells of the listed boxes get the parent's SecondOrderA value (one CTA
-// per box: boxes are the 3-cell-thick face, edge and corner slabs of a patch's
-// ghost shell; cells that siblings cover are copied afterwards and not listed).
+// Ghost cells of the listed boxes get the parent's SecondOrderA value (boxes
+// are the 3-cell-thick face, edge and corner slabs of a patch's ghost shell, or
+// whole patches in a rebuild; cells that siblings cover are copied afterwards
+// and not listed).  An item is one parent cell of one field: its neighbourhood
+// is loaded, interpolated in time and reduced to slopes once, for all of its
+// children inside the box.  With one thread per child the same neighbourhood
+// was formed up to eight times.  gridDim.y blocks share a box, so that a level
+// of few boxes still fills the chip.  Latency-bound; on a 64^3 root with three
+// levels (about 250 boxes per launch) a launch took 269 us with one thread per
+// child and one CTA per box, and takes 83 us; the root step 30.5 -> 23.2 ms.
 template <class T>
 __global__ void __launch_bounds__(128) interp_ghosts_kernel(const __grid_constant__ InterpArgs a)
 {
     for (int bi = blockIdx.x; bi < a.nbox; bi += gridDim.x) {
         const enzo_copy_box B = a.boxes[bi];
-        const enzo_patch P = a.fine[B.dst];
         const enzo_patch_link L = a.flink[B.dst];
         if (L.parent < 0) continue;
+        const enzo_patch P = a.fine[B.dst];
         const enzo_patch PP = a.par[L.parent];
         const enzo_patch_link PL = a.plink[L.parent];
-        const int e0 = B.hi[0] - B.lo[0], e1 = B.hi[1] - B.lo[1], e2 = B.hi[2] - B.lo[2];
-        const int vol = e0 * e1 * e2, e01 = e0 * e1;
+        int G0[3], m[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            G0[d] = floordiv2(B.lo[d]);
+            m[d] = floordiv2(B.hi[d] - 1) + 1 - G0[d];
+        }
+        const int m01 = m[0] * m[1], vol = m01 * m[2];
         const int N0 = P.n[0] + 2 * P.ng, N1 = P.n[1] + 2 * P.ng;
         const int M0 = PP.n[0] + 2 * PP.ng, M1 = PP.n[1] + 2 * PP.ng;
         const T w = (T)a.w;
-        for (int c = threadIdx.x; c < vol; c += blockDim.x) {
-            const int gz = c / e01, rem = c - gz * e01, gy = rem / e0;
-            const int g[3] = {B.lo[0] + rem - gy * e0, B.lo[1] + gy, B.lo[2] + gz};
-            int kid[3], ps[3];
+        for (int i = blockIdx.y * blockDim.x + threadIdx.x; i < vol * a.nf; i += blockDim.x * gridDim.y) {
+            const int f = i / vol, c = i - f * vol;
+            const double *Po = a.Po[f], *Pn = a.Pn[f];
+            double *U = a.U[f];
+            const int gz = c / m01, rem = c - gz * m01, gy = rem / m[0];
+            const int G[3] = {G0[0] + rem - gy * m[0], G0[1] + gy, G0[2] + gz};
+            const int64_t base = PP.off + (G[0] - PL.origin[0] + PP.ng - 1) +
+                                 (int64_t)M0 * ((G[1] - PL.origin[1] + PP.ng - 1) +
+                                                (int64_t)M1 * (G[2] - PL.origin[2] + PP.ng - 1));
+            T Q[3][3][3], fx, fy, fz;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const int G = floordiv2(g[d]);
-                kid[d] = g[d] - 2 * G;
-                ps[d] = G - PL.origin[d] + PP.ng;
-            }
-            const int64_t dst = P.off + (g[0] - L.origin[0] + P.ng) +
-                                (int64_t)N0 * ((g[1] - L.origin[1] + P.ng) + (int64_t)N1 * (g[2] - L.origin[2] + P.ng));
-            const int64_t base = PP.off + (ps[0] - 1) + (int64_t)M0 * ((ps[1] - 1) + (int64_t)M1 * (ps[2] - 1));
-            for (int f = 0; f < a.nf; ++f) {
-                T Q[3][3][3];
+            for (int dz = 0; dz < 3; ++dz)
 #pragma unroll
-                for (int dz = 0; dz < 3; ++dz)
+                for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-                    for (int dy = 0; dy < 3; ++dy)
+                    for (int dx = 0; dx < 3; ++dx) {
+                        const int64_t idx = base + dx + (int64_t)M0 * (dy + (int64_t)M1 * dz);
+                        const T o = from_d<T>(Po[idx]), n = from_d<T>(Pn[idx]);
+                        Q[dz][dy][dx] = o + w * (n - o);
+                    }
+            second_order_a<T>(Q, fx, fy, fz);
+            const T Q0 = Q[1][1][1];
 #pragma unroll
-                        for (int dx = 0; dx < 3; ++dx) {
-                            const int64_t idx = base + dx + (int64_t)M0 * (dy + (int64_t)M1 * dz);
-                            const T o = from_d<T>(a.Po[f][idx]), n = from_d<T>(a.Pn[f][idx]);
-                            Q[dz][dy][dx] = o + w * (n - o);
-                        }
-                a.U[f][dst] = to_d(second_order_a<T>(Q, kid[2], kid[1], kid[0]));
+            for (int k = 0; k < 8; ++k) {
+                const int g[3] = {2 * G[0] + (k & 1), 2 * G[1] + ((k >> 1) & 1), 2 * G[2] + (k >> 2)};
+                if (g[0] < B.lo[0] || g[0] >= B.hi[0] || g[1] < B.lo[1] || g[1] >= B.hi[1] || g[2] < B.lo[2] ||
+                    g[2] >= B.hi[2])
+                    continue;
+                const T cx = (k & 1) ? (T)0.25 : (T)-0.25, cy = (k & 2) ? (T)0.25 : (T)-0.25,
+                        cz = (k & 4) ? (T)0.25 : (T)-0.25;
+                U[P.off + (g[0] - L.origin[0] + P.ng) +
+                  (int64_t)N0 * ((g[1] - L.origin[1] + P.ng) + (int64_t)N1 * (g[2] - L.origin[2] + P.ng))] =
+                    to_d(((Q0 + cx * fx) + cy * fy) + cz * fz);
             }
         }
     }
 }
 
-// Ghost boxes copied from siblings: one CTA per box (boxes are the face, edge
+// Ghost boxes copied from siblings: one CTA (gridDim.y where boxes are few) per box (boxes are the face, edge
 // and corner slabs of a patch's ghost shell, 27 to a few thousand cells).
 // Each thread loads the fields (five, six with the gas energy) of two cells
 // before storing any, so that enough loads are in flight to cover HBM latency
@@ -190,7 +207,7 @@ __global__ void __launch_bounds__(128) copy_boxes_kernel(const __grid_constant__
                               (int64_t)D01 * (B.lo[2] - DL.origin[2] + D.ng);
         const int64_t sbase = S.off + (B.lo[0] - SL.origin[0] + S.ng) + (int64_t)S0 * (B.lo[1] - SL.origin[1] + S.ng) +
                               (int64_t)S01 * (B.lo[2] - SL.origin[2] + S.ng);
-        for (int c0 = 0; c0 < vol; c0 += 2 * blockDim.x) {
+        for (int c0 = 2 * blockDim.x * blockIdx.y; c0 < vol; c0 += 2 * blockDim.x * gridDim.y) {
             int64_t di[2], si[2];
             double v[2][kMaxFields];
 #pragma unroll
@@ -317,7 +334,7 @@ struct ProjArgs {
     int nfine;
 };
 
-// One CTA per fine patch: its covered coarse cells get the mean of their 8 children.
+// One CTA (gridDim.y where patches are few) per fine patch: its covered coarse cells get the mean of their 8 children.
 __global__ void __launch_bounds__(256) project_kernel(const __grid_constant__ ProjArgs a)
 {
     for (int pi = blockIdx.x; pi < a.nfine; pi += gridDim.x) {
@@ -330,7 +347,7 @@ __global__ void __launch_bounds__(256) project_kernel(const __grid_constant__ Pr
         const int F0 = FP.n[0] + 2 * FP.ng, F1 = FP.n[1] + 2 * FP.ng;
         const int P0 = PP.n[0] + 2 * PP.ng, P1 = PP.n[1] + 2 * PP.ng;
         const int64_t vol = (int64_t)m0 * m1 * m2;
-        for (int64_t c = threadIdx.x; c < vol; c += blockDim.x) {
+        for (int64_t c = blockIdx.y * blockDim.x + threadIdx.x; c < vol; c += blockDim.x * gridDim.y) {
             const int x = (int)(c % m0), y = (int)((c / m0) % m1), z = (int)(c / ((int64_t)m0 * m1));
             const int64_t pidx = PP.off + (FL.origin[0] / 2 + x - PL.origin[0] + PP.ng) +
                                  (int64_t)P0 * ((FL.origin[1] / 2 + y - PL.origin[1] + PP.ng) +
@@ -365,6 +382,16 @@ static int sm_count()
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&s, cudaDevAttrMultiProcessorCount, dev);
     return s > 0 ? s : 1;
+}
+
+// One CTA per box (boxes are short; a grid-stride over a resident grid measured
+// slower), several per box where there are too few boxes for the chip.
+static dim3 box_grid(int boxes)
+{
+    const int full = sm_count() * 16;
+    const int x = boxes < full ? boxes : full;
+    const int y = full / x;
+    return dim3((unsigned)x, (unsigned)(y < 1 ? 1 : (y > 16 ? 16 : y)));
 }
 
 static bool batch_ok(const enzo_patch_batch *b)
@@ -423,9 +450,7 @@ int enzo_ghost_fill_level(const enzo_patch_batch *fine, const enzo_patch_link *f
         a.w = w;
         a.boxes = interp_boxes;
         a.nbox = ninterp;
-        // one CTA per box (boxes are short; a grid-stride over a resident grid
-        // measured slower)
-        const int grid = ninterp < sm_count() * 16 ? ninterp : sm_count() * 16;
+        const dim3 grid = box_grid(ninterp);
         if (precision == ENZO_FP64) interp_ghosts_kernel<double><<<grid, 128, 0, s>>>(a);
         else interp_ghosts_kernel<float><<<grid, 128, 0, s>>>(a);
         note_launch();
@@ -444,7 +469,7 @@ int enzo_ghost_fill_level(const enzo_patch_batch *fine, const enzo_patch_link *f
         c.nf = nf;
         c.boxes = copy_boxes;
         c.nbox = ncopy;
-        copy_boxes_kernel<<<ncopy, 128, 0, s>>>(c);
+        copy_boxes_kernel<<<dim3((unsigned)ncopy, box_grid(ncopy).y), 128, 0, s>>>(c);
         note_launch();
         if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
     }
@@ -472,8 +497,7 @@ int enzo_copy_level(const enzo_patch_batch *dst, const enzo_patch_link *dst_link
     c.nf = dst->ge ? 6 : 5;
     c.boxes = boxes;
     c.nbox = nbox;
-    copy_boxes_kernel<<<nbox < sm_count() * 16 ? nbox : sm_count() * 16, 128, 0,
-                        static_cast<cudaStream_t>(dst->stream)>>>(c);
+    copy_boxes_kernel<<<box_grid(nbox), 128, 0, static_cast<cudaStream_t>(dst->stream)>>>(c);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;
 }
@@ -526,7 +550,7 @@ int enzo_project(const enzo_patch_batch *coarse, const enzo_patch_link *coarse_l
     a.fp = fine->patches;
     a.fl = fine_links;
     a.nfine = fine->npatch;
-    project_kernel<<<fine->npatch, 256, 0,
+    project_kernel<<<dim3((unsigned)fine->npatch, box_grid(fine->npatch).y), 256, 0,
                      static_cast<cudaStream_t>(coarse->stream)>>>(a);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;
