@@ -92,20 +92,35 @@ __global__ void __launch_bounds__(1024) prefix_kernel(const enzo_patch *patches,
     if ((t & 31) == 0 && v) atomicAdd(status + ENZO_ST_BAD_PATCH, v);
 }
 
+// Tiles of a fill kernel's batch: the prefix table, or (prefix == nullptr) a
+// list of this CTA's own in `pre`.
+__device__ __forceinline__ int fill_tiles(const enzo_patch *patches, int npatch, int64_t field_len,
+                                          const int *&prefix, int *pre, unsigned long long *status)
+{
+    if (prefix) return prefix[npatch];
+    int tiles = 0;
+    if ((int)threadIdx.x < npatch) {
+        bool bad = false;
+        tiles = tiles_of(patches[threadIdx.x], field_len, kKindFill, 0, 0, kSweepThreads, 0, bad);
+        if (bad && blockIdx.x == 0) atomicAdd(status + ENZO_ST_BAD_PATCH, 1ull);
+    }
+    const int total = list_scan(tiles, pre);
+    prefix = pre;
+    return total;
+}
+
 // Periodic self ghost fill (Sec. 3.1, case 4): every ghost cell copies the
 // active cell it wraps onto, edges and corners included.
 __global__ void __launch_bounds__(kFillThreads) ghost_fill_kernel(const enzo_patch *patches, int npatch,
                                                                   double *U0, double *U1, double *U2,
                                                                   double *U3, double *U4, double *ge,
-                                                                  const int *prefix)
+                                                                  const int *prefix, int64_t field_len,
+                                                                  unsigned long long *status)
 {
-    const int total = prefix[npatch];
+    __shared__ int pre[kListPatches + 1];
+    const int total = fill_tiles(patches, npatch, field_len, prefix, pre, status);
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-        int lo = 0, hi = npatch;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (prefix[mid] <= tile) lo = mid; else hi = mid;
-        }
+        const int lo = find_patch(prefix, npatch, tile);
         const enzo_patch P = patches[lo];
         const int N0 = P.n[0] + 2 * P.ng, N1 = P.n[1] + 2 * P.ng, N2 = P.n[2] + 2 * P.ng;
         const int64_t cell = (int64_t)(tile - prefix[lo]) * kFillThreads + threadIdx.x;
@@ -151,17 +166,15 @@ __device__ __forceinline__ int bc_map(int x, int n, int bc, bool &flip)
 __global__ void __launch_bounds__(kFillThreads) boundary_fill_kernel(const enzo_patch *patches, int npatch,
                                                                      double *U0, double *U1, double *U2,
                                                                      double *U3, double *U4, double *ge,
-                                                                     const int *prefix, int bcx, int bcy, int bcz)
+                                                                     const int *prefix, int bcx, int bcy, int bcz,
+                                                                     int64_t field_len, unsigned long long *status)
 {
+    __shared__ int pre[kListPatches + 1];
     double *const U[5] = {U0, U1, U2, U3, U4};
     const int bc[3] = {bcx, bcy, bcz};
-    const int total = prefix[npatch];
+    const int total = fill_tiles(patches, npatch, field_len, prefix, pre, status);
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-        int lo = 0, hi = npatch;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (prefix[mid] <= tile) lo = mid; else hi = mid;
-        }
+        const int lo = find_patch(prefix, npatch, tile);
         const enzo_patch P = patches[lo];
         const int N0 = P.n[0] + 2 * P.ng, N1 = P.n[1] + 2 * P.ng, N2 = P.n[2] + 2 * P.ng;
         const int64_t cell = (int64_t)(tile - prefix[lo]) * kFillThreads + threadIdx.x;
@@ -182,15 +195,6 @@ __global__ void __launch_bounds__(kFillThreads) boundary_fill_kernel(const enzo_
         if (ge) ge[dst] = ge[s];
         for (int d = 0; d < 3; ++d) U[1 + d][dst] = flip[d] ? -U[1 + d][s] : U[1 + d][s];
     }
-}
-
-__global__ void dt_finalize_kernel(const unsigned long long *rate_bits, double cfl, double *ws_dt,
-                                   double *dt_out)
-{
-    const double r = __longlong_as_double((long long)*rate_bits);
-    const double dt = cfl / r;
-    *ws_dt = dt;
-    if (dt_out) *dt_out = dt;
 }
 
 int resolve_params(const enzo_params *p, MethodParams &m)
@@ -273,6 +277,9 @@ static int device_sms()
     return sms > 0 ? sms : 1;
 }
 
+// Whether a kernel's CTAs can make the work list themselves (list_scan).
+static bool own_list(const enzo_patch_batch *b) { return b->npatch <= kListPatches; }
+
 // FP32 batches too small for the marching sweep, which takes about 3 us per
 // position of its longest pencil however few pencils there are; the staged
 // sweep's time goes with the zones, 0.065 to 0.08 ns each, against 0.05 ns of a
@@ -302,11 +309,14 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
                       : precision == ENZO_FP64                                  ? kStagedZones64
                       : tile_pencils == 0 && few_pencils(b)                     ? kStagedZones32
                                                                                 : 0;
-    launch_tile_prefix(b->patches, b->npatch, b->field_len, kKindSweep, dir, cover,
-                       reinterpret_cast<int *>(scratch + kWsPrefix), reinterpret_cast<unsigned *>(scratch + kWsCounter),
-                       nullptr, b->status, s, tile, zones);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
+    const bool own = zones && own_list(b);
+    if (!own) {
+        launch_tile_prefix(b->patches, b->npatch, b->field_len, kKindSweep, dir, cover,
+                           reinterpret_cast<int *>(scratch + kWsPrefix),
+                           reinterpret_cast<unsigned *>(scratch + kWsCounter), nullptr, b->status, s, tile, zones);
+        note_launch();
+        if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
+    }
     SweepArgs a;
     a.tile = tile;
     a.zones = zones;
@@ -319,7 +329,8 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     a.dt = dt;
     a.dt_ptr = dt_dev;
     a.mp = m;
-    a.prefix = reinterpret_cast<const int *>(scratch + kWsPrefix);
+    a.prefix = own ? nullptr : reinterpret_cast<const int *>(scratch + kWsPrefix);
+    a.sms = device_sms();
     a.tile_counter = reinterpret_cast<unsigned *>(scratch + kWsCounter);
     a.status = b->status;
     a.freg = b->freg;
@@ -350,11 +361,13 @@ static int sweep_impl(const enzo_patch_batch *b, int dir, double dt, const doubl
 static int fill_impl(const enzo_patch_batch *b)
 {
     cudaStream_t s = static_cast<cudaStream_t>(b->stream);
-    int r = launch_prefix(b, kKindFill, 0, 0, false, s);
-    if (r) return r;
+    if (!own_list(b)) {
+        const int r = launch_prefix(b, kKindFill, 0, 0, false, s);
+        if (r) return r;
+    }
     ghost_fill_kernel<<<device_sms() * 8, kFillThreads, 0, s>>>(
         b->patches, b->npatch, b->U[0], b->U[1], b->U[2], b->U[3], b->U[4], b->ge,
-        reinterpret_cast<const int *>(ws(b) + kWsPrefix));
+        own_list(b) ? nullptr : reinterpret_cast<const int *>(ws(b) + kWsPrefix), b->field_len, b->status);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;
 }
@@ -370,11 +383,14 @@ static bool bc_ok(const int32_t *bc)
 static int boundary_impl(const enzo_patch_batch *b, const int32_t *bc)
 {
     cudaStream_t s = static_cast<cudaStream_t>(b->stream);
-    int r = launch_prefix(b, kKindFill, 0, 0, false, s);
-    if (r) return r;
+    if (!own_list(b)) {
+        const int r = launch_prefix(b, kKindFill, 0, 0, false, s);
+        if (r) return r;
+    }
     boundary_fill_kernel<<<device_sms() * 8, kFillThreads, 0, s>>>(
         b->patches, b->npatch, b->U[0], b->U[1], b->U[2], b->U[3], b->U[4], b->ge,
-        reinterpret_cast<const int *>(ws(b) + kWsPrefix), bc[0], bc[1], bc[2]);
+        own_list(b) ? nullptr : reinterpret_cast<const int *>(ws(b) + kWsPrefix), bc[0], bc[1], bc[2], b->field_len,
+        b->status);
     note_launch();
     return cudaGetLastError() == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;
 }
@@ -591,8 +607,13 @@ int enzo_timestep_cfl(const enzo_patch_batch *b, const enzo_params *p, double *d
         *dt_out = INFINITY;
         return ENZO_OK;
     }
-    r = launch_prefix(b, kKindCells, 0, 0, true, s);
-    if (r) return r;
+    if (own_list(b)) {
+        // the done count and the rate (the kernel's CTAs list the tiles)
+        if (cudaMemsetAsync(ws(b), 0, kWsRateBits + 8, s) != cudaSuccess) return ENZO_ERR_CUDA;
+    } else {
+        r = launch_prefix(b, kKindCells, 0, 0, true, s);
+        if (r) return r;
+    }
     CflArgs a;
     a.patches = b->patches;
     a.npatch = b->npatch;
@@ -601,17 +622,18 @@ int enzo_timestep_cfl(const enzo_patch_batch *b, const enzo_params *p, double *d
     a.gamma = m.gamma;
     a.rho_floor = m.rho_floor;
     a.p_floor = m.p_floor;
-    a.prefix = reinterpret_cast<const int *>(ws(b) + kWsPrefix);
+    a.prefix = own_list(b) ? nullptr : reinterpret_cast<const int *>(ws(b) + kWsPrefix);
     a.rate_bits = reinterpret_cast<unsigned long long *>(ws(b) + kWsRateBits);
+    a.done = reinterpret_cast<unsigned *>(ws(b) + kWsCounter);
     a.status = b->status;
-    const int grid = device_sms() * 8;
+    a.cfl = p->cfl;
+    a.ws_dt = reinterpret_cast<double *>(ws(b) + kWsDt);
+    a.dt_out = dt_out_on_device ? dt_out : nullptr;
+    a.sms = device_sms();
+    const int grid = a.sms * 8;
     cudaError_t e = p->precision == ENZO_FP64 ? launch_cfl_fp64(a, grid, s) : launch_cfl_fp32(a, grid, s);
     note_launch();
     if (e != cudaSuccess) return ENZO_ERR_CUDA;
-    dt_finalize_kernel<<<1, 1, 0, s>>>(a.rate_bits, p->cfl, reinterpret_cast<double *>(ws(b) + kWsDt),
-                                       dt_out_on_device ? dt_out : nullptr);
-    note_launch();
-    if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
     if (!dt_out_on_device) {
         if (cudaMemcpyAsync(dt_out, ws(b) + kWsDt, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess)
             return ENZO_ERR_CUDA;

@@ -57,9 +57,10 @@ struct SweepArgs {
     MethodParams mp;
     int tile = kSweepThreads;  // pencils per CTA tile (= threads per CTA)
     int zones = 0;             // staged sweep: zones per CTA tile (0: marching sweep)
-    const int *prefix;         // [npatch + 1]
+    const int *prefix;         // [npatch + 1]; nullptr: each CTA makes its own list (staged sweep)
     unsigned *tile_counter;
     unsigned long long *status;
+    int sms = 1;               // of the device
     // interface-state log (optional): every log_stride-th interface of a
     // pencil, by a hash of (pencil, position), writes its traced left/right
     // states (rho, u, p) x 2 as float32 into log[slot][6]
@@ -109,6 +110,11 @@ constexpr int kStagedMaxPencils = 8;   // windowed pencils per tile
 // pencils of 134 positions, one per tile, took 816 us.)
 __host__ __device__ inline void staged_shape(int L, int zones, int &pencils, int &window)
 {
+    if (3 * L <= zones) {   // whole pencils idle under a quarter of the lanes
+        window = L;
+        pencils = zones / L;
+        return;
+    }
     float best = 1e30f;
     for (int k = 1; k <= 4096; ++k) {
         const int W = (L + 8 * (k - 1) + k - 1) / k;
@@ -151,9 +157,13 @@ struct CflArgs {
     int64_t field_len;
     const double *U[5];
     double gamma, rho_floor, p_floor;
-    const int *prefix;
-    unsigned long long *rate_bits;
+    const int *prefix;             // nullptr: each CTA makes its own list
+    unsigned long long *rate_bits; // max rate; zero before the launch
+    unsigned *done;                // CTAs that have added theirs; zero before the launch
     unsigned long long *status;
+    double cfl;
+    double *ws_dt, *dt_out;        // the last CTA writes cfl / rate
+    int sms;
 };
 cudaError_t launch_cfl_fp64(const CflArgs &a, int grid, cudaStream_t s);
 cudaError_t launch_cfl_fp32(const CflArgs &a, int grid, cudaStream_t s);
@@ -184,6 +194,45 @@ void launch_tile_prefix(const enzo_patch *patches, int npatch, int64_t field_len
                         int zones = 0);
 
 #ifdef __CUDACC__
+// Work lists of small batches.  A batch of at most kListPatches patches needs
+// no tile-table launch before its kernel: each CTA (of kListPatches threads)
+// sums the patches' tile counts for itself, about a microsecond against the
+// 5.7 us of a prefix launch, and takes tiles in a fixed stride.
+constexpr int kListPatches = 256;
+
+// pre[i] = tiles of the patches before i, from each thread's own count;
+// returns the total.  Every thread of the CTA calls it.
+__device__ __forceinline__ int list_scan(int tiles, int *pre)
+{
+    __shared__ int warp_sum[kListPatches / 32];
+    const int t = threadIdx.x, lane = t & 31;
+    int v = tiles;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    if (lane == 31) warp_sum[t >> 5] = v;
+    __syncthreads();
+    int before = 0;
+    for (int w = 0; w < (t >> 5); ++w) before += warp_sum[w];
+    pre[t + 1] = before + v;
+    if (t == 0) pre[0] = 0;
+    __syncthreads();
+    return pre[kListPatches];
+}
+
+// Patch that holds a tile: the last one with prefix[patch] <= tile.
+__device__ __forceinline__ int find_patch(const int *prefix, int npatch, int tile)
+{
+    int lo = 0, hi = npatch;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (prefix[mid] <= tile) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // float <-> double conversions on the integer pipe.  On GB300 the FP64 pipe
 // retires 2 thread-operations per clock per SM (1/64 of FP32) and F2F
 // conversions run on it, so FP32 work converts with bit operations.

@@ -2237,11 +2237,7 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (sizeof
         const int tile = s_tile;
         __syncthreads();
         if (tile >= total) break;
-        int lo = 0, hi = a.npatch;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (a.prefix[mid] <= tile) lo = mid; else hi = mid;
-        }
+        const int lo = find_patch(a.prefix, a.npatch, tile);
         const enzo_patch P = a.patches[lo];
         int rlo[3], rhi[3];
         sweep_ranges(P, DIR, a.cover_mask, rlo, rhi);
@@ -2306,9 +2302,12 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (sizeof
     if constexpr (EXT == 2) warp_flush(a.status, cnt.gep, ENZO_ST_GE_PRESSURE);
 }
 
-// CFL rate of Sec. 9 per active cell, max-reduced into *rate_bits.  A tile is
-// kCflTile active cells of one patch; one thread finds the tile's patch and
-// the block walks the tile's cells with 32-bit index arithmetic.
+// CFL rate of Sec. 9 per active cell, max-reduced into *rate_bits; the last CTA
+// to add its own turns it into the timestep (a launch of one thread did that
+// before).  A tile is kCflTile active cells of one patch, fewer in a small batch,
+// down to one per thread, so that it spreads over the SMs (a 32^3 grid had eight
+// CTAs: 23 us in FP32, 110 in FP64).  One thread finds the tile's patch and the
+// block walks the tile's cells with 32-bit index arithmetic.
 constexpr int kCflTile = kCflCells;
 
 template <class R>
@@ -2316,28 +2315,39 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
 {
     __shared__ double s_max[8];
     __shared__ int s_patch;
-    const int total = a.prefix[a.npatch];
+    __shared__ int s_pre[kListPatches + 1];
+    const int *prefix = a.prefix;
+    int total, tcells = kCflTile;
+    if (prefix) {
+        total = prefix[a.npatch];
+    } else {
+        int64_t cells = 0;
+        if ((int)threadIdx.x < a.npatch) {
+            const enzo_patch &P = a.patches[threadIdx.x];
+            if (patch_ok(P, a.field_len)) cells = (int64_t)P.n[0] * P.n[1] * P.n[2];
+            else if (blockIdx.x == 0) atomicAdd(a.status + ENZO_ST_BAD_PATCH, 1ull);
+        }
+        for (;; tcells /= 2) {
+            total = list_scan((int)((cells + tcells - 1) / tcells), s_pre);
+            if (tcells == 256 || total >= 4 * a.sms) break;
+            __syncthreads();
+        }
+        prefix = s_pre;
+    }
     double best = 0.0;
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-        if (threadIdx.x == 0) {
-            int lo = 0, hi = a.npatch;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (a.prefix[mid] <= tile) lo = mid; else hi = mid;
-            }
-            s_patch = lo;
-        }
+        if (threadIdx.x == 0) s_patch = find_patch(prefix, a.npatch, tile);
         __syncthreads();
         const int pi = s_patch;
         __syncthreads();
         const enzo_patch P = a.patches[pi];
         const int nx = P.n[0], ny = P.n[1];
         const int64_t ncell = (int64_t)nx * ny * P.n[2];
-        const int64_t first = (int64_t)(tile - a.prefix[pi]) * kCflTile;
+        const int64_t first = (int64_t)(tile - prefix[pi]) * tcells;
         const int64_t N0 = nx + 2 * P.ng, N1 = ny + 2 * P.ng;
         const float idx0 = (float)(1.0 / P.dx[0]), idx1 = (float)(1.0 / P.dx[1]), idx2 = (float)(1.0 / P.dx[2]);
         const x64::Recip id0 = x64::recip(P.dx[0]), id1 = x64::recip(P.dx[1]), id2 = x64::recip(P.dx[2]);
-        for (int t = threadIdx.x; t < kCflTile; t += blockDim.x) {
+        for (int t = threadIdx.x; t < tcells; t += blockDim.x) {
             const int64_t cell = first + t;
             if (cell >= ncell) break;
             const int64_t row = cell / nx;
@@ -2384,6 +2394,12 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
         double m = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = s_max[w] > m ? s_max[w] : m;
         if (m > 0.0) atomicMax(a.rate_bits, (unsigned long long)__double_as_longlong(m));
+        __threadfence();
+        if (atomicAdd(a.done, 1u) == gridDim.x - 1u) {
+            const double dt = a.cfl / __longlong_as_double((long long)atomicMax(a.rate_bits, 0ull));
+            *a.ws_dt = dt;
+            if (a.dt_out) *a.dt_out = dt;
+        }
     }
 }
 
