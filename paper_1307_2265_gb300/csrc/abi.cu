@@ -305,10 +305,10 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     int tile = tile_pencils > 0 ? tile_pencils : kSweepThreads;
     if (precision == ENZO_FP64 || m.guess == ENZO_GUESS_MLP || b->freg || m.options || m.fallback == 2)
         tile = kSweepThreads;
-    const int zones = m.options || m.fallback == 2 || m.guess == ENZO_GUESS_MLP ? 0
-                      : precision == ENZO_FP64                                  ? kStagedZones64
-                      : tile_pencils == 0 && few_pencils(b)                     ? kStagedZones32
-                                                                                : 0;
+    int zones = 0;
+    if (precision == ENZO_FP64) zones = kStagedZones64;
+    else if (m.guess != ENZO_GUESS_MLP && !(m.options & ENZO_OPT_DUAL) && tile_pencils == 0 && few_pencils(b))
+        zones = kStagedZones32;
     const bool own = zones && own_list(b);
     if (!own) {
         launch_tile_prefix(b->patches, b->npatch, b->field_len, kKindSweep, dir, cover,
@@ -342,7 +342,7 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     int dev = 0;
     cudaGetDevice(&dev);
     cudaError_t e;
-    if (precision == ENZO_FP64) e = launch_sweep_fp64(a, sweep_grid_fp64(dev), s);
+    if (precision == ENZO_FP64) e = launch_sweep_fp64(a, s);
     else if (m.guess == ENZO_GUESS_MLP) e = launch_sweep_fp32_learned(a, s);
     else if (tile != kSweepThreads) e = launch_sweep_fp32_tiled(a, s);
     else e = launch_sweep_fp32(a, sweep_grid_fp32(dev), s);

@@ -8,7 +8,9 @@ namespace enzo {
 
 cudaError_t launch_sweep_fp32(const SweepArgs &a, int grid, cudaStream_t s)
 {
-    if (a.zones) return launch_staged<float, kStagedZones32, 3>(a, s);
+    if (a.zones)
+        return a.mp.options || a.mp.fallback == 2 ? launch_staged<float, kStagedZones32, 1, 3>(a, s)
+                                                  : launch_staged<float, kStagedZones32, 0, 3>(a, s);
     return launch_sweep_dir<float>(a, grid, s);
 }
 

@@ -6,13 +6,12 @@
 
 namespace enzo {
 
-cudaError_t launch_sweep_fp64(const SweepArgs &a, int grid, cudaStream_t s)
+cudaError_t launch_sweep_fp64(const SweepArgs &a, cudaStream_t s)
 {
-    if (a.zones) return launch_staged<double, kStagedZones64, 2>(a, s);
-    return launch_sweep_dir<double>(a, grid, s);
+    if (a.mp.options & ENZO_OPT_DUAL) return launch_staged<double, kStagedZones64, 2, 2>(a, s);
+    if (a.mp.options || a.mp.fallback == 2) return launch_staged<double, kStagedZones64, 1, 2>(a, s);
+    return launch_staged<double, kStagedZones64, 0, 2>(a, s);
 }
-
-int sweep_grid_fp64(int device) { return sweep_grid_for<double>(device); }
 
 cudaError_t launch_cfl_fp64(const CflArgs &a, int grid, cudaStream_t s)
 {

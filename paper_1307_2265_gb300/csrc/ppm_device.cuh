@@ -70,6 +70,14 @@ __device__ __forceinline__ float mad2(float a, float b, float c, float d)
     return __fadd_rn(__fmul_rn(a, b), __fmul_rn(c, d));
 }
 
+// The same sum in either precision; the statement applies to FP32 with PIN only.
+template <bool PIN, int OPT, class R>
+__device__ __forceinline__ R blend(R a, R b, R c, R d)
+{
+    if constexpr (PIN && sizeof(R) == 4) return mad2<OPT>(a, b, c, d);
+    else return a * b + c * d;
+}
+
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float y;
@@ -1287,6 +1295,129 @@ struct LearnedGuess {
     }
 };
 
+// Optional reconstruction dissipation of zone j (CW84; optional in
+// Sec. 4.1) on its unlimited edge values el/er, in the order the monotone
+// parabola then takes them: contact steepening of the density, then
+// flattening of all five variables.  Zones j-2..j+2 are zj2m (density and
+// pressure only), zj1m, zj, zj1p, zj2p; dm1 / dp1 are the limited density
+// slopes of zones j-1 / j+1.  Detectors and weights as in the oracle:
+// steepening where the density has an inflection across a jump of at least
+// 1% that is a contact, not a shock; flattening where the flow compresses
+// across a pressure jump above 33%, weighted by the ratio of the 2-zone and
+// 4-zone pressure differences.  With dual energy (elx, erx non-null) the
+// edges of eps (zone value qx) are flattened with the same weight.
+template <class R, bool PIN = false>
+__device__ __forceinline__ void dissipate(const Consts<R> &k, const MethodParams &mp, const Zone<R> &zj1m,
+                                          const Zone<R> &zj, const Zone<R> &zj1p, const Zone<R> &zj2p, R rj2m,
+                                          R pj2m, R dm1, R dp1, R el[5], R er[5], R qx = (R)0, R *elx = nullptr,
+                                          R *erx = nullptr)
+{
+    if (mp.options & ENZO_OPT_STEEPEN) {
+        const R Dm = (zj.r - (R)2 * zj1m.r) + rj2m;
+        const R Dp = (zj2p.r - (R)2 * zj1p.r) + zj.r;
+        const R dr = zj1p.r - zj1m.r;
+        const R rmin = zj1p.r < zj1m.r ? zj1p.r : zj1m.r;
+        const R pmin = zj1p.p < zj1m.p ? zj1p.p : zj1m.p;
+        R et = (R)0;
+        const bool contact = fabs(zj1p.p - zj1m.p) / pmin <= (R)0.1 * k.gamma * (fabs(dr) / rmin);
+        if (Dm * Dp < (R)0 && fabs(dr) >= (R)0.01 * rmin && contact) et = -(Dp - Dm) / ((R)6 * dr);
+        R e = (R)20 * (et - (R)0.05);
+        e = e < (R)0 ? (R)0 : (e > (R)1 ? (R)1 : e);
+        if (e > (R)0) {
+            el[0] = blend<PIN, 0, R>(el[0], (R)1 - e, zj1m.r + (R)0.5 * dm1, e);
+            er[0] = blend<PIN, 1, R>(er[0], (R)1 - e, zj1p.r - (R)0.5 * dp1, e);
+        }
+    }
+    if (mp.options & ENZO_OPT_FLATTEN) {
+        const R dp1p = zj1p.p - zj1m.p, dp2p = zj2p.p - pj2m;
+        const R pmin = zj1p.p < zj1m.p ? zj1p.p : zj1m.p;
+        if (zj1m.u - zj1p.u > (R)0 && fabs(dp1p) > (R)0.33 * pmin) {
+            R f = (R)1;
+            if (dp2p != (R)0) {
+                f = (R)10 * (dp1p / dp2p - (R)0.75);
+                f = f < (R)0 ? (R)0 : (f > (R)1 ? (R)1 : f);
+            }
+            if (f > (R)0) {
+                _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                {
+                    const R q = zv(zj, v);
+                    el[v] = blend<PIN, 0, R>(f, q, (R)1 - f, el[v]);
+                    er[v] = blend<PIN, 0, R>(f, q, (R)1 - f, er[v]);
+                }
+                if (elx) {
+                    *elx = f * qx + ((R)1 - f) * *elx;
+                    *erx = f * qx + ((R)1 - f) * *erx;
+                }
+            }
+        }
+    }
+}
+
+// Diffusive flux at the interface between zones a (left) and b (right):
+// 0.1 max(0, u_a - u_b) times the jump of the conserved state rebuilt from
+// the zone primitives (CW84; optional in Sec. 4.1).  With dual energy
+// (Fx non-null) the gas-energy flux too, rho eps being its conserved value.
+template <class R, bool PIN = false>
+__device__ __forceinline__ void diffuse(const Consts<R> &k, const Zone<R> &za, const Zone<R> &zb, R F[5],
+                                        R ea = (R)0, R eb = (R)0, R *Fx = nullptr)
+{
+    const R du = za.u - zb.u;
+    if (!(du > (R)0)) return;
+    const R nu = (R)0.1 * du;
+    if constexpr (PIN && sizeof(R) == 4) {
+        const float Xa = __fmaf_rn(za.t2, za.t2, mad2<0>(za.u, za.u, za.t1, za.t1));
+        const float Xb = __fmaf_rn(zb.t2, zb.t2, mad2<0>(zb.u, zb.u, zb.t1, zb.t1));
+        const float Ea = __fmaf_rn(__fmul_rn(0.5f, za.r), Xa, za.p / k.gm1);
+        const float Eb = __fmaf_rn(__fmul_rn(0.5f, zb.r), Xb, zb.p / k.gm1);
+        const float d[5] = {za.r - zb.r, mad2<0>(za.r, za.u, -zb.r, zb.u), mad2<0>(za.r, za.t1, -zb.r, zb.t1),
+                            mad2<0>(za.r, za.t2, -zb.r, zb.t2), __fsub_rn(Ea, Eb)};
+        _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = __fmaf_rn(nu, d[v], F[v]);
+        return;   // (FP32 dual energy marches)
+    }
+    R Ua[5], Ub[5];
+    const Zone<R> *zs[2] = {&za, &zb};
+    _Pragma("unroll") for (int z = 0; z < 2; ++z)
+    {
+        R *Uz = z ? Ub : Ua;
+        const Zone<R> &q = *zs[z];
+        Uz[0] = q.r;
+        Uz[1] = q.r * q.u;
+        Uz[2] = q.r * q.t1;
+        Uz[3] = q.r * q.t2;
+        Uz[4] = q.p / k.gm1 + (R)0.5 * q.r * ((q.u * q.u + q.t1 * q.t1) + q.t2 * q.t2);
+    }
+    _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = F[v] + nu * (Ua[v] - Ub[v]);
+    if (Fx) *Fx = *Fx + nu * (za.r * ea - zb.r * eb);
+}
+
+// FP32 screen of fallback mode 2: the zone's conserved state rebuilt from its
+// primitives plus the two faces' FP32 increments.  True only when rho and
+// E keep at least 1e-3 of their old values and the internal energy at
+// least 1e-2 of E, far beyond the FP32 rounding of the estimate; a floored
+// zone never passes (its primitives are not its conserved state).
+template <class R>
+__device__ __forceinline__ bool clearly_ok(const Consts<R> &k, const Zone<R> &z, const R Fm[5], const R Fp[5], R dtdx)
+{
+    if (!(z.r > (R)4 * k.rho_floor) || !(z.p > (R)4 * k.p_floor)) return false;
+    const R E0 = z.p * k.gm1inv + (R)0.5 * z.r * ((z.u * z.u + z.t1 * z.t1) + z.t2 * z.t2);
+    const R rn = z.r + dtdx * (Fm[0] - Fp[0]);
+    const R m0 = z.r * z.u + dtdx * (Fm[1] - Fp[1]);
+    const R m1 = z.r * z.t1 + dtdx * (Fm[2] - Fp[2]);
+    const R m2 = z.r * z.t2 + dtdx * (Fm[3] - Fp[3]);
+    const R En = E0 + dtdx * (Fm[4] - Fp[4]);
+    if (!(rn > (R)1e-3 * z.r) || !(En > (R)1e-3 * E0)) return false;
+    const R twoRE = (R)2 * rn * En;
+    return twoRE - ((m0 * m0 + m1 * m1) + m2 * m2) > (R)1e-2 * twoRE;
+}
+
+// Fallback mode 2: is rho <= 0 or the internal energy not positive?
+__device__ __forceinline__ bool fails_state(const double u[5])
+{
+    if (!(u[0] > 0.0)) return true;
+    const double m2 = (u[1] * u[1] + u[2] * u[2]) + u[3] * u[3];
+    return !((2.0 * u[0]) * u[4] - m2 > 0.0);
+}
+
 // EXT: 0 the default kernels; 1 with the reconstruction options (steepening,
 // flattening, diffusive flux); 2 with those and dual energy.
 template <class R, bool WRAP, int DIR, bool REG = false, int EXT = 0>
@@ -1528,32 +1659,6 @@ struct Marcher {
         return fails_state(u);
     }
 
-    // FP32 screen of fallback mode 2: the zone's conserved state rebuilt from its
-    // primitives plus the two faces' FP32 increments.  True only when rho and
-    // E keep at least 1e-3 of their old values and the internal energy at
-    // least 1e-2 of E, far beyond the FP32 rounding of the estimate; a floored
-    // zone never passes (its primitives are not its conserved state).
-    __device__ __forceinline__ bool clearly_ok(const Zone<R> &z, const R Fm[5], const R Fp[5], R dtdx) const
-    {
-        if (!(z.r > (R)4 * k.rho_floor) || !(z.p > (R)4 * k.p_floor)) return false;
-        const R E0 = z.p * k.gm1inv + (R)0.5 * z.r * ((z.u * z.u + z.t1 * z.t1) + z.t2 * z.t2);
-        const R rn = z.r + dtdx * (Fm[0] - Fp[0]);
-        const R m0 = z.r * z.u + dtdx * (Fm[1] - Fp[1]);
-        const R m1 = z.r * z.t1 + dtdx * (Fm[2] - Fp[2]);
-        const R m2 = z.r * z.t2 + dtdx * (Fm[3] - Fp[3]);
-        const R En = E0 + dtdx * (Fm[4] - Fp[4]);
-        if (!(rn > (R)1e-3 * z.r) || !(En > (R)1e-3 * E0)) return false;
-        const R twoRE = (R)2 * rn * En;
-        return twoRE - ((m0 * m0 + m1 * m1) + m2 * m2) > (R)1e-2 * twoRE;
-    }
-
-    static __device__ __forceinline__ bool fails_state(const double u[5])
-    {
-        if (!(u[0] > 0.0)) return true;
-        const double m2 = (u[1] * u[1] + u[2] * u[2]) + u[3] * u[3];
-        return !((2.0 * u[0]) * u[4] - m2 > 0.0);
-    }
-
     // Density of cell s at the start of the sweep (raw, no floor).
     template <bool RING = false>
     __device__ __forceinline__ double rho_old(int s) const
@@ -1666,89 +1771,6 @@ struct Marcher {
         }
     }
 
-    // Optional reconstruction dissipation of zone j (CW84; optional in
-    // Sec. 4.1) on its unlimited edge values el/er, in the order the monotone
-    // parabola then takes them: contact steepening of the density, then
-    // flattening of all five variables.  Zones j-2..j+2 are zj2m (density and
-    // pressure only), zj1m, zj, zj1p, zj2p; dm1 / dp1 are the limited density
-    // slopes of zones j-1 / j+1.  Detectors and weights as in the oracle:
-    // steepening where the density has an inflection across a jump of at least
-    // 1% that is a contact, not a shock; flattening where the flow compresses
-    // across a pressure jump above 33%, weighted by the ratio of the 2-zone and
-    // 4-zone pressure differences.  With dual energy (elx, erx non-null) the
-    // edges of eps (zone value qx) are flattened with the same weight.
-    __device__ __forceinline__ void dissipate(const MethodParams &mp, const Zone<R> &zj1m, const Zone<R> &zj,
-                                              const Zone<R> &zj1p, const Zone<R> &zj2p, R rj2m, R pj2m, R dm1,
-                                              R dp1, R el[5], R er[5], R qx = (R)0, R *elx = nullptr,
-                                              R *erx = nullptr) const
-    {
-        if (mp.options & ENZO_OPT_STEEPEN) {
-            const R Dm = (zj.r - (R)2 * zj1m.r) + rj2m;
-            const R Dp = (zj2p.r - (R)2 * zj1p.r) + zj.r;
-            const R dr = zj1p.r - zj1m.r;
-            const R rmin = zj1p.r < zj1m.r ? zj1p.r : zj1m.r;
-            const R pmin = zj1p.p < zj1m.p ? zj1p.p : zj1m.p;
-            R et = (R)0;
-            const bool contact = fabs(zj1p.p - zj1m.p) / pmin <= (R)0.1 * k.gamma * (fabs(dr) / rmin);
-            if (Dm * Dp < (R)0 && fabs(dr) >= (R)0.01 * rmin && contact) et = -(Dp - Dm) / ((R)6 * dr);
-            R e = (R)20 * (et - (R)0.05);
-            e = e < (R)0 ? (R)0 : (e > (R)1 ? (R)1 : e);
-            if (e > (R)0) {
-                el[0] = el[0] * ((R)1 - e) + (zj1m.r + (R)0.5 * dm1) * e;
-                er[0] = er[0] * ((R)1 - e) + (zj1p.r - (R)0.5 * dp1) * e;
-            }
-        }
-        if (mp.options & ENZO_OPT_FLATTEN) {
-            const R dp1p = zj1p.p - zj1m.p, dp2p = zj2p.p - pj2m;
-            const R pmin = zj1p.p < zj1m.p ? zj1p.p : zj1m.p;
-            if (zj1m.u - zj1p.u > (R)0 && fabs(dp1p) > (R)0.33 * pmin) {
-                R f = (R)1;
-                if (dp2p != (R)0) {
-                    f = (R)10 * (dp1p / dp2p - (R)0.75);
-                    f = f < (R)0 ? (R)0 : (f > (R)1 ? (R)1 : f);
-                }
-                if (f > (R)0) {
-                    _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                    {
-                        const R q = zv(zj, v);
-                        el[v] = f * q + ((R)1 - f) * el[v];
-                        er[v] = f * q + ((R)1 - f) * er[v];
-                    }
-                    if (elx) {
-                        *elx = f * qx + ((R)1 - f) * *elx;
-                        *erx = f * qx + ((R)1 - f) * *erx;
-                    }
-                }
-            }
-        }
-    }
-
-    // Diffusive flux at the interface between zones a (left) and b (right):
-    // 0.1 max(0, u_a - u_b) times the jump of the conserved state rebuilt from
-    // the zone primitives (CW84; optional in Sec. 4.1).  With dual energy
-    // (Fx non-null) the gas-energy flux too, rho eps being its conserved value.
-    __device__ __forceinline__ void diffuse(const Zone<R> &za, const Zone<R> &zb, R F[5], R ea = (R)0,
-                                            R eb = (R)0, R *Fx = nullptr) const
-    {
-        const R du = za.u - zb.u;
-        if (!(du > (R)0)) return;
-        const R nu = (R)0.1 * du;
-        R Ua[5], Ub[5];
-        const Zone<R> *zs[2] = {&za, &zb};
-        _Pragma("unroll") for (int z = 0; z < 2; ++z)
-        {
-            R *Uz = z ? Ub : Ua;
-            const Zone<R> &q = *zs[z];
-            Uz[0] = q.r;
-            Uz[1] = q.r * q.u;
-            Uz[2] = q.r * q.t1;
-            Uz[3] = q.r * q.t2;
-            Uz[4] = q.p / k.gm1 + (R)0.5 * q.r * ((q.u * q.u + q.t1 * q.t1) + q.t2 * q.t2);
-        }
-        _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = F[v] + nu * (Ua[v] - Ub[v]);
-        if (Fx) *Fx = *Fx + nu * (za.r * ea - zb.r * eb);
-    }
-
     // One pencil with the plain guess: a sliding window over the zones; march
     // step kk loads zone kk and solves interface (kk-3)+1/2.
     template <class GS>
@@ -1846,8 +1868,8 @@ struct Marcher {
                             er[v] = qfcur[v];
                         }
                         R ele = qfep, ere = qfce;
-                        dissipate(mp, zm3, zm2, zm1, z0, r4, p4, ds3, dcur[0], el, er, e2, dual ? &ele : nullptr,
-                                  dual ? &ere : nullptr);
+                        dissipate<R>(k, mp, zm3, zm2, zm1, z0, r4, p4, ds3, dcur[0], el, er, e2, dual ? &ele : nullptr,
+                                     dual ? &ere : nullptr);
                         _Pragma("unroll") for (int v = 0; v < 5; ++v) parabola<R>(zv(zm2, v), el[v], er[v], pL[v], pR[v], pd[v], p6[v]);
                         if (dual) {
                             R eL, eR, ed, e6;
@@ -1887,7 +1909,7 @@ struct Marcher {
                             hll_states<R>(sLprev, sR, k, Fg);
                         }
                         if constexpr (EXT) {
-                            if (mp.options & ENZO_OPT_DIFFUSE) diffuse(zm3, zm2, Fg, e3, e2, dual ? &gcur.F : nullptr);
+                            if (mp.options & ENZO_OPT_DIFFUSE) diffuse<R>(k, zm3, zm2, Fg, e3, e2, dual ? &gcur.F : nullptr);
                         }
                         if (kk >= 6) {
                             // cell c = kk-3: does the Godunov update leave rho > 0?
@@ -1899,7 +1921,7 @@ struct Marcher {
                                     // margins; only unclear cells take the exact FP64 test
                                     // (always with dual energy: the zone pressure may come
                                     // from the gas energy, not from E)
-                                    bad = (sizeof(R) == 8 || dual || !clearly_ok(zm3, Fgprev, Fg, dtdx))
+                                    bad = (sizeof(R) == 8 || dual || !clearly_ok<R>(k, zm3, Fgprev, Fg, dtdx))
                                               ? fails_full(c, Fgprev, Fg, dtdx, dtdx64) : false;
                                 } else if (sizeof(R) == 8) {
                                     bad = !x64::gt0(cell_update(rho_old<RING>(c), dtdx64, (double)Fgprev[0], (double)Fg[0]));

@@ -29,22 +29,34 @@
 
 namespace enzo {
 
-template <class R, int THREADS>
+template <class R, int THREADS, int EXT>
 struct StagedSmem {
-    double U[5][THREADS];      // raw conserved values (rho, m_n, m_t1, m_t2, E)
-    R q[6][THREADS];           // zone primitives r, u, p, t1, t2, c
-    R A[5][THREADS];           // slopes, then right states of the zones' left edges
-    R B[5][THREADS];           // interface values at s+1/2, then fluxes
-    R C[5][THREADS];           // left states of the zones' right edges
-    R save[6][3][kStagedMaxPencils];   // windowed wrapped pencils: the first three active zones
+    static constexpr int NV = EXT == 2 ? 6 : 5;        // traced variables (eps with dual energy)
+    static constexpr int NX = EXT == 2 ? THREADS : 1;
+    double U[5][THREADS];           // raw conserved values (rho, m_n, m_t1, m_t2, E)
+    double ge[NX], En[NX];          // gas energy, E after the update
+    R q[NV + 1][THREADS];           // zone primitives r, u, p, t1, t2, c (and eps)
+    R A[NV][THREADS];               // slopes, then right states of the zones' left edges
+    R B[NV][THREADS];               // interface values at s+1/2, then fluxes
+    R C[NV][THREADS];               // left states of the zones' right edges
+    R uf[NX];                       // interface velocities (gas energy)
+    R ds[EXT ? THREADS : 1];        // density slopes (contact steepening)
+    R save[NV + 1][3][kStagedMaxPencils];   // windowed wrapped pencils: the first three active zones
+    double save_E[kStagedMaxPencils];       // and the first one's E
+    // windowed pencils with dual energy: the last updated cell, whose
+    // resynchronisation waits for its right neighbour's new E
+    double pend[4][kStagedMaxPencils];      // advected ge, E - KE, E, left neighbour's E
+    bool pend_ok[kStagedMaxPencils];
     unsigned char bad[THREADS];
 };
 
-template <class R, int DIR, int THREADS, bool REG>
+template <class R, int DIR, int THREADS, bool REG, int EXT>
 struct Staged {
     static constexpr int A1 = DIR == 0 ? 1 : 0;
     static constexpr int A2 = DIR == 2 ? 1 : 2;
-    using Smem = StagedSmem<R, THREADS>;
+    using Smem = StagedSmem<R, THREADS, EXT>;
+    static constexpr int NV = Smem::NV;
+    static constexpr bool dual = EXT == 2;
     const SweepArgs &a;
     const enzo_patch &P;
     Smem &S;
@@ -88,14 +100,40 @@ struct Staged {
     }
 
     // Final flux of the face right of slot z: the Godunov flux, or HLL from the
-    // zone states beside a cell that failed (Sec. 4.1.2).
-    __device__ __forceinline__ void final_flux(int z, bool hll, R F[5]) const
+    // zone states beside a cell that failed (Sec. 4.1.2); with dual energy its
+    // gas-energy flux and interface velocity (HLL: the mass flux times the
+    // upwind eps, the mean zone velocity).
+    __device__ __forceinline__ void final_flux(int z, bool hll, R F[5], R &gF, R &uf) const
     {
         if (hll) {
-            hll_flux<R>(zone(z), zone(z + next()), k, F);
+            const Zone<R> l = zone(z), r = zone(z + next());
+            hll_flux<R>(l, r, k, F);
+            if constexpr (dual) {
+                gF = F[0] * (F[0] >= (R)0 ? S.q[6][z] : S.q[6][z + next()]);
+                uf = (R)0.5 * (l.u + r.u);
+            }
         } else {
             _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = S.B[v][z];
+            if constexpr (dual) {
+                gF = S.B[5][z];
+                uf = S.uf[z];
+            }
         }
+    }
+
+    __device__ __forceinline__ double widen1(R F) const
+    {
+        return sizeof(R) == 8 ? (double)F : f2d_exact((float)(dtdx * F));
+    }
+
+    // Gas energy of a cell after its resynchronisation (Sec. 4.1.1): E - KE
+    // where that exceeds a tenth of the largest E of the cell and its neighbours.
+    __device__ __forceinline__ static double resync(double g, double e, double E, double El, double Er, bool ok)
+    {
+        double emax = El;
+        if (E > emax) emax = E;
+        if (Er > emax) emax = Er;
+        return ok && e > 0.1 * emax ? e : g;
     }
 
     __device__ __forceinline__ void widen(const R F[5], double G[5]) const
@@ -105,8 +143,8 @@ struct Staged {
     }
 
     // Flux registers of face f (left of active cell f) of pencil p, as the
-    // march records them.
-    __device__ __forceinline__ void record(int p, int f, const double G[5]) const
+    // march records them (a sixth component with dual energy).
+    __device__ __forceinline__ void record(int p, int f, const double G[5], double gG) const
     {
         if (!REG || !a.freg) return;
         const int pe = pen0 + p, i2 = pe / cnt1, i1 = pe - i2 * cnt1;
@@ -116,17 +154,19 @@ struct Staged {
         int64_t oall = 0, obnd = 0;
         for (int d = 0; d < DIR; ++d) {
             const int b1 = d == 0 ? 1 : 0, b2 = d == 2 ? 1 : 2;
-            oall += (int64_t)(P.n[d] + 1) * P.n[b1] * P.n[b2] * 5;
-            obnd += (int64_t)2 * P.n[b1] * P.n[b2] * 5;
+            oall += (int64_t)(P.n[d] + 1) * P.n[b1] * P.n[b2] * NV;
+            obnd += (int64_t)2 * P.n[b1] * P.n[b2] * NV;
         }
         const int64_t row = (int64_t)j2 * na1 + j1;
         if (P.freg_all >= 0) {
-            double *o = a.freg + P.freg_all + oall + (row * (n + 1) + f) * 5;
+            double *o = a.freg + P.freg_all + oall + (row * (n + 1) + f) * NV;
             _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = G[v];
+            if constexpr (dual) o[5] = gG;
         }
         if (P.freg_bnd >= 0 && (f == 0 || f == n)) {
-            double *o = a.freg + P.freg_bnd + obnd + (row * 2 + (f == 0 ? 0 : 1)) * 5;
+            double *o = a.freg + P.freg_bnd + obnd + (row * 2 + (f == 0 ? 0 : 1)) * NV;
             _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = o[v] + (sizeof(R) == 8 ? dt64 * G[v] : G[v]);
+            if constexpr (dual) o[5] = o[5] + (sizeof(R) == 8 ? dt64 * gG : gG);
         }
     }
 
@@ -171,16 +211,26 @@ struct Staged {
                 saved = windowed && c >= n;
             }
             Zone<R> q;
+            R eps = (R)0;
             if (saved) {
                 const int i = s - ng - n;
                 q = Zone<R>{S.save[0][i][p], S.save[1][i][p], S.save[2][i][p],
                             S.save[3][i][p], S.save[4][i][p], S.save[5][i][p]};
+                if constexpr (dual) {
+                    eps = S.save[6][i][p];
+                    if (i == 0) S.U[4][z] = S.save_E[p];
+                }
             } else {
                 double u[5];
                 _Pragma("unroll") for (int v = 0; v < 5; ++v) u[v] = a.U[map[v]][idx];
                 Counters c;
                 c.st = count ? cnt.st : nullptr;
-                if constexpr (sizeof(R) == 4) q = prim_f<true, true>(u[0], u[1], u[2], u[3], u[4], k, c);
+                if constexpr (dual) {
+                    const double g = a.ge[idx];
+                    q = prim_dual<true>(u[0], u[1], u[2], u[3], u[4], g, k, c, eps);
+                    cnt.gep += count ? c.gep : 0u;
+                    S.ge[z] = g;
+                } else if constexpr (sizeof(R) == 4) q = prim_f<true, true>(u[0], u[1], u[2], u[3], u[4], k, c);
                 else q = prim<R, true>(u[0], u[1], u[2], u[3], u[4], k, c);
                 _Pragma("unroll") for (int v = 0; v < 5; ++v) S.U[v][z] = u[v];
                 if (windowed && wrap && s >= ng && s < ng + 3) {
@@ -191,6 +241,10 @@ struct Staged {
                     S.save[3][i][p] = q.t1;
                     S.save[4][i][p] = q.t2;
                     S.save[5][i][p] = q.c;
+                    if constexpr (dual) {
+                        S.save[6][i][p] = eps;
+                        if (i == 0) S.save_E[p] = u[4];
+                    }
                 }
             }
             S.q[0][z] = q.r;
@@ -199,6 +253,7 @@ struct Staged {
             S.q[3][z] = q.t1;
             S.q[4][z] = q.t2;
             S.q[5][z] = q.c;
+            if constexpr (dual) S.q[6][z] = eps;
         }
         __syncthreads();
         const int e = next();
@@ -206,16 +261,23 @@ struct Staged {
         deal(t, m - 2, p, j);
         if (p < np && j < m - 2) {
             const int z = slot(p, 1 + j);
-            _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                S.A[v][z] = limited_slope<R>(S.q[v][z - e], S.q[v][z], S.q[v][z + e]);
+            _Pragma("unroll") for (int v = 0; v < NV; ++v)
+            {
+                const int w = v < 5 ? v : 6;
+                S.A[v][z] = limited_slope<R>(S.q[w][z - e], S.q[w][z], S.q[w][z + e]);
+            }
+            if constexpr (EXT) S.ds[z] = S.A[0][z];
         }
         __syncthreads();
         // interface values right of positions 1 .. m-3
         deal(t, m - 3, p, j);
         if (p < np && j < m - 3) {
             const int z = slot(p, 1 + j);
-            _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                S.B[v][z] = face_value<R, true>(S.q[v][z], S.q[v][z + e], S.A[v][z], S.A[v][z + e]);
+            _Pragma("unroll") for (int v = 0; v < NV; ++v)
+            {
+                const int w = v < 5 ? v : 6;
+                S.B[v][z] = face_value<R, true>(S.q[w][z], S.q[w][z + e], S.A[v][z], S.A[v][z + e]);
+            }
         }
         __syncthreads();
         // parabolas and traced states of positions 2 .. m-3
@@ -223,8 +285,32 @@ struct Staged {
         if (p < np && j < m - 4) {
             const int z = slot(p, 2 + j);
             R pL[5], pR[5], pd[5], p6[5], sR[5], sL[5];
-            _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                parabola<R, true>(S.q[v][z], S.B[v][z - e], S.B[v][z], pL[v], pR[v], pd[v], p6[v]);
+            if constexpr (EXT) {
+                R el[5], er[5], elx = (R)0, erx = (R)0;
+                _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                {
+                    el[v] = S.B[v][z - e];
+                    er[v] = S.B[v][z];
+                }
+                if constexpr (dual) {
+                    elx = S.B[5][z - e];
+                    erx = S.B[5][z];
+                }
+                dissipate<R, true>(k, a.mp, zone(z - e), zone(z), zone(z + e), zone(z + 2 * e), S.q[0][z - 2 * e],
+                                   S.q[2][z - 2 * e], S.ds[z - e], S.ds[z + e], el, er, dual ? S.q[NV][z] : (R)0,
+                                   dual ? &elx : nullptr, dual ? &erx : nullptr);
+                _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                    parabola<R, true>(S.q[v][z], el[v], er[v], pL[v], pR[v], pd[v], p6[v]);
+                if constexpr (dual) {
+                    R xL, xR, xd, x6;
+                    parabola<R, true>(S.q[6][z], elx, erx, xL, xR, xd, x6);
+                    S.A[5][z] = trace_passive<R, -1>(xL, xR, xd, x6, S.q[1][z], dtdx);
+                    S.C[5][z] = trace_passive<R, +1>(xL, xR, xd, x6, S.q[1][z], dtdx);
+                }
+            } else {
+                _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                    parabola<R, true>(S.q[v][z], S.B[v][z - e], S.B[v][z], pL[v], pR[v], pd[v], p6[v]);
+            }
             trace<R, true>(pL, pR, pd, p6, S.q[1][z], S.q[5][z], dtdx, k, sR, sL);
             _Pragma("unroll") for (int v = 0; v < 5; ++v)
             {
@@ -239,7 +325,7 @@ struct Staged {
         if (p < np && j < m - 5) {
             const int w = 2 + j, s = w0 + w, z = slot(p, w);
             const bool own = s >= lo - 1 && (s < hi - 1 || last);
-            R l[5], r[5], F[5];
+            R l[5], r[5], F[5], gF = (R)0;
             _Pragma("unroll") for (int v = 0; v < 5; ++v)
             {
                 l[v] = S.C[v][z];
@@ -254,12 +340,22 @@ struct Staged {
                 }
                 const bool up = o.ustar >= (R)0;
                 phys_flux<R, true>(o.rho, o.u, o.p, up ? l[3] : r[3], up ? l[4] : r[4], k, F);
+                if constexpr (dual) {
+                    gF = F[0] * (up ? S.C[5][z] : S.A[5][z + e]);
+                    S.uf[z] = o.u;
+                }
             } else if (a.mp.solver == ENZO_SOLVER_HLLC) {
                 hllc_states<R>(l, r, k, F);
             } else {
                 hll_states<R>(l, r, k, F);
             }
+            if constexpr (EXT) {
+                if (a.mp.options & ENZO_OPT_DIFFUSE)
+                    diffuse<R, true>(k, zone(z), zone(z + e), F, dual ? S.q[NV][z] : (R)0,
+                                     dual ? S.q[NV][z + e] : (R)0, dual ? &gF : nullptr);
+            }
             _Pragma("unroll") for (int v = 0; v < 5; ++v) S.B[v][z] = F[v];
+            if constexpr (dual) S.B[5][z] = gF;
         }
         __syncthreads();
         // does the Godunov update leave rho > 0?  Cells [lo - 1, hi] of the
@@ -273,7 +369,24 @@ struct Staged {
                 const int s = c0 + j, z = slot(p, s - w0);
                 const R fm = S.B[0][z - e], fp = S.B[0][z];
                 bool bad = false;
-                if (sizeof(R) == 8) {
+                if (EXT && a.mp.fallback == 2) {
+                    // FP32: a screen on the zone's own primitives with wide margins; unclear
+                    // cells (with dual energy all) take the exact test on the update they
+                    // would get
+                    R Fm[5], Fp[5];
+                    _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                    {
+                        Fm[v] = S.B[v][z - e];
+                        Fp[v] = S.B[v][z];
+                    }
+                    if (sizeof(R) == 8 || dual || !clearly_ok<R>(k, zone(z), Fm, Fp, dtdx)) {
+                        double u[5];
+                        _Pragma("unroll") for (int v = 0; v < 5; ++v)
+                            u[v] = sizeof(R) == 8 ? cell_update(S.U[v][z], dtdx64, (double)Fm[v], (double)Fp[v])
+                                                  : (S.U[v][z] + widen1(Fm[v])) - widen1(Fp[v]);
+                        bad = fails_state(u);
+                    }
+                } else if (sizeof(R) == 8) {
                     bad = !x64::gt0(cell_update(S.U[0][z], dtdx64, (double)fm, (double)fp));
                 } else {
                     // FP32 screen; cells near zero are decided in FP64
@@ -289,33 +402,90 @@ struct Staged {
         }
         // update of cells [lo, hi)
         deal(t, hi - lo, p, j);
-        if (p < np && j < hi - lo) {
-            const int s = lo + j, z = slot(p, s - w0);
+        const bool mine = p < np && j < hi - lo;
+        const int s = lo + j, z = mine ? slot(p, s - w0) : 0;
+        const int64_t idx = mine ? base(p) + (int64_t)s * sd : 0;
+        double u[5], gnew = 0.0, enew = 0.0;
+        bool ok = false;
+        if (mine) {
             bool hm = false, hp = false;
             if (any) {
                 const bool b0 = S.bad[z];
                 hm = b0 || (s > ng && S.bad[z - e]);
                 hp = b0 || (s < L - ng - 1 && S.bad[z + e]);
             }
-            R Fm[5], Fp[5];
-            double Gm[5], Gp[5], u[5];
-            final_flux(z - e, hm, Fm);
-            final_flux(z, hp, Fp);
-            widen(Fm, Gm);
-            widen(Fp, Gp);
-            if (REG) {
-                record(p, s - ng, Gm);
-                if (s == L - ng - 1) record(p, n, Gp);
+            R Fm[5], Fp[5], gm = (R)0, gp = (R)0, um = (R)0, up = (R)0;
+            double Gm[5], Gp[5];
+            final_flux(z - e, hm, Fm, gm, um);
+            final_flux(z, hp, Fp, gp, up);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            {
+                Gm[v] = widen1(Fm[v]);
+                Gp[v] = widen1(Fp[v]);
             }
-            const int64_t idx = base(p) + (int64_t)s * sd;
+            const double ggm = dual ? widen1(gm) : 0.0, ggp = dual ? widen1(gp) : 0.0;
+            if (REG) {
+                record(p, s - ng, Gm, ggm);
+                if (s == L - ng - 1) record(p, n, Gp, ggp);
+            }
             _Pragma("unroll") for (int v = 0; v < 5; ++v)
             {
                 const double U = S.U[v][z];
                 u[v] = sizeof(R) == 8 ? cell_update(U, dtdx64, Gm[v], Gp[v]) : (U + Gm[v]) - Gp[v];
             }
-            if (fb && !x64::gt0(u[0])) cnt.rare(ENZO_ST_NEG_AFTER);
+            if constexpr (dual) {
+                const double g0 = S.ge[z];
+                const R pz = S.q[2][z];
+                if (sizeof(R) == 8)
+                    gnew = (g0 + dtdx64 * (ggm - ggp)) - dtdx64 * (double)pz * ((double)up - (double)um);
+                else gnew = ((g0 + ggm) - ggp) - f2d_exact((float)(dtdx * pz * (up - um)));
+                ok = x64::gt0(u[0]);
+                if (ok) {
+                    if (sizeof(R) == 8) {
+                        enew = u[4] - x64::div<-1>((u[1] * u[1] + u[2] * u[2]) + u[3] * u[3], u[0], x64::recip(u[0]));
+                    } else {
+                        const float r = d2f_rz(u[0]), m0 = d2f_rz(u[1]), m1 = d2f_rz(u[2]), m2 = d2f_rz(u[3]);
+                        enew = u[4] - f2d_exact((R)0.5 * ((m0 * m0 + m1 * m1) + m2 * m2) / r);
+                    }
+                }
+            }
+            if (fb && (EXT && a.mp.fallback == 2 ? fails_state(u) : !x64::gt0(u[0]))) cnt.rare(ENZO_ST_NEG_AFTER);
             if (x64::is_nan(u[0]) || x64::is_nan(u[4])) cnt.rare(ENZO_ST_NAN);
             _Pragma("unroll") for (int v = 0; v < 5; ++v) a.U[map[v]][idx] = u[v];
+        }
+        if constexpr (dual) {
+            // resynchronisation: neighbours' new E; ghosts beside the pencil's
+            // ends keep theirs from the start of the sweep
+            double keep[4] = {0.0, 0.0, 0.0, 0.0};
+            bool keep_ok = false;
+            if (mine) S.En[z] = u[4];
+            __syncthreads();
+            if (mine) {
+                double El = s > lo ? S.En[z - e] : S.U[4][z - e];
+                if (!first && s == lo) {
+                    // the window before left its last cell pending
+                    _Pragma("unroll") for (int i = 0; i < 4; ++i) keep[i] = S.pend[i][p];
+                    keep_ok = S.pend_ok[p];
+                    El = keep[2];
+                    a.ge[idx - sd] = resync(keep[0], keep[1], keep[2], keep[3], u[4], keep_ok);
+                }
+                if (s == hi - 1 && !last) {
+                    keep[0] = gnew;
+                    keep[1] = enew;
+                    keep[2] = u[4];
+                    keep[3] = El;
+                    keep_ok = ok;
+                } else {
+                    a.ge[idx] = resync(gnew, enew, u[4], El, s < hi - 1 ? S.En[z + e] : S.U[4][z + e], ok);
+                }
+            }
+            if (!last) {
+                __syncthreads();
+                if (mine && s == hi - 1) {
+                    _Pragma("unroll") for (int i = 0; i < 4; ++i) S.pend[i][p] = keep[i];
+                    S.pend_ok[p] = keep_ok;
+                }
+            }
         }
     }
 
@@ -336,18 +506,20 @@ struct Staged {
             int p, j;
             deal(threadIdx.x, 8, p, j);
             const bool mine = p < np && j < 8;
-            R q[6];
-            double u[5];
+            R q[NV + 1];
+            double u[5], g = 0.0;
             if (mine) {
                 const int z = slot(p, nw - w0 + j);
-                _Pragma("unroll") for (int v = 0; v < 6; ++v) q[v] = S.q[v][z];
+                _Pragma("unroll") for (int v = 0; v < NV + 1; ++v) q[v] = S.q[v][z];
                 _Pragma("unroll") for (int v = 0; v < 5; ++v) u[v] = S.U[v][z];
+                if constexpr (dual) g = S.ge[z];
             }
             __syncthreads();
             if (mine) {
                 const int z = slot(p, j);
-                _Pragma("unroll") for (int v = 0; v < 6; ++v) S.q[v][z] = q[v];
+                _Pragma("unroll") for (int v = 0; v < NV + 1; ++v) S.q[v][z] = q[v];
                 _Pragma("unroll") for (int v = 0; v < 5; ++v) S.U[v][z] = u[v];
+                if constexpr (dual) S.ge[z] = g;
             }
             w0 = nw;
             lo = hi;
@@ -406,7 +578,7 @@ __device__ __forceinline__ int staged_list(const SweepArgs &a, int *pre, int &zo
 
 // Persistent kernel: CTAs take (patch, tile) items from a device counter, or in
 // a fixed stride from their own list of a small batch.
-template <class R, int DIR, int THREADS, bool REG, int MINB>
+template <class R, int DIR, int THREADS, bool REG, int EXT, int MINB>
 __global__ void __launch_bounds__(THREADS, MINB) ppm_staged_kernel(const __grid_constant__ SweepArgs a)
 {
     extern __shared__ __align__(16) unsigned char dsmem[];
@@ -416,7 +588,7 @@ __global__ void __launch_bounds__(THREADS, MINB) ppm_staged_kernel(const __grid_
     __shared__ enzo_patch s_patch;
     __shared__ double s_dtdx;
     __shared__ int s_tile, s_index, s_per, s_window, s_pre[kListPatches + 1];
-    StagedSmem<R, THREADS> &S = *reinterpret_cast<StagedSmem<R, THREADS> *>(dsmem);
+    StagedSmem<R, THREADS, EXT> &S = *reinterpret_cast<StagedSmem<R, THREADS, EXT> *>(dsmem);
     constexpr int A1 = DIR == 0 ? 1 : 0, A2 = DIR == 2 ? 1 : 2;
     Counters cnt;
     cnt.st = a.status;
@@ -462,7 +634,7 @@ __global__ void __launch_bounds__(THREADS, MINB) ppm_staged_kernel(const __grid_
         const int np = min(per, cnt1 * cnt2 - pen0);
         const double dtdx64 = s_dtdx;
         if (threadIdx.x == 0) interfaces += (unsigned long long)np * (P.n[DIR] + 1);
-        Staged<R, DIR, THREADS, REG> t{a,  P,    S,  k,  cnt,  (R)dtdx64, dtdx64, dt, np, W, L, P.n[DIR], P.ng, pen0,
+        Staged<R, DIR, THREADS, REG, EXT> t{a,  P,    S,  k,  cnt,  (R)dtdx64, dtdx64, dt, np, W, L, P.n[DIR], P.ng, pen0,
                                        cnt1, rlo[A1], rlo[A2], stride[A1], stride[A2], stride[DIR],
                                        (P.flags & ENZO_PATCH_PERIODIC) != 0, s_index};
         t.run();
@@ -471,13 +643,14 @@ __global__ void __launch_bounds__(THREADS, MINB) ppm_staged_kernel(const __grid_
     warp_flush(a.status, interfaces, ENZO_ST_INTERFACES);
     warp_flush(a.status, cnt.iters, ENZO_ST_NEWTON_ITERS);
     warp_flush(a.status, cnt.restarts, ENZO_ST_GUESS_RESTARTS);
+    if constexpr (EXT == 2) warp_flush(a.status, cnt.gep, ENZO_ST_GE_PRESSURE);
 }
 
-template <class R, int DIR, int THREADS, bool REG, int MINB>
+template <class R, int DIR, int THREADS, bool REG, int EXT, int MINB>
 cudaError_t launch_staged_one(const SweepArgs &a, cudaStream_t s)
 {
-    auto kern = ppm_staged_kernel<R, DIR, THREADS, REG, MINB>;
-    constexpr int bytes = (int)sizeof(StagedSmem<R, THREADS>);
+    auto kern = ppm_staged_kernel<R, DIR, THREADS, REG, EXT, MINB>;
+    constexpr int bytes = (int)sizeof(StagedSmem<R, THREADS, EXT>);
     static int cached[64] = {0};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -494,20 +667,20 @@ cudaError_t launch_staged_one(const SweepArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <class R, int THREADS, int MINB>
+template <class R, int THREADS, int EXT, int MINB>
 cudaError_t launch_staged(const SweepArgs &a, cudaStream_t s)
 {
     if (a.freg) {
         switch (a.dir) {
-        case 0: return launch_staged_one<R, 0, THREADS, true, MINB>(a, s);
-        case 1: return launch_staged_one<R, 1, THREADS, true, MINB>(a, s);
-        default: return launch_staged_one<R, 2, THREADS, true, MINB>(a, s);
+        case 0: return launch_staged_one<R, 0, THREADS, true, EXT, MINB>(a, s);
+        case 1: return launch_staged_one<R, 1, THREADS, true, EXT, MINB>(a, s);
+        default: return launch_staged_one<R, 2, THREADS, true, EXT, MINB>(a, s);
         }
     }
     switch (a.dir) {
-    case 0: return launch_staged_one<R, 0, THREADS, false, MINB>(a, s);
-    case 1: return launch_staged_one<R, 1, THREADS, false, MINB>(a, s);
-    default: return launch_staged_one<R, 2, THREADS, false, MINB>(a, s);
+    case 0: return launch_staged_one<R, 0, THREADS, false, EXT, MINB>(a, s);
+    case 1: return launch_staged_one<R, 1, THREADS, false, EXT, MINB>(a, s);
+    default: return launch_staged_one<R, 2, THREADS, false, EXT, MINB>(a, s);
     }
 }
 

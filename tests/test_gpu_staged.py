@@ -42,15 +42,60 @@ def test_fp64_equals_oracle(name, mach, flags):
 
 @pytest.mark.parametrize("flags", [0, ez.PATCH_PERIODIC])
 @pytest.mark.parametrize("mach", [1.0, 12.0])
+@pytest.mark.parametrize("options", [0, ez.OPT_STEEPEN | ez.OPT_FLATTEN | ez.OPT_DIFFUSE])
 @pytest.mark.parametrize("name", sorted(BATCHES))
-def test_fp32_equals_march(name, mach, flags):
+def test_fp32_equals_march(name, options, mach, flags):
     dx = [1.0 / 64] * 3
     out = []
     for tile in ((0, 0, 0), (128, 128, 128)):
         b = batch_from_patches(_patches(BATCHES[name], mach), dx, flags=flags)
-        gpu_evolve(b, ez.Params(precision=ez.FP32, tile=tile), 2)
+        gpu_evolve(b, ez.Params(precision=ez.FP32, tile=tile, options=options), 2)
         out.append((gpu_patches(b), b.read_status()))
     assert out[0][1] == out[1][1]
     for G, M in zip(out[0][0], out[1][0]):
         for g, m in zip(G, M):
             assert np.array_equal(active(g), active(m), equal_nan=True)
+
+
+OPTIONS = ez.OPT_STEEPEN | ez.OPT_FLATTEN | ez.OPT_DIFFUSE
+
+
+@pytest.mark.parametrize("flags", [0, ez.PATCH_PERIODIC])
+@pytest.mark.parametrize("mach", [1.0, 12.0])
+@pytest.mark.parametrize("name", ["over", "windows", "ragged"])
+def test_fp64_options_and_fallback_2_equal_oracle(name, mach, flags):
+    dx = [1.0 / 64] * 3
+    patches = _patches(BATCHES[name], mach)
+    ora = [[f.copy() for f in U] for U in patches]
+    oracle_evolve_batch(ora, dx, 2, oracle.Params(options=OPTIONS, fallback=2))
+    b = batch_from_patches(patches, dx, flags=flags)
+    gpu_evolve(b, ez.Params(precision=ez.FP64, options=OPTIONS, fallback=2), 2)
+    for G, O in zip(gpu_patches(b), ora):
+        for g, o in zip(G, O):
+            assert np.array_equal(active(g), active(o))
+
+
+@pytest.mark.parametrize("flags", [0, ez.PATCH_PERIODIC])
+@pytest.mark.parametrize("mach", [1.0, 12.0])
+@pytest.mark.parametrize("name", ["over", "windows", "ragged"])
+def test_fp64_dual_equals_oracle(name, mach, flags):
+    """The gas energy's resynchronisation reaches across a window's edge."""
+    dx = [1.0 / 64] * 3
+    patches = _patches(BATCHES[name], mach)
+    P = oracle.Params(options=oracle.OPT_DUAL | OPTIONS)
+    rng = np.random.default_rng(9)
+    ges = [(U[4] - 0.5 * (U[1] ** 2 + U[2] ** 2 + U[3] ** 2) / np.where(U[0] > 0, U[0], 1.0)) *
+           rng.uniform(0.5, 1.5, U[0].shape) for U in patches]
+    b = batch_from_patches(patches, dx, flags=flags)
+    import torch
+    b.ge = torch.from_numpy(np.concatenate([g.ravel() for g in ges])).to(b.device)
+    for s in range(2):
+        dt = 0.3 / max(oracle.cfl_rate(U, dx, P) for U in patches)
+        for U, g in zip(patches, ges):
+            oracle.step_periodic_dual(U, g, dx, dt, s, P)
+        b.dt_dev.fill_(dt)
+        ez.step(b, ez.Params(precision=ez.FP64, options=ez.OPT_DUAL | OPTIONS), s, b.dt_dev)
+    for i, (G, O) in enumerate(zip(gpu_patches(b), patches)):
+        for g, o in zip(G, O):
+            assert np.array_equal(active(g), active(o))
+        assert np.array_equal(active(b.patch_ge(i).cpu().numpy()), active(ges[i]))
