@@ -122,11 +122,16 @@ __device__ __forceinline__ bool forward_tile(FwdSmem &S, uint32_t &phase, float 
     return true;
 }
 
-__device__ __forceinline__ void write_a1_row(FwdSmem &S, const float x[kMlpIn])
+__device__ __forceinline__ void write_a1_row(FwdSmem &S, int row, const float x[kMlpIn])
 {
-    const int row = threadIdx.x;
+    uint32_t v[3];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) st_bf16(S.a1, tile_off(row, k, 16), k < kMlpIn ? x[k] : 0.0f);
+    for (int k = 0; k < 3; ++k) {
+        const __nv_bfloat162 p = __floats2bfloat162_rn(x[2 * k], x[2 * k + 1]);
+        v[k] = *reinterpret_cast<const uint32_t *>(&p);
+    }
+    *reinterpret_cast<uint4 *>(S.a1 + tile_off(row, 0, 16)) = make_uint4(v[0], v[1], v[2], 0u);
+    *reinterpret_cast<uint4 *>(S.a1 + tile_off(row, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
 __global__ void __launch_bounds__(128) mlp_forward_kernel(const unsigned char *__restrict__ blob,
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const unsigned char *_
         float xi[kMlpIn];
 #pragma unroll
         for (int k = 0; k < kMlpIn; ++k) xi[k] = r < n ? x[r * kMlpIn + k] : 0.0f;
-        write_a1_row(S, xi);
+        write_a1_row(S, threadIdx.x, xi);
         float z2[64];
         if (!forward_tile(S, phase, z2, 0, 64)) {
             S.error = 1;   // every thread of the CTA sees the same result
@@ -178,11 +183,24 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const unsigned char *_
 // ---------------------------------------------------------------------------
 // training
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float warp_sum(float v)
+// Column sums of a warp's 32 x 32 values, v[j] of lane r being row r, column j:
+// lane j returns the sum of column j.  At each step a lane keeps the half of
+// its columns that carries its own bit and gives the other half away, so 31
+// shuffles do what 32 warp reductions (160 shuffles) did.
+__device__ __forceinline__ float column_sums(float v[32])
 {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const float give = up ? v[j] : v[j + o];
+            const float keep = up ? v[j + o] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0];
 }
 
 struct alignas(1024) TrainSmem {
@@ -194,12 +212,41 @@ struct alignas(1024) TrainSmem {
     unsigned char adw1[128 * 128 * 2];       // A of dW1: rows hidden (64 used), cols sample (dZ1^T)
     unsigned char bx[16 * 128 * 2];          // B of dW1: rows input (6 used), cols sample (X^T)
     float gsmall[4 * 64 + 4];                // (unused), db2, dw3, db3 partial sums
+    float part[2][128];                      // each half's part of the output unit
     float loss;
 };
 
 constexpr int kTZ1 = 0, kTZ2 = 64, kTDH1 = 128, kTDW2 = 192, kTDW1 = 256;
 
-__global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__restrict__ blob,
+// Zeros the gradient and the loss (one launch instead of two clears).
+__global__ void mlp_zero_kernel(float *__restrict__ grad, float *__restrict__ loss)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kMlpParams) grad[i] = 0.0f;
+    if (i == 0) *loss = 0.0f;
+}
+
+// Gradient flush of four consecutive parameters.
+__device__ __forceinline__ void add4(float *g, float a, float b, float c, float d)
+{
+    if ((reinterpret_cast<uintptr_t>(g) & 15u) == 0) {
+        atomicAdd(reinterpret_cast<float4 *>(g), make_float4(a, b, c, d));
+    } else {
+        atomicAdd(g, a);
+        atomicAdd(g + 1, b);
+        atomicAdd(g + 2, c);
+        atomicAdd(g + 3, d);
+    }
+}
+
+// A tile of 128 samples per CTA, two threads per sample: each takes 32 of the 64
+// hidden columns (a warp's TMEM lanes go by its index modulo 4, so warps w and
+// w + 4 share rows).  The kernel is one latency chain per tile (four products,
+// each waiting for the activations of the one before) on a chip of one CTA per
+// SM; halving a thread's columns halves the chain's arithmetic.  With one thread
+// per sample, a shuffle reduction per column, scalar gradient adds and five
+// launches a step of 16384 samples took 62 us; with these, 27.6 (this kernel 22).
+__global__ void __launch_bounds__(256) mlp_train_kernel(const unsigned char *__restrict__ blob,
                                                          const float *__restrict__ x,
                                                          const float *__restrict__ target, int64_t n,
                                                          float *__restrict__ grad, float *__restrict__ loss,
@@ -208,24 +255,24 @@ __global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__r
     extern __shared__ unsigned char smem_raw[];
     TrainSmem &T = *reinterpret_cast<TrainSmem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     FwdSmem &S = T.f;
-    const int row = threadIdx.x;
+    const int tid = threadIdx.x, row = tid & 127, half = tid >> 7, c0 = 32 * half;
     load_tile(S.w1, blob + kBlobW1, sizeof(S.w1));
     load_tile(S.w2, blob + kBlobW2, sizeof(S.w2));
     load_tile(T.w2t, blob + kBlobW2T, sizeof(T.w2t));
     const float *f = reinterpret_cast<const float *>(blob + kBlobF32);
-    for (int i = row; i < 193; i += blockDim.x) S.bias[i] = f[i];
-    for (int i = row; i < 4 * 64 + 4; i += blockDim.x) T.gsmall[i] = 0.0f;
-    // rows 64..127 of the weight-gradient A tiles stay zero
-    for (int i = row; i < (int)(sizeof(T.adw2) / 16); i += blockDim.x) {
-        reinterpret_cast<uint4 *>(T.adw2)[i] = make_uint4(0, 0, 0, 0);
-        reinterpret_cast<uint4 *>(T.adw1)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < 193; i += blockDim.x) S.bias[i] = f[i];
+    for (int i = tid; i < 4 * 64 + 4; i += blockDim.x) T.gsmall[i] = 0.0f;
+    // rows 64..127 of the weight-gradient A tiles (the second half of each) stay zero
+    for (int i = tid; i < (int)(sizeof(T.adw2) / 32); i += blockDim.x) {
+        reinterpret_cast<uint4 *>(T.adw2)[sizeof(T.adw2) / 32 + i] = make_uint4(0, 0, 0, 0);
+        reinterpret_cast<uint4 *>(T.adw1)[sizeof(T.adw1) / 32 + i] = make_uint4(0, 0, 0, 0);
     }
-    if (row == 0) {
+    if (tid == 0) {
         mbar_init(&S.mbar, 1);
         S.error = 0;
         T.loss = 0.0f;
     }
-    if (row < 32) tmem_alloc(&S.tmem, 512);
+    if (tid < 32) tmem_alloc(&S.tmem, 512);
     fence_before();
     __syncthreads();
     fence_after();
@@ -241,107 +288,103 @@ __global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__r
         float xi[kMlpIn];
 #pragma unroll
         for (int k = 0; k < kMlpIn; ++k) xi[k] = valid ? x[r * kMlpIn + k] : 0.0f;
-        write_a1_row(S, xi);
-        // X^T for dW1, with input column 6 held at 1 for valid rows: its column
-        // of dW1 = dZ1^T X is then sum_r dz1[r][j], the gradient of b1
+        const float tr = valid ? target[r] : 0.0f;
+        if (half == 0) {
+            write_a1_row(S, row, xi);
+        } else {
+            // X^T for dW1, with input column 6 held at 1 for valid rows: its column
+            // of dW1 = dZ1^T X is then sum_r dz1[r][j], the gradient of b1
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            st_bf16(T.bx, tile_off(k, row, 128), k < kMlpIn ? xi[k] : (k == kMlpIn && valid ? 1.0f : 0.0f));
+            for (int k = 0; k < 16; ++k)
+                st_bf16(T.bx, tile_off(k, row, 128), k < kMlpIn ? xi[k] : (k == kMlpIn && valid ? 1.0f : 0.0f));
+        }
         // forward; keep H1^T for dW2
-        float z2[64];
-        {
-            fence_async_smem();
-            fence_before();
-            __syncthreads();
-            if (row == 0) {
-                fence_after();
-                mma_bf16(S.tmem + kTZ1, smem_desc(smem_u32(S.a1), 128, 256), smem_desc(smem_u32(S.w1), 128, 256),
-                         idesc_bf16_f32(128, 64), false);
-                commit(&S.mbar);
+        fence_async_smem();
+        fence_before();
+        __syncthreads();
+        if (tid == 0) {
+            fence_after();
+            mma_bf16(S.tmem + kTZ1, smem_desc(smem_u32(S.a1), 128, 256), smem_desc(smem_u32(S.w1), 128, 256),
+                     idesc_bf16_f32(128, 64), false);
+            commit(&S.mbar);
+        }
+        if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
+        phase ^= 1u;
+        fence_after();
+#pragma unroll
+        for (int c = c0; c < c0 + 32; c += 16) {
+            float v[16];
+            tmem_ld16(S.tmem + lane_off + kTZ1 + c, v);
+            uint32_t pk[8];
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+                const int j = c + i;
+                const float h0 = silu(v[i] + S.bias[j]), h1 = silu(v[i + 1] + S.bias[j + 1]);
+                const __nv_bfloat162 hp = __floats2bfloat162_rn(h0, h1);
+                pk[i / 2] = *reinterpret_cast<const uint32_t *>(&hp);
+                st_bf16(T.bh1, tile_off(j, row, 128), valid ? h0 : 0.0f);
+                st_bf16(T.bh1, tile_off(j + 1, row, 128), valid ? h1 : 0.0f);
             }
-            if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
-            phase ^= 1u;
+            *reinterpret_cast<uint4 *>(S.a2 + tile_off(row, c, 64)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *reinterpret_cast<uint4 *>(S.a2 + tile_off(row, c + 8, 64)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+        }
+        fence_async_smem();
+        fence_before();
+        __syncthreads();
+        if (tid == 0) {
             fence_after();
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float v[16];
-                tmem_ld16(S.tmem + lane_off + kTZ1 + c * 16, v);
-                uint32_t pk[8];
+            for (int ks = 0; ks < 4; ++ks)
+                mma_bf16(S.tmem + kTZ2, smem_desc(smem_u32(S.a2) + ks * 256, 128, 1024),
+                         smem_desc(smem_u32(S.w2) + ks * 256, 128, 1024), idesc_bf16_f32(128, 64), ks > 0);
+            commit(&S.mbar);
+        }
+        if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
+        phase ^= 1u;
+        fence_after();
+        float z2[32], h2[32];
+        float yp = 0.0f;
 #pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                    const int j = c * 16 + i;
-                    const float h0 = silu(v[i] + S.bias[j]), h1 = silu(v[i + 1] + S.bias[j + 1]);
-                    const __nv_bfloat162 hp = __floats2bfloat162_rn(h0, h1);
-                    pk[i / 2] = *reinterpret_cast<const uint32_t *>(&hp);
-                    st_bf16(T.bh1, tile_off(j, row, 128), valid ? h0 : 0.0f);
-                    st_bf16(T.bh1, tile_off(j + 1, row, 128), valid ? h1 : 0.0f);
-                }
-                *reinterpret_cast<uint4 *>(S.a2 + tile_off(row, c * 16, 64)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                *reinterpret_cast<uint4 *>(S.a2 + tile_off(row, c * 16 + 8, 64)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-            }
-            fence_async_smem();
-            fence_before();
-            __syncthreads();
-            if (row == 0) {
-                fence_after();
+        for (int c = 0; c < 32; c += 16) {
+            float v[16];
+            tmem_ld16(S.tmem + lane_off + kTZ2 + c0 + c, v);
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                    mma_bf16(S.tmem + kTZ2, smem_desc(smem_u32(S.a2) + ks * 256, 128, 1024),
-                             smem_desc(smem_u32(S.w2) + ks * 256, 128, 1024), idesc_bf16_f32(128, 64), ks > 0);
-                commit(&S.mbar);
-            }
-            if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
-            phase ^= 1u;
-            fence_after();
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                float v[16];
-                tmem_ld16(S.tmem + lane_off + kTZ2 + c * 16, v);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) z2[c * 16 + i] = v[i] + S.bias[64 + c * 16 + i];
+            for (int i = 0; i < 16; ++i) {
+                z2[c + i] = v[i] + S.bias[64 + c0 + c + i];
+                h2[c + i] = silu(z2[c + i]);
+                yp = fmaf(S.bias[128 + c0 + c + i], h2[c + i], yp);
             }
         }
+        T.part[half][row] = yp;
+        __syncthreads();
         // output, loss and dL/dz2
-        float yv = S.bias[192];
-#pragma unroll
-        for (int j = 0; j < 64; ++j) yv = fmaf(S.bias[128 + j], silu(z2[j]), yv);
-        const float e = valid ? yv - target[r] : 0.0f;
-        lsum += e * e;
+        const float yv = S.bias[192] + (T.part[0][row] + T.part[1][row]);
+        const float e = valid ? yv - tr : 0.0f;
+        if (half == 0) lsum += e * e;
         const float dy = 2.0f * e * inv_n;
-        // sums over the tile's rows (db3, dw3, db2): reduced across the warp with
-        // shuffles, then one shared-memory add per warp (the 128 rows of a tile
-        // adding into the same 64 words would serialise)
-        const bool lead = (row & 31) == 0;
-        const float sdy = warp_sum(dy);
-        if (lead) atomicAdd(&T.gsmall[192], sdy);
 #pragma unroll
-        for (int j8 = 0; j8 < 64; j8 += 8) {
+        for (int j8 = 0; j8 < 32; j8 += 8) {
             uint32_t pk[4];
 #pragma unroll
             for (int i = 0; i < 8; i += 2) {
-                float d[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int j = j8 + i + h;
-                    const float h2 = silu(z2[j]);
-                    d[h] = dy * S.bias[128 + j] * silu_grad(z2[j]);
-                    const float s3 = warp_sum(dy * h2), s2 = warp_sum(d[h]);
-                    if (lead) {
-                        atomicAdd(&T.gsmall[128 + j], s3);      // dw3
-                        atomicAdd(&T.gsmall[64 + j], s2);       // db2
-                    }
-                    st_bf16(T.adw2, tile_off(j, row, 128), d[h]);
+                    const float d = dy * S.bias[128 + c0 + j] * silu_grad(z2[j]);
+                    st_bf16(T.adw2, tile_off(c0 + j, row, 128), d);
+                    z2[j] = d;
+                    h2[j] *= dy;
                 }
-                const __nv_bfloat162 dp = __floats2bfloat162_rn(d[0], d[1]);
+                const __nv_bfloat162 dp = __floats2bfloat162_rn(z2[j8 + i], z2[j8 + i + 1]);
                 pk[i / 2] = *reinterpret_cast<const uint32_t *>(&dp);
             }
-            *reinterpret_cast<uint4 *>(T.ad2 + tile_off(row, j8, 64)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            *reinterpret_cast<uint4 *>(T.ad2 + tile_off(row, c0 + j8, 64)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
         // dH1 = dZ2 W2 and dW2 += dZ2^T H1
         fence_async_smem();
         fence_before();
         __syncthreads();
-        if (row == 0) {
+        if (tid == 0) {
             fence_after();
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
@@ -354,18 +397,30 @@ __global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__r
                          !first || ks > 0);
             commit(&S.mbar);
         }
+        // while the products run: sums over the tile's rows (db2, dw3, db3), one
+        // shared-memory add per warp and column
+        {
+            const int lane = tid & 31;
+            const float sb = column_sums(z2), s3 = column_sums(h2);
+            atomicAdd(&T.gsmall[64 + c0 + lane], sb);
+            atomicAdd(&T.gsmall[128 + c0 + lane], s3);
+            float sdy = half == 0 ? dy : 0.0f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sdy += __shfl_xor_sync(0xffffffffu, sdy, o);
+            if (half == 0 && lane == 0) atomicAdd(&T.gsmall[192], sdy);
+        }
         if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
         phase ^= 1u;
         fence_after();
         // dz1 = dH1 * silu'(z1), z1 re-read from TMEM
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = c0; c < c0 + 32; c += 16) {
             float dh[16], z1[16];
-            tmem_ld16(S.tmem + lane_off + kTDH1 + c * 16, dh);
-            tmem_ld16(S.tmem + lane_off + kTZ1 + c * 16, z1);
+            tmem_ld16(S.tmem + lane_off + kTDH1 + c, dh);
+            tmem_ld16(S.tmem + lane_off + kTZ1 + c, z1);
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
-                const int j = c * 16 + i;
+                const int j = c + i;
                 const float dz1 = valid ? dh[i] * silu_grad(z1[i] + S.bias[j]) : 0.0f;
                 st_bf16(T.adw1, tile_off(j, row, 128), dz1);   // db1 comes with dW1
             }
@@ -373,7 +428,7 @@ __global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__r
         fence_async_smem();
         fence_before();
         __syncthreads();
-        if (row == 0) {
+        if (tid == 0) {
             fence_after();
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
@@ -393,42 +448,47 @@ __global__ void __launch_bounds__(128) mlp_train_kernel(const unsigned char *__r
     fence_after();
     if (!S.error && !first) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = c0; c < c0 + 32; c += 16) {
             float v[16];
-            tmem_ld16(S.tmem + lane_off + kTDW2 + c * 16, v);
+            tmem_ld16(S.tmem + lane_off + kTDW2 + c, v);
             if (row < 64) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) atomicAdd(&grad[kMW2 + row * 64 + c * 16 + i], v[i]);
+                for (int i = 0; i < 16; i += 4)
+                    add4(&grad[kMW2 + row * 64 + c + i], v[i], v[i + 1], v[i + 2], v[i + 3]);
             }
         }
-        float v[16];
-        tmem_ld16(S.tmem + lane_off + kTDW1, v);
-        if (row < 64) {
+        if (half == 0) {
+            float v[16];
+            tmem_ld16(S.tmem + lane_off + kTDW1, v);
+            if (row < 64) {
 #pragma unroll
-            for (int k = 0; k < kMlpIn; ++k) atomicAdd(&grad[kMW1 + row * kMlpIn + k], v[k]);
-            atomicAdd(&grad[kMB1 + row], v[kMlpIn]);    // the column of ones
+                for (int k = 0; k < kMlpIn; ++k) atomicAdd(&grad[kMW1 + row * kMlpIn + k], v[k]);
+                atomicAdd(&grad[kMB1 + row], v[kMlpIn]);    // the column of ones
+            }
         }
     }
     for (int o = 16; o > 0; o >>= 1) lsum += __shfl_down_sync(0xffffffffu, lsum, o);
-    if ((row & 31) == 0) atomicAdd(&T.loss, lsum);
+    if (half == 0 && (row & 31) == 0) atomicAdd(&T.loss, lsum);
     fence_before();
     __syncthreads();
     if (!S.error) {
-        if (row < 64) {
-            atomicAdd(&grad[kMB2 + row], T.gsmall[64 + row]);
-            atomicAdd(&grad[kMW3 + row], T.gsmall[128 + row]);
-        }
-        if (row == 0) {
+        if (tid < 64) atomicAdd(&grad[kMB2 + tid], T.gsmall[64 + tid]);
+        else if (tid < 128) atomicAdd(&grad[kMW3 + tid - 64], T.gsmall[64 + tid]);
+        else if (tid == 128) {
             atomicAdd(&grad[kMB3], T.gsmall[192]);
             atomicAdd(loss, T.loss * inv_n);
         }
     }
-    if (row == 0 && S.error) atomicAdd(status + ENZO_ST_TIMEOUT, 1ull);
-    if (row < 32) tmem_dealloc(S.tmem, 512);
+    if (tid == 0 && S.error) atomicAdd(status + ENZO_ST_TIMEOUT, 1ull);
+    if (tid < 32) tmem_dealloc(S.tmem, 512);
 }
 
+// Adam on the FP32 master weights; each weight's new value goes straight into
+// its places in the blob (the padding columns keep the zeros of the first
+// packing), which was a launch of its own.
 __global__ void mlp_adam_kernel(float *__restrict__ m, float *__restrict__ mo, float *__restrict__ vo,
-                                const float *__restrict__ g, int step, float lr, float b1, float b2, float eps)
+                                const float *__restrict__ g, int step, float lr, float b1, float b2, float eps,
+                                unsigned char *__restrict__ blob)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kMlpParams) return;
@@ -439,7 +499,24 @@ __global__ void mlp_adam_kernel(float *__restrict__ m, float *__restrict__ mo, f
     vo[i] = vi;
     const float mhat = mi / (1.0f - powf(b1, (float)step));
     const float vhat = vi / (1.0f - powf(b2, (float)step));
-    m[i] -= lr * mhat / (sqrtf(vhat) + eps);
+    const float w = m[i] - lr * mhat / (sqrtf(vhat) + eps);
+    m[i] = w;
+    float *f = reinterpret_cast<float *>(blob + kBlobF32);
+    if (i < kMB1) {
+        st_bf16(blob + kBlobW1, tile_off(i / kMlpIn, i % kMlpIn, 16), w);
+    } else if (i < kMW2) {
+        f[i - kMB1] = w;
+    } else if (i < kMB2) {
+        const int r = i - kMW2, o = r / 64, k = r % 64;
+        st_bf16(blob + kBlobW2, tile_off(o, k, 64), w);
+        st_bf16(blob + kBlobW2T, tile_off(k, o, 64), w);
+    } else if (i < kMW3) {
+        f[64 + i - kMB2] = w;
+    } else if (i < kMB3) {
+        f[128 + i - kMW3] = w;
+    } else {
+        f[192] = w;
+    }
 }
 
 // Riemann-invariant features of left/right states (same definition as the guess
@@ -517,6 +594,7 @@ int enzo_mlp_train_step(float *master, float *adam_m, float *adam_v, int32_t ste
                         unsigned long long *status, void *stream)
 {
     if (!master || !blob || !grad || !loss || !status || n <= 0 || !x || !target) return ENZO_ERR_ARG;
+    if (reinterpret_cast<uintptr_t>(blob) & 15u) return ENZO_ERR_ARG;
     if (lr > 0.0f && (!adam_m || !adam_v || step < 1)) return ENZO_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t smem = sizeof(TrainSmem) + 1024;
@@ -527,20 +605,20 @@ int enzo_mlp_train_step(float *master, float *adam_m, float *adam_v, int32_t ste
             return ENZO_ERR_CUDA;
         attr = true;
     }
-    if (cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, s) != cudaSuccess) return ENZO_ERR_CUDA;
-    if (cudaMemsetAsync(loss, 0, sizeof(float), s) != cudaSuccess) return ENZO_ERR_CUDA;
+    mlp_zero_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(grad, loss);
+    note_launch();
+    if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
     const int64_t tiles = (n + 127) / 128;
     const int grid = (int)(tiles < (int64_t)sms() ? tiles : (int64_t)sms());
-    mlp_train_kernel<<<grid, 128, smem, s>>>(static_cast<const unsigned char *>(blob), x, target, n, grad, loss,
+    mlp_train_kernel<<<grid, 256, smem, s>>>(static_cast<const unsigned char *>(blob), x, target, n, grad, loss,
                                               status);
     note_launch();
     if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
     if (lr > 0.0f) {
         mlp_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(master, adam_m, adam_v, grad, step, lr, 0.9f,
-                                                                 0.999f, 1e-8f);
+                                                                 0.999f, 1e-8f, static_cast<unsigned char *>(blob));
         note_launch();
         if (cudaGetLastError() != cudaSuccess) return ENZO_ERR_CUDA;
-        return enzo_mlp_pack(master, blob, stream);
     }
     return ENZO_OK;
 }

@@ -1,0 +1,36 @@
+"""The training kernel at the edges of its tiles (one sample, one short of a tile,
+one over, more tiles than SMs): gradients against the FP64 backprop with the
+tolerance of test_gpu_mlp.py, and the blob an Adam step leaves equal to the one
+packed from its weights."""
+import numpy as np
+import pytest
+
+import paper_1307_2265_gb300 as ez
+from oracle import mlp as omlp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 127, 129, 20001])
+def test_gradients_and_blob_at_tile_edges(n):
+    import torch
+    rng = np.random.default_rng(100 + n)
+    P = omlp.init(8)
+    P["b1"] = rng.normal(0, 0.1, 64)
+    P["b2"] = rng.normal(0, 0.1, 64)
+    x = rng.normal(0, 1, (n, 6)).astype(np.float32).astype(np.float64)
+    t = rng.normal(0, 1, n).astype(np.float32).astype(np.float64)
+    net = ez.MLP(P)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    loss = net.train_step(xd, td, 0.0)
+    y, cache = omlp.forward(P, x)
+    ref = omlp.backward(P, cache, y, t)
+    assert abs(float(loss.item()) - omlp.mse(y, t)) <= 2e-2 * omlp.mse(y, t)
+    g = net.grads()
+    for k in ref:
+        assert np.linalg.norm(g[k] - ref[k]) <= 1e-2 * np.linalg.norm(ref[k]) + 1e-6, k
+    net.train_step(xd, td, 1e-3)
+    blob = net.blob.clone()
+    net.pack()
+    assert torch.equal(blob.view(torch.int32), net.blob.view(torch.int32))
+    assert int(net.status[12].item()) == 0
