@@ -339,13 +339,11 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     a.log_count = log_count;
     a.log_cap = log_cap;
     a.log_stride = log_stride;
-    int dev = 0;
-    cudaGetDevice(&dev);
     cudaError_t e;
     if (precision == ENZO_FP64) e = launch_sweep_fp64(a, s);
     else if (m.guess == ENZO_GUESS_MLP) e = launch_sweep_fp32_learned(a, s);
     else if (tile != kSweepThreads) e = launch_sweep_fp32_tiled(a, s);
-    else e = launch_sweep_fp32(a, sweep_grid_fp32(dev), s);
+    else e = launch_sweep_fp32(a, s);
     note_launch();
     return e == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;
 }

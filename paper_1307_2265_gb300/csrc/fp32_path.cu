@@ -6,15 +6,13 @@
 
 namespace enzo {
 
-cudaError_t launch_sweep_fp32(const SweepArgs &a, int grid, cudaStream_t s)
+cudaError_t launch_sweep_fp32(const SweepArgs &a, cudaStream_t s)
 {
     if (a.zones)
         return a.mp.options || a.mp.fallback == 2 ? launch_staged<float, kStagedZones32, 1, 3>(a, s)
                                                   : launch_staged<float, kStagedZones32, 0, 3>(a, s);
-    return launch_sweep_dir<float>(a, grid, s);
+    return launch_sweep_dir<float>(a, s);
 }
-
-int sweep_grid_fp32(int device) { return sweep_grid_for<float>(device); }
 
 // Sweep with the learned Newton guess (tensor cores inside the sweep).  TMEM
 // holds 128 columns per CTA, so at most 4 CTAs share an SM.

@@ -134,9 +134,8 @@ __host__ __device__ inline void staged_shape(int L, int zones, int &pencils, int
 
 // Launch helpers implemented in the precision translation units.
 cudaError_t launch_sweep_fp64(const SweepArgs &a, cudaStream_t s);
-cudaError_t launch_sweep_fp32(const SweepArgs &a, int grid, cudaStream_t s);
+cudaError_t launch_sweep_fp32(const SweepArgs &a, cudaStream_t s);
 cudaError_t launch_sweep_fp32_learned(const SweepArgs &a, cudaStream_t s);
-int sweep_grid_fp32(int device);
 // FP32 plain sweep with a chosen tile size (64, 128 or 256 pencils per CTA).
 cudaError_t launch_sweep_fp32_tiled(const SweepArgs &a, cudaStream_t s);
 

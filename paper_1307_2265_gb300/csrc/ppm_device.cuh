@@ -1438,13 +1438,17 @@ struct Marcher {
     // kernel's per-thread slots, stride kSave), FP64 in registers.
     float *wsave;
     static constexpr int kSave = EXT == 2 ? 7 : 6;   // r, u, p, t1, t2, c (and eps with dual energy)
-    // Plain FP32 march: the raw FP64 values (rho, m_n, m_t1, m_t2, E) of the
-    // last kRingSlots positions, in shared memory ([slot][field] x blockDim.x,
-    // this thread's column), so the update of a cell four steps after its load
-    // and the fallback test read them there instead of going back to L2.  In y
-    // and z sweeps the ring also holds the kStage positions ahead of the march,
-    // copied in asynchronously (cp.async) while the march works on earlier
-    // ones: positions k-4 .. k+kStage at step k.
+    // FP32 march with the plain guess: the raw FP64 values (rho, m_n, m_t1,
+    // m_t2, E, and ge with dual energy) of the last kRingSlots positions, in
+    // shared memory ([slot][field] x blockDim.x, this thread's column), so the
+    // update of a cell four steps after its load and the fallback test read
+    // them there instead of going back to L2.  In y and z sweeps the ring also
+    // holds the kStage positions ahead of the march, copied in asynchronously
+    // (cp.async) while the march works on earlier ones: positions k-4 ..
+    // k+kStage at step k.  The option and dual-energy kernels, which loaded
+    // each zone when they needed it and again for its update, took 10.0 and
+    // 14.3 ms a step of a 1000-patch level; with the ring 8.7 and 12.4, and
+    // their spills fell from 72..88 to 16..28 B.
     double *uring;
     static constexpr int kRingSlots = DIR == 0 ? 5 : 8;
     static constexpr int kStage = 3;
@@ -1452,10 +1456,11 @@ struct Marcher {
     // network's shared memory, only for the loads: positions k..k+2, staged
     // two steps ahead, after the network's shared memory.
     static constexpr int kLearnedSlots = 3;
+    static constexpr int kRingFields = EXT == 2 ? 6 : 5;   // and the gas energy with dual energy
     template <int SLOTS = kRingSlots>
     __device__ __forceinline__ double &ring(int s, int f) const
     {
-        return uring[((s % SLOTS) * 5 + f) * (int)blockDim.x];
+        return uring[((s % SLOTS) * kRingFields + f) * (int)blockDim.x];
     }
     Zone<R> c0, c1, c2;
     R ce0, ce1, ce2;
@@ -1551,9 +1556,9 @@ struct Marcher {
         if (s < pc.L) {
             const int64_t idx = index_of(s);
             if (idx >= 0) {
-                const double *src[5] = {a.U[0] + idx, a.U[1 + DIR] + idx, a.U[1 + A1] + idx, a.U[1 + A2] + idx,
-                                        a.U[4] + idx};
-                _Pragma("unroll") for (int f = 0; f < 5; ++f)
+                const double *src[6] = {a.U[0] + idx, a.U[1 + DIR] + idx, a.U[1 + A1] + idx, a.U[1 + A2] + idx,
+                                        a.U[4] + idx, EXT == 2 ? a.ge + idx : nullptr};
+                _Pragma("unroll") for (int f = 0; f < kRingFields; ++f)
                 {
                     const unsigned dst = (unsigned)__cvta_generic_to_shared(&ring<SLOTS>(s, f));
                     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src[f]) : "memory");
@@ -1575,6 +1580,25 @@ struct Marcher {
         asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD) : "memory");
         return prim<R, true>(ring<SLOTS>(s, 0), ring<SLOTS>(s, 1), ring<SLOTS>(s, 2), ring<SLOTS>(s, 3),
                              ring<SLOTS>(s, 4), k, cnt);
+    }
+
+    // The same two with dual energy (zone_dual's primitives).
+    __device__ __forceinline__ Zone<R> zone_staged_dual(int s, Counters &cnt, R &eps)
+    {
+        if (index_of(s) < 0) return saved((s - pc.ng - pc.n) % pc.n, eps);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStage) : "memory");
+        return prim_dual<true>(ring(s, 0), ring(s, 1), ring(s, 2), ring(s, 3), ring(s, 4), ring(s, 5), k, cnt, eps);
+    }
+    __device__ __forceinline__ Zone<R> zone_keep_dual(int s, Counters &cnt, R &eps)
+    {
+        const int64_t idx = index_of(s);
+        if (idx < 0) return saved((s - pc.ng - pc.n) % pc.n, eps);
+        const double *src[6] = {a.U[0] + idx, a.U[1 + DIR] + idx, a.U[1 + A1] + idx, a.U[1 + A2] + idx,
+                                a.U[4] + idx, a.ge + idx};
+        double v[6];
+        _Pragma("unroll") for (int f = 0; f < 6; ++f) v[f] = ld_march<DIR>(src[f]);
+        _Pragma("unroll") for (int f = 0; f < 6; ++f) ring(s, f) = v[f];
+        return prim_dual<true>(v[0], v[1], v[2], v[3], v[4], v[5], k, cnt, eps);
     }
 
     // Zone at pencil position s, its raw values also kept in the ring.
@@ -1645,6 +1669,7 @@ struct Marcher {
     // fluxes Fm, Fp leave rho <= 0 or a non-positive internal energy (tested as
     // 2 rho E - |m|^2 <= 0)?  Decided in FP64 on the exact update the cell would
     // get: the FP64 flux difference, or the FP32 path's widened increments.
+    template <bool RING = false>
     __device__ __forceinline__ bool fails_full(int s, const R Fm[5], const R Fp[5], R dtdx, double dtdx64) const
     {
         const int64_t idx = pc.at(s);
@@ -1652,7 +1677,7 @@ struct Marcher {
         double u[5];
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
         {
-            const double U = a.U[map[v]][idx];
+            const double U = RING ? ring(s, v) : a.U[map[v]][idx];
             if (sizeof(R) == 8) u[v] = cell_update(U, dtdx64, (double)Fm[v], (double)Fp[v]);
             else u[v] = (U + f2d_exact((float)(dtdx * Fm[v]))) - f2d_exact((float)(dtdx * Fp[v]));
         }
@@ -1690,7 +1715,7 @@ struct Marcher {
         double gnew = 0.0;
         const bool dual = EXT == 2 && gm != nullptr;
         if (dual) {
-            const double g0 = a.ge[idx];
+            const double g0 = RING ? ring(s, 5) : a.ge[idx];
             if (sizeof(R) == 8) {
                 gnew = (g0 + dtdx64 * ((double)gm->F - (double)gp->F)) -
                        dtdx64 * (double)pz * ((double)gp->uf - (double)gm->uf);
@@ -1776,7 +1801,7 @@ struct Marcher {
     template <class GS>
     __device__ void run(R dtdx, double dtdx64, const MethodParams &mp, Counters &cnt, GS &guess)
     {
-        constexpr bool RING = sizeof(R) == 4 && EXT == 0;   // the shared-memory ring of raw values
+        constexpr bool RING = sizeof(R) == 4;   // the shared-memory ring of raw values
         const int L = pc.L;
         const bool fb = mp.fallback != 0;
         Zone<R> zm2, zm1, z0;                 // zones k-2, k-1, k
@@ -1824,8 +1849,13 @@ struct Marcher {
             }
             zm2 = zm1;
             zm1 = z0;
-            if (dual) {
-                z0 = zone_dual<true>(kk, cnt, e0);
+            if constexpr (RING && EXT == 2) {
+                if constexpr (DIR != 0) {
+                    stage(kk + kStage);
+                    z0 = zone_staged_dual(kk, cnt, e0);
+                } else {
+                    z0 = zone_keep_dual(kk, cnt, e0);
+                }
             } else {
                 if constexpr (RING && DIR != 0) {
                     stage(kk + kStage);
@@ -1922,7 +1952,7 @@ struct Marcher {
                                     // (always with dual energy: the zone pressure may come
                                     // from the gas energy, not from E)
                                     bad = (sizeof(R) == 8 || dual || !clearly_ok<R>(k, zm3, Fgprev, Fg, dtdx))
-                                              ? fails_full(c, Fgprev, Fg, dtdx, dtdx64) : false;
+                                              ? fails_full<RING>(c, Fgprev, Fg, dtdx, dtdx64) : false;
                                 } else if (sizeof(R) == 8) {
                                     bad = !x64::gt0(cell_update(rho_old<RING>(c), dtdx64, (double)Fgprev[0], (double)Fg[0]));
                                 } else {
@@ -2195,16 +2225,15 @@ __device__ __forceinline__ void warp_flush(unsigned long long *status, unsigned 
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(status + word, v);
 }
 
-// Dynamic shared memory of a plain (not learned) sweep kernel: the FP32
-// default kernels keep the raw values of their last five positions there, and
-// in y and z sweeps three more staged ahead.  The x sweep keeps the ring at
-// five: it depends on L1 keeping its rows' cache lines, and L1 gets what
-// shared memory leaves (with eight slots the x sweep took 20.9 ms instead of
-// 11.9 on the 4000-patch level).
+// Dynamic shared memory of a sweep kernel with the plain guess: the FP32 kernels
+// keep the raw values of their last five positions there, and in y and z sweeps
+// three more staged ahead.  The x sweep keeps the ring at five: it depends on L1
+// keeping its rows' cache lines, and L1 gets what shared memory leaves (with
+// eight slots the x sweep took 20.9 ms instead of 11.9 on the 4000-patch level).
 template <class R, int THREADS, int EXT, int DIR>
 __host__ __device__ constexpr int ring_bytes()
 {
-    return (sizeof(R) == 4 && EXT == 0) ? (DIR == 0 ? 5 : 8) * 5 * THREADS * (int)sizeof(double) : 0;
+    return sizeof(R) == 4 ? (DIR == 0 ? 5 : 8) * (EXT == 2 ? 6 : 5) * THREADS * (int)sizeof(double) : 0;
 }
 
 // Learned kernels: the network's shared memory (aligned to 128 bytes inside
@@ -2447,41 +2476,18 @@ __global__ void __launch_bounds__(256) riemann_kernel(const __grid_constant__ Ri
 
 // Allow a plain kernel's ring (with its static shared memory the total can pass
 // the 48 KB default), once per device.
-template <class R, int DIR, int THREADS, bool REG>
+template <class R, int DIR, int THREADS, bool REG, int EXT = 0>
 cudaError_t ring_prepare(int dev)
 {
-    constexpr int bytes = ring_bytes<R, THREADS, 0, DIR>();
+    constexpr int bytes = ring_bytes<R, THREADS, EXT, DIR>();
     if (bytes == 0) return cudaSuccess;
     static bool done[64] = {false};
     if (dev < 0 || dev >= 64) dev = 0;
     if (done[dev]) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(ppm_sweep_kernel<R, DIR, false, THREADS, REG>,
+    const cudaError_t e = cudaFuncSetAttribute(ppm_sweep_kernel<R, DIR, false, THREADS, REG, EXT>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e == cudaSuccess) done[dev] = true;
     return e;
-}
-
-template <class R>
-int sweep_grid_for(int device)
-{
-    static int cached[64] = {0};
-    if (device < 0 || device >= 64) device = 0;
-    if (cached[device]) return cached[device];
-    int sms = 0, per = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    if constexpr (sizeof(R) == 8) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, kSweepThreads, false, 1>,
-                                                      kSweepThreads, 0);
-    } else {
-        ring_prepare<R, 0, kSweepThreads, false>(device);
-        ring_prepare<R, 1, kSweepThreads, false>(device);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false>, kSweepThreads,
-                                                      ring_bytes<R, kSweepThreads, 0, 1>());
-    }
-    if (sms < 1) sms = 1;
-    if (per < 1) per = 1;
-    cached[device] = sms * per;
-    return cached[device];
 }
 
 template <class R, int THREADS>
@@ -2527,97 +2533,52 @@ cudaError_t launch_tiled(const SweepArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-template <class R>
-cudaError_t launch_sweep_dir(const SweepArgs &a, int grid, cudaStream_t s)
+// One sweep of a kernel family, each direction with its ring; the grid fills the
+// device at the y sweep's occupancy.
+template <class R, int DIR, bool REG, int EXT>
+cudaError_t launch_march_one(const SweepArgs &a, int dev, int grid, cudaStream_t s)
 {
-    if (a.mp.options & ENZO_OPT_DUAL) {
-        // dual energy has its own instantiations too (with and without flux
-        // registers), so the option kernels without it keep their registers;
-        // their persistent grid follows their own occupancy
-        static int cached[2][64] = {{0}};
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64) dev = 0;
-        const int withreg = a.freg ? 1 : 0;
-        if (!cached[withreg][dev]) {
-            int sms = 0, per = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (withreg)
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &per, ppm_sweep_kernel<R, 0, false, kSweepThreads, true, 2>, kSweepThreads, 0);
-            else
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &per, ppm_sweep_kernel<R, 0, false, kSweepThreads, false, 2>, kSweepThreads, 0);
-            cached[withreg][dev] = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
-        }
-        grid = cached[withreg][dev];
-        if (a.freg) {
-            switch (a.dir) {
-            case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, true, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-            case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, true, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-            default: ppm_sweep_kernel<R, 2, false, kSweepThreads, true, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-            }
-            return cudaGetLastError();
-        }
-        switch (a.dir) {
-        case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, false, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-        case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, false, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-        default: ppm_sweep_kernel<R, 2, false, kSweepThreads, false, 2><<<grid, kSweepThreads, 0, s>>>(a); break;
-        }
-        return cudaGetLastError();
+    const cudaError_t e = ring_prepare<R, DIR, kSweepThreads, REG, EXT>(dev);
+    if (e != cudaSuccess) return e;
+    ppm_sweep_kernel<R, DIR, false, kSweepThreads, REG, EXT>
+        <<<grid, kSweepThreads, ring_bytes<R, kSweepThreads, EXT, DIR>(), s>>>(a);
+    return cudaGetLastError();
+}
+
+template <class R, bool REG, int EXT>
+cudaError_t launch_march(const SweepArgs &a, cudaStream_t s)
+{
+    static int cached[64] = {0};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    if (!cached[dev]) {
+        int sms = 0, per = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const cudaError_t e = ring_prepare<R, 1, kSweepThreads, REG, EXT>(dev);
+        if (e != cudaSuccess) return e;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, kSweepThreads, REG, EXT>,
+                                                      kSweepThreads, ring_bytes<R, kSweepThreads, EXT, 1>());
+        cached[dev] = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
     }
-    if (a.mp.options || a.mp.fallback == 2) {
-        // the reconstruction options (and fallback mode 2) have their own
-        // instantiations, so the default kernels stay as they are
-        if (a.freg) {
-            switch (a.dir) {
-            case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, true, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, true, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            default: ppm_sweep_kernel<R, 2, false, kSweepThreads, true, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            }
-        } else {
-            switch (a.dir) {
-            case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, false, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, false, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            default: ppm_sweep_kernel<R, 2, false, kSweepThreads, false, 1><<<grid, kSweepThreads, 0, s>>>(a); break;
-            }
-        }
-        return cudaGetLastError();
+    switch (a.dir) {
+    case 0: return launch_march_one<R, 0, REG, EXT>(a, dev, cached[dev], s);
+    case 1: return launch_march_one<R, 1, REG, EXT>(a, dev, cached[dev], s);
+    default: return launch_march_one<R, 2, REG, EXT>(a, dev, cached[dev], s);
     }
-    if constexpr (sizeof(R) == 8) {
-        return cudaErrorInvalidValue;   // the default FP64 sweep is the staged one
-    } else {
-        constexpr int sx = ring_bytes<R, kSweepThreads, 0, 0>(), syz = ring_bytes<R, kSweepThreads, 0, 1>();
-        {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaError_t e = cudaSuccess;
-            if (a.freg) {
-                if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, true>(dev);
-                if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, true>(dev);
-                if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, true>(dev);
-            } else {
-                if (e == cudaSuccess) e = ring_prepare<R, 0, kSweepThreads, false>(dev);
-                if (e == cudaSuccess) e = ring_prepare<R, 1, kSweepThreads, false>(dev);
-                if (e == cudaSuccess) e = ring_prepare<R, 2, kSweepThreads, false>(dev);
-            }
-            if (e != cudaSuccess) return e;
-        }
-        if (a.freg) {
-            switch (a.dir) {
-            case 0: ppm_sweep_kernel<R, 0, false, kSweepThreads, true><<<grid, kSweepThreads, sx, s>>>(a); break;
-            case 1: ppm_sweep_kernel<R, 1, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
-            default: ppm_sweep_kernel<R, 2, false, kSweepThreads, true><<<grid, kSweepThreads, syz, s>>>(a); break;
-            }
-            return cudaGetLastError();
-        }
-        switch (a.dir) {
-        case 0: ppm_sweep_kernel<R, 0, false><<<grid, kSweepThreads, sx, s>>>(a); break;
-        case 1: ppm_sweep_kernel<R, 1, false><<<grid, kSweepThreads, syz, s>>>(a); break;
-        default: ppm_sweep_kernel<R, 2, false><<<grid, kSweepThreads, syz, s>>>(a); break;
-        }
-        return cudaGetLastError();
-    }
+}
+
+// The reconstruction options (and fallback mode 2) and dual energy have their
+// own instantiations, with and without flux registers, so the default kernels
+// keep their registers.
+template <class R>
+cudaError_t launch_sweep_dir(const SweepArgs &a, cudaStream_t s)
+{
+    if (a.mp.options & ENZO_OPT_DUAL)
+        return a.freg ? launch_march<R, true, 2>(a, s) : launch_march<R, false, 2>(a, s);
+    if (a.mp.options || a.mp.fallback == 2)
+        return a.freg ? launch_march<R, true, 1>(a, s) : launch_march<R, false, 1>(a, s);
+    return a.freg ? launch_march<R, true, 0>(a, s) : launch_march<R, false, 0>(a, s);
 }
 
 }  // namespace enzo
