@@ -2366,6 +2366,7 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
 {
     __shared__ double s_max[8];
     __shared__ int s_patch;
+    __shared__ float s_inv[3];   // 1/dx (three FP64 divisions per thread and tile cost more than the loads)
     __shared__ int s_pre[kListPatches + 1];
     const int *prefix = a.prefix;
     int total, tcells = kCflTile;
@@ -2386,55 +2387,76 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
         prefix = s_pre;
     }
     double best = 0.0;
+    float fbest = 0.0f;
     for (int tile = blockIdx.x; tile < total; tile += gridDim.x) {
-        if (threadIdx.x == 0) s_patch = find_patch(prefix, a.npatch, tile);
+        if (threadIdx.x < 3) {
+            const int pt = find_patch(prefix, a.npatch, tile);
+            s_inv[threadIdx.x] = (float)x64::div(1.0, a.patches[pt].dx[threadIdx.x]);
+            s_patch = pt;
+        }
         __syncthreads();
         const int pi = s_patch;
+        const float idx0 = s_inv[0], idx1 = s_inv[1], idx2 = s_inv[2];
         __syncthreads();
         const enzo_patch P = a.patches[pi];
-        const int nx = P.n[0], ny = P.n[1];
-        const int64_t ncell = (int64_t)nx * ny * P.n[2];
         const int64_t first = (int64_t)(tile - prefix[pi]) * tcells;
+        const int64_t left = (int64_t)P.n[0] * P.n[1] * P.n[2] - first;
+        const int cells = left < tcells ? (int)left : tcells;
+        // cell coordinates from 32-bit divisions: the tile's first row, then
+        // offsets within the tile
+        const unsigned nx = P.n[0], ny = P.n[1];
+        const int64_t row0 = first / nx;
+        const unsigned x0 = (unsigned)(first - row0 * nx), z0 = (unsigned)(row0 / ny), y0 = (unsigned)(row0 - (int64_t)z0 * ny);
         const int64_t N0 = nx + 2 * P.ng, N1 = ny + 2 * P.ng;
-        const float idx0 = (float)(1.0 / P.dx[0]), idx1 = (float)(1.0 / P.dx[1]), idx2 = (float)(1.0 / P.dx[2]);
         const x64::Recip id0 = x64::recip(P.dx[0]), id1 = x64::recip(P.dx[1]), id2 = x64::recip(P.dx[2]);
-        for (int t = threadIdx.x; t < tcells; t += blockDim.x) {
-            const int64_t cell = first + t;
-            if (cell >= ncell) break;
-            const int64_t row = cell / nx;
-            const int i = (int)(cell - row * nx);
-            const int j = (int)(row % ny);
-            const int kz = (int)(row / ny);
-            const int64_t idx = P.off + (i + P.ng) + N0 * ((j + P.ng) + N1 * (int64_t)(kz + P.ng));
-            if (sizeof(R) == 8) {
-                double rho = a.U[0][idx];
-                if (!x64::ge_pos(rho, a.rho_floor)) rho = a.rho_floor;
-                const double mx = a.U[1][idx], my = a.U[2][idx], mz = a.U[3][idx];
-                const x64::Recip ir = x64::recip(rho);
-                const double ke = x64::div<-1>((mx * mx + my * my) + mz * mz, rho, ir);
-                double p = (a.gamma - 1.0) * (a.U[4][idx] - ke);
-                if (!x64::ge_pos(p, a.p_floor)) p = a.p_floor;
-                const double c = x64::sqrt_rn(x64::div(a.gamma * p, rho, ir));
-                const double r = (x64::div(c + fabs(x64::div(mx, rho, ir)), P.dx[0], id0) +
-                                  x64::div(c + fabs(x64::div(my, rho, ir)), P.dx[1], id1)) +
-                                 x64::div(c + fabs(x64::div(mz, rho, ir)), P.dx[2], id2);
-                best = r > best ? r : best;
-            } else {
-                Counters quiet;
-                Consts<float> k;
-                k.gamma = (float)a.gamma;
-                k.gm1 = (float)(a.gamma - 1.0);
-                k.rho_floor = (float)a.rho_floor;
-                k.p_floor = (float)a.p_floor;
-                k.eta_eke = 0.05f;
-                const Zone<float> z = prim_f<false>(a.U[0][idx], a.U[1][idx], a.U[2][idx], a.U[3][idx],
-                                                    a.U[4][idx], k, quiet);
-                const float r = ((z.c + fabsf(z.u)) * idx0 + (z.c + fabsf(z.t1)) * idx1) +
-                                (z.c + fabsf(z.t2)) * idx2;
-                best = (double)r > best ? (double)r : best;
+        // U cells of a thread at a time, every load before the first use
+        constexpr int U = sizeof(R) == 8 ? 2 : 4;
+        for (int t0 = threadIdx.x; t0 < cells; t0 += U * blockDim.x) {
+            double v[U][5];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const unsigned t = t0 + i * blockDim.x;
+                const unsigned xx = x0 + ((int)t < cells ? t : 0u), r = xx / nx, yy = y0 + r;
+                const unsigned zz = yy / ny;
+                const int64_t idx = P.off + (xx - r * nx + P.ng) +
+                                    N0 * ((yy - zz * ny + P.ng) + N1 * (int64_t)(z0 + zz + P.ng));
+#pragma unroll
+                for (int f = 0; f < 5; ++f) v[i][f] = (int)t < cells ? __ldg(a.U[f] + idx) : 0.0;
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                if (t0 + i * (int)blockDim.x >= cells) break;
+                if (sizeof(R) == 8) {
+                    double rho = v[i][0];
+                    if (!x64::ge_pos(rho, a.rho_floor)) rho = a.rho_floor;
+                    const double mx = v[i][1], my = v[i][2], mz = v[i][3];
+                    const x64::Recip ir = x64::recip(rho);
+                    const double ke = x64::div<-1>((mx * mx + my * my) + mz * mz, rho, ir);
+                    double p = (a.gamma - 1.0) * (v[i][4] - ke);
+                    if (!x64::ge_pos(p, a.p_floor)) p = a.p_floor;
+                    const double c = x64::sqrt_rn(x64::div(a.gamma * p, rho, ir));
+                    const double r = (x64::div(c + fabs(x64::div(mx, rho, ir)), P.dx[0], id0) +
+                                      x64::div(c + fabs(x64::div(my, rho, ir)), P.dx[1], id1)) +
+                                     x64::div(c + fabs(x64::div(mz, rho, ir)), P.dx[2], id2);
+                    best = r > best ? r : best;
+                } else {
+                    Counters quiet;
+                    Consts<float> k;
+                    k.gamma = (float)a.gamma;
+                    k.gm1 = (float)(a.gamma - 1.0);
+                    k.rho_floor = (float)a.rho_floor;
+                    k.p_floor = (float)a.p_floor;
+                    k.eta_eke = 0.05f;
+                    const Zone<float> z = prim_f<false>(v[i][0], v[i][1], v[i][2], v[i][3], v[i][4], k, quiet);
+                    const float r = ((z.c + fabsf(z.u)) * idx0 + (z.c + fabsf(z.t1)) * idx1) +
+                                    (z.c + fabsf(z.t2)) * idx2;
+                    fbest = r > fbest ? r : fbest;
+                }
             }
         }
     }
+    // (exact, and off the FP64 pipe: one widening per thread, not per cell)
+    if (sizeof(R) == 4 && fbest > 0.0f) best = (double)fbest;
     for (int o = 16; o > 0; o >>= 1) {
         const double other = __shfl_down_sync(0xffffffffu, best, o);
         best = other > best ? other : best;
