@@ -305,9 +305,8 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     // pencils per tile of the default FP32 march: 64 (more, smaller CTAs even out
     // the ends of ragged patches: 30.8 -> 30.4 ms a step of the 4000-patch level,
     // 31.7 with 256)
-    int tile = tile_pencils > 0 ? tile_pencils : 64;
-    if (precision == ENZO_FP64 || m.guess == ENZO_GUESS_MLP || b->freg || m.options || m.fallback == 2)
-        tile = kSweepThreads;
+    int tile = tile_pencils > 0 && !b->freg ? tile_pencils : 64;
+    if (precision == ENZO_FP64 || m.guess == ENZO_GUESS_MLP || m.options || m.fallback == 2) tile = kSweepThreads;
     int zones = 0;
     if (precision == ENZO_FP64) zones = kStagedZones64;
     else if (m.guess != ENZO_GUESS_MLP && !(m.options & ENZO_OPT_DUAL) && tile_pencils == 0 && few_pencils(b))
@@ -345,7 +344,6 @@ int sweep_with_scratch(const enzo_patch_batch *b, char *scratch, int dir, double
     cudaError_t e;
     if (precision == ENZO_FP64) e = launch_sweep_fp64(a, s);
     else if (m.guess == ENZO_GUESS_MLP) e = launch_sweep_fp32_learned(a, s);
-    else if (!zones && tile != kSweepThreads) e = launch_sweep_fp32_tiled(a, s);
     else e = launch_sweep_fp32(a, s);
     note_launch();
     return e == cudaSuccess ? ENZO_OK : ENZO_ERR_CUDA;

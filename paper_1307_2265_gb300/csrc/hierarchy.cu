@@ -450,7 +450,13 @@ int enzo_ghost_fill_level(const enzo_patch_batch *fine, const enzo_patch_link *f
         a.w = w;
         a.boxes = interp_boxes;
         a.nbox = ninterp;
-        const dim3 grid = box_grid(ninterp);
+        // a face box of a 24^3 patch is 1440 items: eight CTAs, unless the boxes
+        // alone are sixteen times what the chip holds (the many edge and corner
+        // boxes leave most of their CTAs without an item, which costs less than
+        // a face's items in a row)
+        dim3 grid = box_grid((ninterp + 15) / 16);
+        grid.x = (unsigned)ninterp < (unsigned)sm_count() * 256u ? (unsigned)ninterp : (unsigned)sm_count() * 256u;
+        if (grid.y > 8) grid.y = 8;
         if (precision == ENZO_FP64) interp_ghosts_kernel<double><<<grid, 128, 0, s>>>(a);
         else interp_ghosts_kernel<float><<<grid, 128, 0, s>>>(a);
         note_launch();

@@ -136,8 +136,6 @@ __host__ __device__ inline void staged_shape(int L, int zones, int &pencils, int
 cudaError_t launch_sweep_fp64(const SweepArgs &a, cudaStream_t s);
 cudaError_t launch_sweep_fp32(const SweepArgs &a, cudaStream_t s);
 cudaError_t launch_sweep_fp32_learned(const SweepArgs &a, cudaStream_t s);
-// FP32 plain sweep with a chosen tile size (64, 128 or 256 pencils per CTA).
-cudaError_t launch_sweep_fp32_tiled(const SweepArgs &a, cudaStream_t s);
 
 // Checks and defaults of enzo_params shared by every sweep entry point
 // (ENZO_OK or an ENZO_ERR_* code).

@@ -2512,62 +2512,19 @@ cudaError_t ring_prepare(int dev)
     return e;
 }
 
-template <class R, int THREADS>
-int tiled_grid(int device)
-{
-    static int cached[64] = {0};
-    if (device < 0 || device >= 64) device = 0;
-    if (cached[device]) return cached[device];
-    int sms = 0, per = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    ring_prepare<R, 1, THREADS, false>(device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, THREADS>, THREADS,
-                                                  ring_bytes<R, THREADS, 0, 1>());
-    cached[device] = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
-    return cached[device];
-}
-
-template <class R, int THREADS>
-cudaError_t launch_tiled(const SweepArgs &a, cudaStream_t s)
-{
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const int grid = tiled_grid<R, THREADS>(dev);
-    cudaError_t e = cudaSuccess;
-    switch (a.dir) {
-    case 0:
-        e = ring_prepare<R, 0, THREADS, false>(dev);
-        if (e == cudaSuccess)
-            ppm_sweep_kernel<R, 0, false, THREADS><<<grid, THREADS, ring_bytes<R, THREADS, 0, 0>(), s>>>(a);
-        break;
-    case 1:
-        e = ring_prepare<R, 1, THREADS, false>(dev);
-        if (e == cudaSuccess)
-            ppm_sweep_kernel<R, 1, false, THREADS><<<grid, THREADS, ring_bytes<R, THREADS, 0, 1>(), s>>>(a);
-        break;
-    default:
-        e = ring_prepare<R, 2, THREADS, false>(dev);
-        if (e == cudaSuccess)
-            ppm_sweep_kernel<R, 2, false, THREADS><<<grid, THREADS, ring_bytes<R, THREADS, 0, 2>(), s>>>(a);
-        break;
-    }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-}
-
 // One sweep of a kernel family, each direction with its ring; the grid fills the
 // device at the y sweep's occupancy.
-template <class R, int DIR, bool REG, int EXT>
+template <class R, int DIR, bool REG, int EXT, int THREADS>
 cudaError_t launch_march_one(const SweepArgs &a, int dev, int grid, cudaStream_t s)
 {
-    const cudaError_t e = ring_prepare<R, DIR, kSweepThreads, REG, EXT>(dev);
+    const cudaError_t e = ring_prepare<R, DIR, THREADS, REG, EXT>(dev);
     if (e != cudaSuccess) return e;
-    ppm_sweep_kernel<R, DIR, false, kSweepThreads, REG, EXT>
-        <<<grid, kSweepThreads, ring_bytes<R, kSweepThreads, EXT, DIR>(), s>>>(a);
+    ppm_sweep_kernel<R, DIR, false, THREADS, REG, EXT>
+        <<<grid, THREADS, ring_bytes<R, THREADS, EXT, DIR>(), s>>>(a);
     return cudaGetLastError();
 }
 
-template <class R, bool REG, int EXT>
+template <class R, bool REG, int EXT, int THREADS>
 cudaError_t launch_march(const SweepArgs &a, cudaStream_t s)
 {
     static int cached[64] = {0};
@@ -2577,16 +2534,16 @@ cudaError_t launch_march(const SweepArgs &a, cudaStream_t s)
     if (!cached[dev]) {
         int sms = 0, per = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const cudaError_t e = ring_prepare<R, 1, kSweepThreads, REG, EXT>(dev);
+        const cudaError_t e = ring_prepare<R, 1, THREADS, REG, EXT>(dev);
         if (e != cudaSuccess) return e;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, kSweepThreads, REG, EXT>,
-                                                      kSweepThreads, ring_bytes<R, kSweepThreads, EXT, 1>());
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, ppm_sweep_kernel<R, 1, false, THREADS, REG, EXT>, THREADS,
+                                                      ring_bytes<R, THREADS, EXT, 1>());
         cached[dev] = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
     }
     switch (a.dir) {
-    case 0: return launch_march_one<R, 0, REG, EXT>(a, dev, cached[dev], s);
-    case 1: return launch_march_one<R, 1, REG, EXT>(a, dev, cached[dev], s);
-    default: return launch_march_one<R, 2, REG, EXT>(a, dev, cached[dev], s);
+    case 0: return launch_march_one<R, 0, REG, EXT, THREADS>(a, dev, cached[dev], s);
+    case 1: return launch_march_one<R, 1, REG, EXT, THREADS>(a, dev, cached[dev], s);
+    default: return launch_march_one<R, 2, REG, EXT, THREADS>(a, dev, cached[dev], s);
     }
 }
 
@@ -2597,10 +2554,14 @@ template <class R>
 cudaError_t launch_sweep_dir(const SweepArgs &a, cudaStream_t s)
 {
     if (a.mp.options & ENZO_OPT_DUAL)
-        return a.freg ? launch_march<R, true, 2>(a, s) : launch_march<R, false, 2>(a, s);
+        return a.freg ? launch_march<R, true, 2, kSweepThreads>(a, s) : launch_march<R, false, 2, kSweepThreads>(a, s);
     if (a.mp.options || a.mp.fallback == 2)
-        return a.freg ? launch_march<R, true, 1>(a, s) : launch_march<R, false, 1>(a, s);
-    return a.freg ? launch_march<R, true, 0>(a, s) : launch_march<R, false, 0>(a, s);
+        return a.freg ? launch_march<R, true, 1, kSweepThreads>(a, s) : launch_march<R, false, 1, kSweepThreads>(a, s);
+    switch (a.tile) {
+    case 64: return a.freg ? launch_march<R, true, 0, 64>(a, s) : launch_march<R, false, 0, 64>(a, s);
+    case 256: return launch_march<R, false, 0, 256>(a, s);
+    default: return launch_march<R, false, 0, kSweepThreads>(a, s);
+    }
 }
 
 }  // namespace enzo
