@@ -255,6 +255,13 @@ ENZO_HD bool ge0(double x) { return bits(x) <= 0x7ff0000000000000ull || bits(x) 
 ENZO_HD bool lt0(double x) { return bits(x) - 0x8000000000000001ull < 0x7ff0000000000000ull; }
 ENZO_HD bool le0(double x) { return bits(x) - 0x8000000000000000ull <= 0x7ff0000000000000ull || bits(x) == 0; }
 ENZO_HD bool is_nan(double x) { return (bits(x) << 1) > 0xffe0000000000000ull; }
+// a < b.  Magnitudes order as integers, negative ones the other way round.
+ENZO_HD bool less(double a, double b)
+{
+    const int64_t u = (int64_t)bits(a), v = (int64_t)bits(b);
+    const int64_t ku = u ^ (int64_t)((uint64_t)(u >> 63) >> 1), kv = v ^ (int64_t)((uint64_t)(v >> 63) >> 1);
+    return ku < kv && !is_nan(a) && !is_nan(b) && ((uint64_t)(u | v) << 1) != 0;
+}
 ENZO_HD bool finite(double x) { return (hi32(x) & 0x7ff00000u) != 0x7ff00000u; }
 ENZO_HD double neg_if(bool c, double x) { return from_bits(bits(x) ^ (c ? 0x8000000000000000ull : 0ull)); }
 ENZO_HD uint64_t mag(double x) { return bits(x) & 0x7fffffffffffffffull; }

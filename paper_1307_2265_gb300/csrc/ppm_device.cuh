@@ -189,8 +189,10 @@ __device__ __forceinline__ Zone<float> prim_f(double rho64, double mn64, double 
     }
     if (e < k.eta_eke * E) {
         // high-Mach cell: the internal energy is a small difference of two
-        // large numbers, so it is recovered in FP64
-        const double ke64 = 0.5 * ((mn64 * mn64 + m164 * m164) + m264 * m264) / rho64;
+        // large numbers, so it is recovered in FP64 (the division off the FP64
+        // pipe, where it took more than everything else in the sweep of a
+        // supersonic region)
+        const double ke64 = x64::div<-1>((mn64 * mn64 + m164 * m164) + m264 * m264, rho64, x64::recip(rho64));
         e = (float)(E64 - ke64);
         if (COUNT) cnt.rare(ENZO_ST_FP64_EKE);
     }
@@ -235,7 +237,7 @@ __device__ __forceinline__ Zone<double> prim_dual(double rho, double mn, double 
     const x64::Recip ir = x64::recip(rho);
     const double ke = x64::div<-1>((mn * mn + m1 * m1) + m2 * m2, rho, ir);
     double p;
-    if (E - ke < 1e-3 * E) {
+    if (x64::less(E - ke, 1e-3 * E)) {
         p = k.gm1 * ge;
         if (COUNT) cnt.gep++;
     } else {
@@ -268,8 +270,8 @@ __device__ __forceinline__ Zone<float> prim_dual(double rho64, double mn64, doub
     const float ke = 0.5f * ((mn * mn + m1 * m1) + m2 * m2) * inv;
     float e = E - ke;
     if (e < k.eta_eke * E) {
-        const double ke64 = 0.5 * ((mn64 * mn64 + m164 * m164) + m264 * m264) / rho64;
-        if (E64 - ke64 < 1e-3 * E64) {
+        const double ke64 = x64::div<-1>((mn64 * mn64 + m164 * m164) + m264 * m264, rho64, x64::recip(rho64));
+        if (x64::less(E64 - ke64, 1e-3 * E64)) {
             e = d2f_rz(ge64);
             if (COUNT) cnt.gep++;
         } else {
@@ -1509,6 +1511,7 @@ struct Marcher {
     __device__ __forceinline__ void ge_commit(double Eright)
     {
         double emax = gpend.Eleft;
+        // (FP64 compares: this kernel is short of issue slots, not of the FP64 pipe)
         if (gpend.E > emax) emax = gpend.E;
         if (Eright > emax) emax = Eright;
         const double g = gpend.ok && gpend.e > 0.1 * emax ? gpend.e : gpend.ge;
@@ -1726,7 +1729,7 @@ struct Marcher {
                 gnew = ((g0 + g_m) - g_p) - src;
             }
             double enew = 0.0;
-            const bool ok = u[0] > 0.0;
+            const bool ok = x64::gt0(u[0]);
             if (ok) {
                 if (sizeof(R) == 8) {
                     const double ke = 0.5 * ((u[1] * u[1] + u[2] * u[2]) + u[3] * u[3]) / u[0];

@@ -131,9 +131,9 @@ struct Staged {
     __device__ __forceinline__ static double resync(double g, double e, double E, double El, double Er, bool ok)
     {
         double emax = El;
-        if (E > emax) emax = E;
-        if (Er > emax) emax = Er;
-        return ok && e > 0.1 * emax ? e : g;
+        if (x64::less(emax, E)) emax = E;
+        if (x64::less(emax, Er)) emax = Er;
+        return ok && x64::less(0.1 * emax, e) ? e : g;
     }
 
     __device__ __forceinline__ void widen(const R F[5], double G[5]) const

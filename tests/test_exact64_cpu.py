@@ -77,6 +77,8 @@ int main(int argc, char **argv)
         truth("< 0", a, 0, a < 0.0, lt0(a));
         truth("<= 0", a, 0, a <= 0.0, le0(a));
         truth("nan", a, 0, a != a, is_nan(a));
+        truth("less", a, b, a < b, less(a, b));
+        truth("less", a, a, false, less(a, a));
     }
     for (double a : special)
         for (double b : special) {
@@ -84,6 +86,7 @@ int main(int argc, char **argv)
             same("div", a, b, va / vb, div(a, b));
             same("sqrt", a, 0.0, std::sqrt(va), sqrt_rn(a));
             same("div6", a, 6.0, va / 6.0, div6(a));
+            truth("less", a, b, va < vb, less(a, b));
         }
     printf("%ld differ\n", bad);
     return bad != 0;
