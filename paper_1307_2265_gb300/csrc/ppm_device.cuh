@@ -2382,11 +2382,14 @@ __global__ void __launch_bounds__(256) cfl_kernel(const __grid_constant__ CflArg
             if (patch_ok(P, a.field_len)) cells = (int64_t)P.n[0] * P.n[1] * P.n[2];
             else if (blockIdx.x == 0) atomicAdd(a.status + ENZO_ST_BAD_PATCH, 1ull);
         }
-        for (;; tcells /= 2) {
-            total = list_scan((int)((cells + tcells - 1) / tcells), s_pre);
-            if (tcells == 256 || total >= 4 * a.sms) break;
-            __syncthreads();
-        }
+        // four tiles per SM if the cells are enough for it
+        __shared__ unsigned long long s_cells;
+        if (threadIdx.x == 0) s_cells = 0ull;
+        __syncthreads();
+        if (cells) atomicAdd(&s_cells, (unsigned long long)cells);
+        __syncthreads();
+        while (tcells > 256 && s_cells < (unsigned long long)tcells * 4u * (unsigned)a.sms) tcells /= 2;
+        total = list_scan((int)((cells + tcells - 1) / tcells), s_pre);
         prefix = s_pre;
     }
     double best = 0.0;
