@@ -1,13 +1,15 @@
 // Device code of the split PPM sweep, templated on the arithmetic type.
 //
 // R = double: the FP64 path.  Its translation unit is compiled with
-// --fmad=false and IEEE division/square root, and every formula keeps the
-// association written here, so results are reproducible operation by
-// operation.
+// --fmad=false and IEEE division/square root, and every value that reaches a
+// result keeps the association written here, so results are reproducible
+// operation by operation (division, square root and comparisons run on the
+// integer pipe, exact64.cuh).  FP64 sweeps are staged (ppm_staged.cuh).
 // R = float: the FP32 path (fast reciprocal/sqrt, FMA contraction allowed);
 // conserved variables stay FP64 in memory and are updated in FP64, and the
 // internal energy E - KE is recovered in FP64 where E - KE < eta * E
-// (high-Mach cells).
+// (high-Mach cells).  FP32 sweeps march (below), or are staged where pencils
+// are few.
 //
 // Method (paper Sec. 4.1 and 4.1.2, reconstruction formulas of CW84 that the
 // paper defers to):
@@ -22,7 +24,7 @@
 //   the FP32 path, a small network evaluated on the tensor cores
 //   (LearnedGuess).
 //
-// Thread layout: one thread marches one pencil from one end to the other,
+// Thread layout of the march: one thread marches one pencil from one end to the other,
 // holding a sliding window of zones in registers: reading cell k it finishes
 // the slope of zone k-1, the interface value at (k-2)+1/2, the parabola and
 // both edge states of zone k-2, the Riemann problem at (k-3)+1/2, decides
@@ -39,20 +41,9 @@
 #include "mlp_layout.cuh"
 #include "tc05.cuh"
 
-// Cache prefetch of the march: a position's five fields are requested this
-// many steps before their load (0: off).
-#ifndef ENZO_PREFETCH_AHEAD
-#define ENZO_PREFETCH_AHEAD 2
-#endif
 #ifndef ENZO_NEWTON_HEAD
 #define ENZO_NEWTON_HEAD 3   // FP32 Newton: evaluations done as straight-line code before the loop
 #endif
-#ifdef ENZO_PREFETCH_TO_L2
-#define ENZO_PREFETCH(p) asm volatile("prefetch.global.L2 [%0];" ::"l"(p))
-#else
-#define ENZO_PREFETCH(p) asm volatile("prefetch.global.L1 [%0];" ::"l"(p))
-#endif
-
 namespace enzo {
 
 // FP32 expressions whose rounding the compiler may choose (which product of a
@@ -1028,16 +1019,11 @@ struct Pencil {
     __device__ __forceinline__ int64_t at(int s) const { return base + (int64_t)s * sd; }
 };
 
-// Face contribution to the FP64 conservative update.  FP64 path: the flux
-// itself (the update is U + dt/dx (F_m - F_p), as in the oracle).  FP32 path:
-// G = dt/dx * F rounded once in FP32 and widened exactly to FP64; a cell then
-// gets (U + G_m) - G_p in FP64, so each face's contribution enters its two
-// cells with opposite signs exactly and the totals change only by FP64 rounding.
-template <class R>
-struct Face {
-    double g[5];
-};
-
+// Conservative update.  FP64 path: U + dt/dx (F_m - F_p), as in the oracle.
+// FP32 path: G = dt/dx * F rounded once in FP32 and widened exactly to FP64; a
+// cell then gets (U + G_m) - G_p in FP64, so each face's contribution enters its
+// two cells with opposite signs exactly and the totals change only by FP64
+// rounding.
 __device__ __forceinline__ double cell_update(double U, double dtdx64, double Fm, double Fp)
 {
     return U + dtdx64 * (Fm - Fp);
@@ -1424,6 +1410,7 @@ __device__ __forceinline__ bool fails_state(const double u[5])
 // flattening, diffusive flux); 2 with those and dual energy.
 template <class R, bool WRAP, int DIR, bool REG = false, int EXT = 0>
 struct Marcher {
+    static_assert(sizeof(R) == 4, "FP64 sweeps are staged (ppm_staged.cuh)");
     static constexpr int A1 = DIR == 0 ? 1 : 0;
     static constexpr int A2 = DIR == 2 ? 1 : 2;
     const SweepArgs &a;
@@ -1433,7 +1420,6 @@ struct Marcher {
     unsigned log_key;     // pencil identity for the interface-state log
     double *reg_all;      // this pencil's all-face flux register row, or nullptr
     double *reg_bnd;      // this pencil's boundary-face register pair, or nullptr
-    double dt64;
     // WRAP: the initial state of the first three active cells (and their eps
     // with dual energy), which the trailing ghost positions reuse after the
     // pencil has updated those cells.  FP32 keeps them in shared memory (the
@@ -1464,32 +1450,17 @@ struct Marcher {
     {
         return uring[((s % SLOTS) * kRingFields + f) * (int)blockDim.x];
     }
-    Zone<R> c0, c1, c2;
-    R ce0, ce1, ce2;
-
     __device__ __forceinline__ void save(int t, const Zone<R> &z, R e)
     {
-        if constexpr (sizeof(R) == 4) {
-            float *o = wsave + t * kSave * blockDim.x;
-            const float v[7] = {z.r, z.u, z.p, z.t1, z.t2, z.c, e};
-            _Pragma("unroll") for (int i = 0; i < kSave; ++i) o[i * blockDim.x] = v[i];
-        } else {
-            if (t == 0) { c0 = z; ce0 = e; }
-            else if (t == 1) { c1 = z; ce1 = e; }
-            else { c2 = z; ce2 = e; }
-        }
+        float *o = wsave + t * kSave * blockDim.x;
+        const float v[7] = {z.r, z.u, z.p, z.t1, z.t2, z.c, e};
+        _Pragma("unroll") for (int i = 0; i < kSave; ++i) o[i * blockDim.x] = v[i];
     }
     __device__ __forceinline__ Zone<R> saved(int t, R &e) const
     {
-        if constexpr (sizeof(R) == 4) {
-            const float *o = wsave + t * kSave * blockDim.x;
-            e = EXT == 2 ? o[6 * blockDim.x] : 0.0f;
-            return Zone<R>{o[0], o[blockDim.x], o[2 * blockDim.x], o[3 * blockDim.x], o[4 * blockDim.x],
-                           o[5 * blockDim.x]};
-        } else {
-            e = t == 0 ? ce0 : (t == 1 ? ce1 : ce2);
-            return t == 0 ? c0 : (t == 1 ? c1 : c2);
-        }
+        const float *o = wsave + t * kSave * blockDim.x;
+        e = EXT == 2 ? o[6 * blockDim.x] : 0.0f;
+        return Zone<R>{o[0], o[blockDim.x], o[2 * blockDim.x], o[3 * blockDim.x], o[4 * blockDim.x], o[5 * blockDim.x]};
     }
 
     // Dual energy: gas-energy flux and interface velocity of one face.
@@ -1530,23 +1501,6 @@ struct Marcher {
             return pc.at(pc.ng + (j < 0 ? (pc.n - ((-j) % pc.n)) % pc.n : j));
         }
         return pc.at(s);
-    }
-
-    // Ask the memory system for the five fields of pencil position s ahead of
-    // their load (a cache prefetch: no registers are held), so that the load
-    // a few march steps later hits the cache instead of waiting for HBM.
-    __device__ __forceinline__ void warm(int s) const
-    {
-        // x pencils walk their own rows, which the cache lines they already
-        // loaded cover 16 positions at a time
-        if (ENZO_PREFETCH_AHEAD == 0 || DIR == 0 || s >= pc.L) return;
-        const int64_t idx = index_of(s);
-        if (idx < 0) return;
-        ENZO_PREFETCH(a.U[0] + idx);
-        ENZO_PREFETCH(a.U[1] + idx);
-        ENZO_PREFETCH(a.U[2] + idx);
-        ENZO_PREFETCH(a.U[3] + idx);
-        ENZO_PREFETCH(a.U[4] + idx);
     }
 
     // Start the asynchronous copy of pencil position s's five raw values into
@@ -1681,8 +1635,7 @@ struct Marcher {
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
         {
             const double U = RING ? ring(s, v) : a.U[map[v]][idx];
-            if (sizeof(R) == 8) u[v] = cell_update(U, dtdx64, (double)Fm[v], (double)Fp[v]);
-            else u[v] = (U + f2d_exact((float)(dtdx * Fm[v]))) - f2d_exact((float)(dtdx * Fp[v]));
+            u[v] = (U + f2d_exact((float)(dtdx * Fm[v]))) - f2d_exact((float)(dtdx * Fp[v]));
         }
         return fails_state(u);
     }
@@ -1712,35 +1665,23 @@ struct Marcher {
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
         {
             const double U = RING ? ring(s, v) : ld_march<DIR>(a.U[map[v]] + idx);
-            if (sizeof(R) == 8) u[v] = cell_update(U, dtdx64, (double)Fm[v], (double)Fp[v]);
-            else u[v] = (U + Gm[v]) - Gp[v];
+            u[v] = (U + Gm[v]) - Gp[v];
         }
         double gnew = 0.0;
         const bool dual = EXT == 2 && gm != nullptr;
         if (dual) {
             const double g0 = RING ? ring(s, 5) : a.ge[idx];
-            if (sizeof(R) == 8) {
-                gnew = (g0 + dtdx64 * ((double)gm->F - (double)gp->F)) -
-                       dtdx64 * (double)pz * ((double)gp->uf - (double)gm->uf);
-            } else {
-                const double g_m = f2d_exact((float)(dtdx * gm->F));
-                const double g_p = f2d_exact((float)(dtdx * gp->F));
-                const double src = f2d_exact((float)(dtdx * pz * (gp->uf - gm->uf)));
-                gnew = ((g0 + g_m) - g_p) - src;
-            }
+            const double g_m = f2d_exact((float)(dtdx * gm->F));
+            const double g_p = f2d_exact((float)(dtdx * gp->F));
+            const double src = f2d_exact((float)(dtdx * pz * (gp->uf - gm->uf)));
+            gnew = ((g0 + g_m) - g_p) - src;
             double enew = 0.0;
             const bool ok = x64::gt0(u[0]);
             if (ok) {
-                if (sizeof(R) == 8) {
-                    const double ke = 0.5 * ((u[1] * u[1] + u[2] * u[2]) + u[3] * u[3]) / u[0];
-                    enew = u[4] - ke;
-                } else {
-                    // FP32 path: KE in FP32 off the FP64 pipe; E - KE is only
-                    // taken where it exceeds 0.1 E, so its error stays below
-                    // 1e-6 of it
-                    const float r = d2f_rz(u[0]), m0 = d2f_rz(u[1]), m1 = d2f_rz(u[2]), m2 = d2f_rz(u[3]);
-                    enew = u[4] - f2d_exact((R)0.5 * ((m0 * m0 + m1 * m1) + m2 * m2) / r);
-                }
+                // KE in FP32 off the FP64 pipe; E - KE is only taken where it
+                // exceeds 0.1 E, so its error stays below 1e-6 of it
+                const float r = d2f_rz(u[0]), m0 = d2f_rz(u[1]), m1 = d2f_rz(u[2]), m2 = d2f_rz(u[3]);
+                enew = u[4] - f2d_exact((R)0.5 * ((m0 * m0 + m1 * m1) + m2 * m2) / r);
             }
             if (gpend.idx >= 0) {
                 ge_commit(u[4]);
@@ -1760,9 +1701,7 @@ struct Marcher {
 
     __device__ __forceinline__ void widen(const R Fv[5], R dtdx, double G[5]) const
     {
-        if (sizeof(R) == 4) {
-            _Pragma("unroll") for (int v = 0; v < 5; ++v) G[v] = f2d_exact((float)(dtdx * Fv[v]));
-        }
+        _Pragma("unroll") for (int v = 0; v < 5; ++v) G[v] = f2d_exact((float)(dtdx * Fv[v]));
     }
 
     __device__ __forceinline__ void log_states(int kk, const R sl[5], const R sr[5])
@@ -1777,25 +1716,24 @@ struct Marcher {
     }
 
     // Flux register entries of face f (left of active cell f; f = n is the
-    // right face of the last cell) once its final flux is known.  FP64 path:
-    // the flux F (all faces) and dt F summed over steps (boundary faces).  FP32
-    // path: the increment G = dt/dx F exactly as the cells applied it, and its
-    // sum, so a flux correction cancels the applied coarse increment exactly.
-    // With dual energy (EXT == 2) a face has a sixth entry, the gas-energy
-    // flux gF (FP32 path: its applied increment gG); the -p div v source is a
-    // zone term and has none.
+    // right face of the last cell) once its final flux is known: the increment
+    // G = dt/dx F exactly as the cells applied it (all faces), and its sum over
+    // steps (boundary faces), so a flux correction cancels the applied coarse
+    // increment exactly.  With dual energy (EXT == 2) a face has a sixth entry,
+    // the gas energy's applied increment gG; the -p div v source is a zone term
+    // and has none.
     static constexpr int NC = EXT == 2 ? 6 : 5;
-    __device__ __forceinline__ void record(int f, const R Fv[5], const double G[5], R gF = (R)0, double gG = 0.0)
+    __device__ __forceinline__ void record(int f, const double G[5], double gG = 0.0)
     {
         if (!REG) return;
         if (reg_all) {
-            _Pragma("unroll") for (int v = 0; v < 5; ++v) reg_all[f * NC + v] = sizeof(R) == 8 ? (double)Fv[v] : G[v];
-            if constexpr (EXT == 2) reg_all[f * NC + 5] = sizeof(R) == 8 ? (double)gF : gG;
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) reg_all[f * NC + v] = G[v];
+            if constexpr (EXT == 2) reg_all[f * NC + 5] = gG;
         }
         if (reg_bnd && (f == 0 || f == pc.n)) {
             double *o = reg_bnd + (f == 0 ? 0 : NC);
-            _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = o[v] + (sizeof(R) == 8 ? dt64 * (double)Fv[v] : G[v]);
-            if constexpr (EXT == 2) o[5] = o[5] + (sizeof(R) == 8 ? dt64 * (double)gF : gG);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = o[v] + G[v];
+            if constexpr (EXT == 2) o[5] = o[5] + gG;
         }
     }
 
@@ -1804,7 +1742,7 @@ struct Marcher {
     template <class GS>
     __device__ void run(R dtdx, double dtdx64, const MethodParams &mp, Counters &cnt, GS &guess)
     {
-        constexpr bool RING = sizeof(R) == 4;   // the shared-memory ring of raw values
+        constexpr bool RING = true;             // the shared-memory ring of raw values
         const int L = pc.L;
         const bool fb = mp.fallback != 0;
         Zone<R> zm2, zm1, z0;                 // zones k-2, k-1, k
@@ -1839,7 +1777,7 @@ struct Marcher {
             gpend.Eleft = a.U[4][WRAP ? pc.at(pc.ng + pc.n - 1) : pc.at(pc.ng - 1)];
             Eghost_right = a.U[4][WRAP ? pc.at(pc.ng) : pc.at(pc.ng + pc.n)];
         }
-        if constexpr (RING && DIR != 0)
+        if constexpr (DIR != 0)
             for (int q = 0; q < kStage; ++q) stage(q);
         for (int kk = 0; kk < L; ++kk) {
             if constexpr (EXT) {
@@ -1852,7 +1790,7 @@ struct Marcher {
             }
             zm2 = zm1;
             zm1 = z0;
-            if constexpr (RING && EXT == 2) {
+            if constexpr (EXT == 2) {
                 if constexpr (DIR != 0) {
                     stage(kk + kStage);
                     z0 = zone_staged_dual(kk, cnt, e0);
@@ -1860,26 +1798,21 @@ struct Marcher {
                     z0 = zone_keep_dual(kk, cnt, e0);
                 }
             } else {
-                if constexpr (RING && DIR != 0) {
+                if constexpr (DIR != 0) {
                     stage(kk + kStage);
                     z0 = zone_staged(kk, cnt);
-                } else if constexpr (RING) {
-                    z0 = zone_keep(kk, cnt);
                 } else {
-                    warm(kk + ENZO_PREFETCH_AHEAD);
-                    z0 = zone<true>(kk, cnt);
+                    z0 = zone_keep(kk, cnt);
                 }
             }
             if (WRAP) {
                 const int j = kk - pc.ng;
                 if (j >= 0 && j < 3) save(j, z0, e0);
             }
-            if (sizeof(R) == 4) {
-                rho3 = rho2;
-                rho2 = rho1;
-                rho1 = rho0;
-                rho0 = z0.r;
-            }
+            rho3 = rho2;
+            rho2 = rho1;
+            rho1 = rho0;
+            rho0 = z0.r;
             if (kk < 2) continue;
             R dcur[5];
             _Pragma("unroll") for (int v = 0; v < 5; ++v) dcur[v] = limited_slope<R>(zv(zm2, v), zv(zm1, v), zv(z0, v));
@@ -1954,10 +1887,8 @@ struct Marcher {
                                     // margins; only unclear cells take the exact FP64 test
                                     // (always with dual energy: the zone pressure may come
                                     // from the gas energy, not from E)
-                                    bad = (sizeof(R) == 8 || dual || !clearly_ok<R>(k, zm3, Fgprev, Fg, dtdx))
+                                    bad = (dual || !clearly_ok<R>(k, zm3, Fgprev, Fg, dtdx))
                                               ? fails_full<RING>(c, Fgprev, Fg, dtdx, dtdx64) : false;
-                                } else if (sizeof(R) == 8) {
-                                    bad = !x64::gt0(cell_update(rho_old<RING>(c), dtdx64, (double)Fgprev[0], (double)Fg[0]));
                                 } else {
                                     // FP32 screen; cells near zero are decided in FP64
                                     const R rt = rho3 + dtdx * (Fgprev[0] - Fg[0]);
@@ -1979,8 +1910,8 @@ struct Marcher {
                             double G1[5];
                             widen(Fu1, dtdx, G1);
                             if constexpr (REG && EXT == 2)
-                                record(kk - 6, Fu1, G1, gfin.F, sizeof(R) == 4 ? f2d_exact((float)(dtdx * gfin.F)) : 0.0);
-                            else record(kk - 6, Fu1, G1);
+                                record(kk - 6, G1, f2d_exact((float)(dtdx * gfin.F)));
+                            else record(kk - 6, G1);
                             if (kk >= 7)
                                 update<RING>(kk - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt,
                                              dual ? &gfin2 : nullptr, &gfin, p4, dtdx);
@@ -2015,8 +1946,8 @@ struct Marcher {
         double G1[5];
         widen(Fu1, dtdx, G1);
         if constexpr (REG && EXT == 2)
-            record(pc.n, Fu1, G1, gfin.F, sizeof(R) == 4 ? f2d_exact((float)(dtdx * gfin.F)) : 0.0);
-        else record(pc.n, Fu1, G1);
+            record(pc.n, G1, f2d_exact((float)(dtdx * gfin.F)));
+        else record(pc.n, G1);
         // the pressure of zone L-4 is the last window's zone k-3
         update<RING>(L - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt, dual ? &gfin2 : nullptr, &gfin, zm3.p, dtdx);
         if (dual) ge_commit(Eghost_right);
@@ -2088,7 +2019,6 @@ struct Marcher {
                     stage<kLearnedSlots>(kk + kLearnedSlots - 1);
                     z0 = zone_staged<kLearnedSlots, kLearnedSlots - 1>(kk, cnt);
                 } else {
-                    warm(kk + ENZO_PREFETCH_AHEAD);
                     z0 = zone<true>(kk, cnt);
                 }
                 if (WRAP) {
@@ -2096,10 +2026,8 @@ struct Marcher {
                     if (j >= 0 && j < 3) save(j, z0, (R)0);
                 }
             }
-            if (sizeof(R) == 4) {
-                _Pragma("unroll") for (int i = 5; i > 0; --i) rh[i] = rh[i - 1];
-                rh[0] = kk < L ? z0.r : (R)0;
-            }
+            _Pragma("unroll") for (int i = 5; i > 0; --i) rh[i] = rh[i - 1];
+            rh[0] = kk < L ? z0.r : (R)0;
             if (kk < L && kk >= 2) {
                 R dcur[5];
                 _Pragma("unroll") for (int v = 0; v < 5; ++v) dcur[v] = limited_slope<R>(zv(zm2, v), zv(zm1, v), zv(z0, v));
@@ -2168,17 +2096,13 @@ struct Marcher {
                 const int c = jj - 3;
                 bool bad = false;
                 if (fb) {
-                    if (sizeof(R) == 8) {
-                        bad = !(cell_update(rho_old(c), dtdx64, (double)Fgprev[0], (double)Fg[0]) > 0.0);
-                    } else {
-                        // FP32 screen; cells near zero are decided in FP64
-                        const R rc = rh[3 + D];
-                        const R rt = rc + dtdx * (Fgprev[0] - Fg[0]);
-                        if (!(rt > (R)1e-3 * rc)) {
-                            const double g0 = f2d_exact((float)(dtdx * Fgprev[0]));
-                            const double g1 = f2d_exact((float)(dtdx * Fg[0]));
-                            bad = !((rho_old(c) + g0) - g1 > 0.0);
-                        }
+                    // FP32 screen; cells near zero are decided in FP64
+                    const R rc = rh[3 + D];
+                    const R rt = rc + dtdx * (Fgprev[0] - Fg[0]);
+                    if (!(rt > (R)1e-3 * rc)) {
+                        const double g0 = f2d_exact((float)(dtdx * Fgprev[0]));
+                        const double g1 = f2d_exact((float)(dtdx * Fg[0]));
+                        bad = !((rho_old(c) + g0) - g1 > 0.0);
                     }
                     if (bad && active) cnt.rare(ENZO_ST_HLL_CELLS);
                 }
@@ -2194,7 +2118,7 @@ struct Marcher {
                 }
                 double G1[5];
                 widen(Fu1, dtdx, G1);
-                record(jj - 6, Fu1, G1);
+                record(jj - 6, G1);
                 if (jj >= 7) update(jj - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt);
                 _Pragma("unroll") for (int v = 0; v < 5; ++v)
                 {
@@ -2217,7 +2141,7 @@ struct Marcher {
         }
         double G1[5];
         widen(Fu1, dtdx, G1);
-        record(pc.n, Fu1, G1);
+        record(pc.n, G1);
         update(L - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt);
     }
 };
@@ -2236,7 +2160,7 @@ __device__ __forceinline__ void warp_flush(unsigned long long *status, unsigned 
 template <class R, int THREADS, int EXT, int DIR>
 __host__ __device__ constexpr int ring_bytes()
 {
-    return sizeof(R) == 4 ? (DIR == 0 ? 5 : 8) * (EXT == 2 ? 6 : 5) * THREADS * (int)sizeof(double) : 0;
+    return (DIR == 0 ? 5 : 8) * (EXT == 2 ? 6 : 5) * THREADS * (int)sizeof(double);
 }
 
 // Learned kernels: the network's shared memory (aligned to 128 bytes inside
@@ -2265,13 +2189,13 @@ __host__ __device__ constexpr size_t learned_smem_bytes()
 // REG: the batch has flux registers (hierarchy levels); the per-pencil register
 // rows are then tracked, otherwise the recording compiles away.
 template <class R, int DIR, bool LEARNED, int THREADS = kSweepThreads, bool REG = false, int EXT = 0>
-__global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (sizeof(R) == 4 ? (EXT == 2 ? ENZO_SWEEP_MIN_BLOCKS_DUAL : ENZO_SWEEP_MIN_BLOCKS_FP32 * 128 / THREADS) : 2))
+__global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (EXT == 2 ? ENZO_SWEEP_MIN_BLOCKS_DUAL : ENZO_SWEEP_MIN_BLOCKS_FP32 * 128 / THREADS))
     ppm_sweep_kernel(const __grid_constant__ SweepArgs a)
 {
     constexpr int A1 = DIR == 0 ? 1 : 0, A2 = DIR == 2 ? 1 : 2;
     __shared__ int s_tile;
     // FP32: per-thread slots for the wrapped pencils' first three cells
-    __shared__ float s_wrap[sizeof(R) == 4 ? 3 * (EXT == 2 ? 7 : 6) * THREADS : 1];
+    __shared__ float s_wrap[3 * (EXT == 2 ? 7 : 6) * THREADS];
     extern __shared__ __align__(16) unsigned char dsmem[];
     // plain FP32 default kernels: the ring of raw values in dynamic shared memory
     double *uring = nullptr;
@@ -2336,11 +2260,11 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (sizeof
         // a stand-in row counts none of its rare events (floors, FP64 E - KE)
         cnt.st = valid ? a.status : nullptr;
         if (P.flags & ENZO_PATCH_PERIODIC) {
-            Marcher<R, true, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, dt, s_wrap + threadIdx.x, uring};
+            Marcher<R, true, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, s_wrap + threadIdx.x, uring};
             if constexpr (LEARNED) m.run_piped(dtdx, dtdx64, a.mp, cnt, guess);
             else m.run(dtdx, dtdx64, a.mp, cnt, guess);
         } else {
-            Marcher<R, false, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, dt, s_wrap + threadIdx.x, uring};
+            Marcher<R, false, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, s_wrap + threadIdx.x, uring};
             if constexpr (LEARNED) m.run_piped(dtdx, dtdx64, a.mp, cnt, guess);
             else m.run(dtdx, dtdx64, a.mp, cnt, guess);
         }
