@@ -96,10 +96,11 @@ __host__ __device__ inline bool patch_ok(const enzo_patch &P, int64_t field_len)
 }
 
 // Staged sweep (ppm_staged.cuh): zones, and threads, per CTA tile.  FP64: 256
-// zones, two CTAs per SM (128 registers): a 400-patch level step took 84 ms
+// zones, two CTAs per SM (128 registers): a 400-patch level step takes 84 ms
 // against 89 (192 zones), 99 (128 zones, four CTAs) and 85 (512 zones, one).
-// FP32: 256 zones, three CTAs per SM (80 registers): a 32^3 step took 102 us
-// against 108 (four CTAs, 64 registers), 104 and 115 (512 zones, one and two).
+// FP32: 256 zones, three CTAs per SM (80 registers): when first built a 32^3 step
+// took 102 us (76 now) against 108 (four CTAs, 64 registers), 104 and 115 (512
+// zones, one and two).
 constexpr int kStagedZones64 = 256, kStagedZones32 = 256;
 constexpr int kStagedMaxPencils = 8;   // windowed pencils per tile
 

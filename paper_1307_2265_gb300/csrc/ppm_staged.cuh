@@ -12,14 +12,14 @@
 // value is formed by the same functions as in the march, so results agree bit
 // for bit (FP32 through the functions' PIN forms).
 //
-// Measured, a step against the march: FP64, where the pipe is the bound, 82%
-// busy instead of 49% (the march's warps wait for instructions): 400 patches
-// (2e7 cells) 142 -> 85 ms, a walled 100x75x50 grid 10.0 -> 1.59 ms, a 32^3
-// grid 4.2 -> 0.32 ms.  FP32, for batches of few pencils only (a march that
-// fills the chip issues 35% fewer instructions per cell): a 32^3 grid 324 ->
-// 104 us, 96^3 890 -> 323 us.  (Dealing items by a reciprocal instead of integer
-// divisions took another 2% off: the 400-patch level 84.4 ms, a walled
-// 240x125x61 FP32 grid with options 754 us.)
+// Measured, a step against the march with the same arithmetic: FP64, where the
+// pipe is the bound, 82% busy instead of 49% (the march's warps wait for
+// instructions): 400 patches (2e7 cells) 142 -> 84 ms, a walled 100x75x50 grid
+// 10.0 -> 1.55 ms, a 32^3 grid 4.2 -> 0.20 ms.  FP32, for batches of few pencils
+// only (a march that fills the chip issues 35% fewer instructions per cell): a
+// 32^3 grid 324 -> 76 us, a walled 240x125x61 grid with the reconstruction options
+// 1730 -> 754 us.  (Dealing items by a reciprocal instead of integer divisions is
+// 2% of that.)
 //
 // A pencil longer than the tile goes in windows of W positions.  A window
 // updates cells [lo, hi), reads the four positions on either side (the
