@@ -831,10 +831,11 @@ __device__ __forceinline__ RiemannOut<double> riemann_exact(double rl, double ul
     // comfortable range
     double tlo, thi;
     {
-        const float us = (fabsf(d2f_rz(ul)) + fabsf(d2f_rz(ur))) +
-                         (sqrtf(d2f_rz(gpl) / d2f_rz(rl)) + sqrtf(d2f_rz(gpr) / d2f_rz(rr)));
+        const float a = d2f_rz(gpl), b = d2f_rz(rl), c = d2f_rz(gpr), d = d2f_rz(rr);
+        const float us = (fabsf(d2f_rz(ul)) + fabsf(d2f_rz(ur))) + (sqrtf(a / b) + sqrtf(c / d));
         const float t = us * d2f_rz(k.tol);
-        const bool ok = us > 1e-12f && us < 1e30f && t > 1e-30f;
+        const float lo = fminf(fminf(a, b), fminf(c, d)), hi = fmaxf(fmaxf(a, b), fmaxf(c, d));
+        const bool ok = lo > 1e-36f && hi < 1e37f && us > 1e-12f && us < 1e30f && t > 1e-30f;
         tlo = ok ? f2d_exact(t * 0.9999f) : 0.0;
         thi = ok ? f2d_exact(t * 1.0001f) : __longlong_as_double(0x7ff0000000000000ll);
     }

@@ -99,3 +99,22 @@ def test_fp64_dual_equals_oracle(name, mach, flags):
         for g, o in zip(G, O):
             assert np.array_equal(active(g), active(o))
         assert np.array_equal(active(b.patch_ge(i).cpu().numpy()), active(ges[i]))
+
+
+@pytest.mark.parametrize("left", [(1.0, 1.0), (1e-37, 1e-41), (1e39, 1e38), (1e-60, 1e-30)])
+@pytest.mark.parametrize("right", [(1.0, 1.0), (1e-37, 1e-41), (1e-45, 1e-45), (1e60, 1e20)])
+def test_riemann_fp64_beyond_the_range_of_fp32(left, right):
+    """Newton's stopping bound is first formed in FP32: states outside FP32's
+    range (density and pressure scaled per side) take the FP64 bound."""
+    import torch
+    rng = np.random.default_rng(21)
+    rl, ul, pl, rr, ur, pr = (rng.uniform(0.5, 2.0, 512) for _ in range(6))
+    rl, pl, rr, pr = rl * left[0], pl * left[1], rr * right[0], pr * right[1]
+    ul = (ul - 1.25) * np.sqrt(left[1] / left[0])
+    ur = (ur - 1.25) * np.sqrt(right[1] / right[0])
+    kw = dict(rho_floor=1e-300, p_floor=1e-300)
+    o = oracle.riemann(rl, ul, pl, rr, ur, pr, oracle.Params(**kw))
+    g = ez.riemann_solve(*[torch.from_numpy(a).cuda() for a in (rl, ul, pl, rr, ur, pr)],
+                         ez.Params(precision=ez.FP64, **kw))
+    for k in ("pstar", "ustar", "rho", "u", "p", "iters"):
+        assert np.array_equal(g[k].cpu().numpy(), o[k], equal_nan=k != "iters"), k
