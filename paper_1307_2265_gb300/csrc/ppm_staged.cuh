@@ -106,28 +106,6 @@ struct Staged {
         return Zone<R>{S.q[0][z], S.q[1][z], S.q[2][z], S.q[3][z], S.q[4][z], S.q[5][z]};
     }
 
-    // Final flux of the face right of slot z: the Godunov flux, or HLL from the
-    // zone states beside a cell that failed (Sec. 4.1.2); with dual energy its
-    // gas-energy flux and interface velocity (HLL: the mass flux times the
-    // upwind eps, the mean zone velocity).
-    __device__ __forceinline__ void final_flux(int z, bool hll, R F[5], R &gF, R &uf) const
-    {
-        if (hll) {
-            const Zone<R> l = zone(z), r = zone(z + next());
-            hll_flux<R>(l, r, k, F);
-            if constexpr (dual) {
-                gF = F[0] * (F[0] >= (R)0 ? S.q[6][z] : S.q[6][z + next()]);
-                uf = (R)0.5 * (l.u + r.u);
-            }
-        } else {
-            _Pragma("unroll") for (int v = 0; v < 5; ++v) F[v] = S.B[v][z];
-            if constexpr (dual) {
-                gF = S.B[5][z];
-                uf = S.uf[z];
-            }
-        }
-    }
-
     __device__ __forceinline__ double widen1(R F) const
     {
         return sizeof(R) == 8 ? (double)F : f2d_exact((float)(dtdx * F));
@@ -369,8 +347,8 @@ struct Staged {
         // does the Godunov update leave rho > 0?  Cells [lo - 1, hi] of the
         // pencil's active ones (the neighbours' answers decide shared faces)
         const bool fb = a.mp.fallback != 0;
-        bool any = false;
         if (fb) {
+            bool any = false;
             const int c0 = first ? lo : lo - 1, c1 = last ? hi : hi + 1;
             deal(t, c1 - c0, p, j);
             if (p < np && j < c1 - c0) {
@@ -406,7 +384,27 @@ struct Staged {
                 S.bad[z] = bad;
                 any = bad;
             }
-            any = __syncthreads_or(any) != 0;
+            if (__syncthreads_or(any)) {
+                // a face beside a failing cell takes HLL from the zone states
+                // (Sec. 4.1.2), its gas-energy flux the mass flux times the upwind
+                // eps, its interface velocity the mean zone velocity; formed here
+                // once, for both of its cells and the flux register
+                deal(t, hi - lo + 1, p, j);
+                if (p < np && j < hi - lo + 1) {
+                    const int s = lo - 1 + j, z = slot(p, s - w0);
+                    if ((s >= ng && S.bad[z]) || (s + 1 < L - ng && S.bad[z + e])) {
+                        const Zone<R> l = zone(z), r = zone(z + e);
+                        R F[5];
+                        hll_flux<R>(l, r, k, F);
+                        _Pragma("unroll") for (int v = 0; v < 5; ++v) S.B[v][z] = F[v];
+                        if constexpr (dual) {
+                            S.B[5][z] = F[0] * (F[0] >= (R)0 ? S.q[6][z] : S.q[6][z + e]);
+                            S.uf[z] = (R)0.5 * (l.u + r.u);
+                        }
+                    }
+                }
+                __syncthreads();
+            }
         }
         // update of cells [lo, hi)
         deal(t, hi - lo, p, j);
@@ -416,16 +414,19 @@ struct Staged {
         double u[5], gnew = 0.0, enew = 0.0;
         bool ok = false;
         if (mine) {
-            bool hm = false, hp = false;
-            if (any) {
-                const bool b0 = S.bad[z];
-                hm = b0 || (s > ng && S.bad[z - e]);
-                hp = b0 || (s < L - ng - 1 && S.bad[z + e]);
-            }
             R Fm[5], Fp[5], gm = (R)0, gp = (R)0, um = (R)0, up = (R)0;
             double Gm[5], Gp[5];
-            final_flux(z - e, hm, Fm, gm, um);
-            final_flux(z, hp, Fp, gp, up);
+            _Pragma("unroll") for (int v = 0; v < 5; ++v)
+            {
+                Fm[v] = S.B[v][z - e];
+                Fp[v] = S.B[v][z];
+            }
+            if constexpr (dual) {
+                gm = S.B[5][z - e];
+                gp = S.B[5][z];
+                um = S.uf[z - e];
+                up = S.uf[z];
+            }
             _Pragma("unroll") for (int v = 0; v < 5; ++v)
             {
                 Gm[v] = widen1(Fm[v]);
