@@ -919,12 +919,28 @@ __device__ __forceinline__ RiemannOut<R> riemann(R rl, R ul, R pl, R rr, R ur, R
     else return riemann_exact(rl, ul, pl, rr, ur, pr, pguess, k, cnt);
 }
 
+// Total energy density of a primitive state, FP32 with its roundings stated.
+__device__ __forceinline__ float total_energy(float rho, float u, float p, float t1, float t2, const Consts<float> &k)
+{
+    const float X = __fmaf_rn(t2, t2, mad2<0>(u, u, t1, t1));
+    return __fmaf_rn(p, k.gm1inv, __fmul_rn(__fmul_rn(0.5f, rho), X));
+}
+
 // Physical flux of the split 1-D equations (Sec. 4.1): mass, normal momentum,
 // transverse momenta, total energy.
 // (FP64: the half is exact, so one fused operation adds the kinetic energy.)
 template <class R, bool PIN = false>
 __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Consts<R> &k, R F[5])
 {
+    if constexpr (PIN && sizeof(R) == 4) {
+        const float m = __fmul_rn(rho, u);
+        F[0] = m;
+        F[1] = __fmaf_rn(m, u, p);
+        F[2] = __fmul_rn(m, t1);
+        F[3] = __fmul_rn(m, t2);
+        F[4] = __fmul_rn(u, __fadd_rn(total_energy(rho, u, p, t1, t2, k), p));
+        return;
+    }
     const R mflux = rho * u;
     F[0] = mflux;
     F[1] = mflux * u + p;
@@ -932,9 +948,6 @@ __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Con
     F[3] = mflux * t2;
     if constexpr (sizeof(R) == 8) {
         F[4] = u * (__fma_rn(0.5, rho * ((u * u + t1 * t1) + t2 * t2), p * k.gm1inv) + p);
-    } else if constexpr (PIN) {
-        const float X = __fmaf_rn(t2, t2, mad2<0>(u, u, t1, t1));
-        F[4] = __fmul_rn(u, __fadd_rn(__fmaf_rn(p, k.gm1inv, __fmul_rn(__fmul_rn(0.5f, rho), X)), p));
     } else {
         const R eint = p * k.gm1inv;
         const R ke = (R)0.5 * rho * ((u * u + t1 * t1) + t2 * t2);
@@ -943,6 +956,9 @@ __device__ __forceinline__ void phys_flux(R rho, R u, R p, R t1, R t2, const Con
 }
 
 // HLL flux with Davis wave-speed bounds from first-order zone states (fallback).
+// FP32: every rounding is stated, so that all kernels form the same flux (left
+// to the compiler, the march over ghosted pencils rounded E another way than the
+// other two).
 template <class R>
 __device__ __forceinline__ void hll_flux(const Zone<R> &L, const Zone<R> &Rz, const Consts<R> &k,
                                          R F[5])
@@ -951,14 +967,23 @@ __device__ __forceinline__ void hll_flux(const Zone<R> &L, const Zone<R> &Rz, co
     const R SL = L.u - cl < Rz.u - cr ? L.u - cl : Rz.u - cr;
     const R SR = L.u + cl > Rz.u + cr ? L.u + cl : Rz.u + cr;
     R FL[5], FR[5];
-    phys_flux(L.r, L.u, L.p, L.t1, L.t2, k, FL);
-    phys_flux(Rz.r, Rz.u, Rz.p, Rz.t1, Rz.t2, k, FR);
+    phys_flux<R, true>(L.r, L.u, L.p, L.t1, L.t2, k, FL);
+    phys_flux<R, true>(Rz.r, Rz.u, Rz.p, Rz.t1, Rz.t2, k, FR);
     if (SL >= (R)0) {
         _Pragma("unroll") for (int c = 0; c < 5; ++c) F[c] = FL[c];
         return;
     }
     if (SR <= (R)0) {
         _Pragma("unroll") for (int c = 0; c < 5; ++c) F[c] = FR[c];
+        return;
+    }
+    if constexpr (sizeof(R) == 4) {
+        const float EL = total_energy(L.r, L.u, L.p, L.t1, L.t2, k), ER = total_energy(Rz.r, Rz.u, Rz.p, Rz.t1, Rz.t2, k);
+        const float d[5] = {__fsub_rn(Rz.r, L.r), __fsub_rn(FR[0], FL[0]), mad2<0>(Rz.r, Rz.t1, -L.r, L.t1),
+                            mad2<0>(Rz.r, Rz.t2, -L.r, L.t2), __fsub_rn(ER, EL)};
+        const float SS = __fmul_rn(SL, SR), inv = rcp_approx(__fsub_rn(SR, SL));
+        _Pragma("unroll") for (int c = 0; c < 5; ++c)
+            F[c] = __fmul_rn(__fmaf_rn(SS, d[c], mad2<0>(SR, FL[c], -SL, FR[c])), inv);
         return;
     }
     const R UL[5] = {L.r, L.r * L.u, L.r * L.t1, L.r * L.t2,

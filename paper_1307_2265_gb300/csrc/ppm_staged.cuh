@@ -10,7 +10,8 @@
 // memory, and its zones, faces or cells are dealt out to consecutive threads,
 // so no lane of a warp idles in a ghost zone where ghosts have no part.  Every
 // value is formed by the same functions as in the march, so results agree bit
-// for bit (FP32 through the functions' PIN forms).
+// for bit (FP32 through the functions' stated roundings; the HLLC flux's are the
+// compiler's, the same in both kernels as far as the tests compare them).
 //
 // Measured, a step against the march with the same arithmetic: FP64, where the
 // pipe is the bound, 82% busy instead of 49% (the march's warps wait for
