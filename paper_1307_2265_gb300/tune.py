@@ -1,20 +1,24 @@
 """Autotuner of the sweep's tile shape, and CUDA-graph capture of a step.
 
-The FP32 plain-guess sweep can run 64, 128 or 256 pencils per CTA tile
-(enzo_params.tile per axis).  The best choice depends on the batch: patch
-sizes set how many pencils each patch has and how full its last tile is.
+enzo_params.tile names, per axis, the pencils per CTA tile of the FP32
+plain-guess march: 64, 128 or 256.  0 leaves tile and kernel to the library,
+which is the only way to its staged sweep for batches of few pencils; with the
+reconstruction options, fallback mode 2 or flux registers a named tile's size is
+not used, only the march it asks for.  The best choice depends on the batch:
+patch sizes set how many pencils each patch has and how full its last tile is.
 `autotune_tiles` times each candidate on the batch itself, one sweep per
 candidate and direction with CUDA events, and restores the fields afterwards.
 
 `capture_steps` records one level step (device CFL + three sweeps, reading dt
 on the device) for each sweep order into CUDA graphs, so a run replays one
-graph per step instead of launching nine kernels.
+graph per step instead of launching each kernel.
 """
 from __future__ import annotations
 
 from . import Params, PatchBatch, ppm_sweep_dev, timestep_cfl
 
-CANDIDATES = (64, 128, 256)
+# A 32^3 step takes 76 us with 0 (staged) and about 330 with a named tile.
+CANDIDATES = (0, 64, 128, 256)
 
 
 def autotune_tiles(batch: PatchBatch, params: Params, candidates=CANDIDATES, reps=2):
