@@ -484,14 +484,17 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const unsigned char *__r
 }
 
 // Adam on the FP32 master weights; each weight's new value goes straight into
-// its places in the blob (the padding columns keep the zeros of the first
-// packing), which was a launch of its own.
+// its places in the blob, and the first threads write the padding columns of W1
+// (zeros), so the step leaves the blob that mlp_pack_kernel would, whatever it
+// held before, without that launch.
 __global__ void mlp_adam_kernel(float *__restrict__ m, float *__restrict__ mo, float *__restrict__ vo,
                                 const float *__restrict__ g, int step, float lr, float b1, float b2, float eps,
                                 unsigned char *__restrict__ blob)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kMlpParams) return;
+    constexpr int kPad = 16 - kMlpIn;
+    if (i < kMlpHidden * kPad) st_bf16(blob + kBlobW1, tile_off(i / kPad, kMlpIn + i % kPad, 16), 0.0f);
     const float gi = g[i];
     const float mi = b1 * mo[i] + (1.0f - b1) * gi;
     const float vi = b2 * vo[i] + (1.0f - b2) * gi * gi;
