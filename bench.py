@@ -169,21 +169,29 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-def measured_traffic(cells_per_sweep, kernel):
-    """DRAM bytes per sweep launch from the committed ncu capture of `kernel`,
-    scaled by the cells a launch processes; None when there is no capture of
-    that kernel or its source changed since."""
+def _capture(name):
+    """The committed ncu record profiles/<name>, or None when it is missing or a
+    source its figures depend on has changed since: the record lists those
+    sources and holds the hash of their concatenation."""
     import hashlib
     try:
-        with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
+        with open(os.path.join(ROOT, "profiles", name)) as f:
             t = json.load(f)
-        if t.get("kernel") != kernel:
-            return None
-        with open(os.path.join(ROOT, t["source"]), "rb") as f:
-            sha = hashlib.sha256(f.read()).hexdigest()[:16]
+        h = hashlib.sha256()
+        for src in t["sources"]:
+            with open(os.path.join(ROOT, src), "rb") as f:
+                h.update(f.read())
+        return t if h.hexdigest()[:16] == t["sources_sha256_16"] else None
     except (OSError, KeyError, ValueError):
         return None
-    if sha != t["source_sha256_16"]:
+
+
+def measured_traffic(cells_per_sweep, kernel):
+    """DRAM bytes per sweep launch from the committed ncu capture of `kernel`,
+    scaled by the cells a launch processes; None when there is no current
+    capture of that kernel."""
+    t = _capture("traffic.json")
+    if t is None or t.get("kernel") != kernel:
         return None
     return float(t["bytes_per_cell_sweep"]) * cells_per_sweep
 
@@ -192,16 +200,10 @@ def issue_bound(value_mcu, sm_mhz, sms=152):
     """The learned sweep's issue bound: warp instructions per cell-sweep from the
     committed ncu capture (null once the kernel source changed), against 4
     schedulers x 1 warp instruction per clock per SM at the sampled SM clock."""
-    import hashlib
-    try:
-        with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
-            t = json.load(f)
-        with open(os.path.join(ROOT, t["source"]), "rb") as f:
-            if hashlib.sha256(f.read()).hexdigest()[:16] != t["source_sha256_16"]:
-                return None
-        wi = float(t["warp_instr_per_cell_sweep"])
-    except (OSError, KeyError, ValueError):
+    t = _capture("traffic.json")
+    if t is None or "warp_instr_per_cell_sweep" not in t:
         return None
+    wi = float(t["warp_instr_per_cell_sweep"])
     peak = sms * 4 * sm_mhz * 1e6                    # warp instructions per second
     bound = peak / (3 * wi) / 1e6                    # Mcell-updates/s at 100% issue
     return {"warp_instr_per_cell_sweep": wi, "issue_active_ncu": t.get("issue_active"),
@@ -257,16 +259,10 @@ def fp64_alu_roofline(value_mcu, probe):
     thread instructions per cell-sweep from the committed ncu capture (null
     once the kernel source changed) times the measured cell-sweeps per second,
     against the DFMA rate the probe measured in the same run."""
-    import hashlib
-    try:
-        with open(os.path.join(ROOT, "profiles", "fp64_alu.json")) as f:
-            t = json.load(f)
-        with open(os.path.join(ROOT, t["source"]), "rb") as f:
-            if hashlib.sha256(f.read()).hexdigest()[:16] != t["source_sha256_16"]:
-                return None
-        per = float(t["fp64_arith_thread_inst_per_cell_sweep"])
-    except (OSError, KeyError, ValueError):
+    t = _capture("fp64_alu.json")
+    if t is None:
         return None
+    per = float(t["fp64_arith_thread_inst_per_cell_sweep"])
     peak = probe["dfma"]["ops_per_s"]
     achieved = per * 3 * value_mcu * 1e6
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "FP64 thread-instructions/s",
