@@ -128,6 +128,8 @@ __global__ void __launch_bounds__(128) interp_ghosts_kernel(const __grid_constan
         const enzo_patch P = a.fine[B.dst];
         const enzo_patch PP = a.par[L.parent];
         const enzo_patch_link PL = a.plink[L.parent];
+        // (an empty box has no children, but up to one parent cell along the axis)
+        if (B.hi[0] <= B.lo[0] || B.hi[1] <= B.lo[1] || B.hi[2] <= B.lo[2]) continue;
         int G0[3], m[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
