@@ -72,7 +72,8 @@ struct SweepArgs {
     double *ge = nullptr;      // gas energy of the dual-energy option, else nullptr
 };
 
-// Tiles of a sweep along dir for one patch: ceil(pencils / kSweepThreads).
+// Cross-section of a sweep along dir over one patch: its pencils are the positions
+// [lo, hi) of the two other axes (lo, hi along dir are the active cells).
 __host__ __device__ inline void sweep_ranges(const enzo_patch &P, int dir, int cover_mask,
                                              int lo[3], int hi[3])
 {

@@ -211,7 +211,7 @@ struct alignas(1024) TrainSmem {
     unsigned char bh1[64 * 128 * 2];         // B of dW2: rows in, cols sample (H1^T)
     unsigned char adw1[128 * 128 * 2];       // A of dW1: rows hidden (64 used), cols sample (dZ1^T)
     unsigned char bx[16 * 128 * 2];          // B of dW1: rows input (6 used), cols sample (X^T)
-    float gsmall[4 * 64 + 4];                // (unused), db2, dw3, db3 partial sums
+    float gsmall[2 * 64 + 4];                // db2, dw3, db3 partial sums
     float part[2][128];                      // each half's part of the output unit
     float loss;
 };
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const unsigned char *__r
     load_tile(T.w2t, blob + kBlobW2T, sizeof(T.w2t));
     const float *f = reinterpret_cast<const float *>(blob + kBlobF32);
     for (int i = tid; i < 193; i += blockDim.x) S.bias[i] = f[i];
-    for (int i = tid; i < 4 * 64 + 4; i += blockDim.x) T.gsmall[i] = 0.0f;
+    for (int i = tid; i < 2 * 64 + 4; i += blockDim.x) T.gsmall[i] = 0.0f;
     // rows 64..127 of the weight-gradient A tiles (the second half of each) stay zero
     for (int i = tid; i < (int)(sizeof(T.adw2) / 32); i += blockDim.x) {
         reinterpret_cast<uint4 *>(T.adw2)[sizeof(T.adw2) / 32 + i] = make_uint4(0, 0, 0, 0);
@@ -402,12 +402,12 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const unsigned char *__r
         {
             const int lane = tid & 31;
             const float sb = column_sums(z2), s3 = column_sums(h2);
-            atomicAdd(&T.gsmall[64 + c0 + lane], sb);
-            atomicAdd(&T.gsmall[128 + c0 + lane], s3);
+            atomicAdd(&T.gsmall[c0 + lane], sb);
+            atomicAdd(&T.gsmall[64 + c0 + lane], s3);
             float sdy = half == 0 ? dy : 0.0f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) sdy += __shfl_xor_sync(0xffffffffu, sdy, o);
-            if (half == 0 && lane == 0) atomicAdd(&T.gsmall[192], sdy);
+            if (half == 0 && lane == 0) atomicAdd(&T.gsmall[128], sdy);
         }
         if (__syncthreads_or(!mbar_wait(&S.mbar, phase))) { S.error = 1; break; }
         phase ^= 1u;
@@ -472,10 +472,10 @@ __global__ void __launch_bounds__(256) mlp_train_kernel(const unsigned char *__r
     fence_before();
     __syncthreads();
     if (!S.error) {
-        if (tid < 64) atomicAdd(&grad[kMB2 + tid], T.gsmall[64 + tid]);
-        else if (tid < 128) atomicAdd(&grad[kMW3 + tid - 64], T.gsmall[64 + tid]);
+        if (tid < 64) atomicAdd(&grad[kMB2 + tid], T.gsmall[tid]);
+        else if (tid < 128) atomicAdd(&grad[kMW3 + tid - 64], T.gsmall[tid]);
         else if (tid == 128) {
-            atomicAdd(&grad[kMB3], T.gsmall[192]);
+            atomicAdd(&grad[kMB3], T.gsmall[128]);
             atomicAdd(loss, T.loss * inv_n);
         }
     }

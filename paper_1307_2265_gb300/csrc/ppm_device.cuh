@@ -1448,11 +1448,11 @@ struct Marcher {
     double *reg_bnd;      // this pencil's boundary-face register pair, or nullptr
     // WRAP: the initial state of the first three active cells (and their eps
     // with dual energy), which the trailing ghost positions reuse after the
-    // pencil has updated those cells.  FP32 keeps them in shared memory (the
-    // kernel's per-thread slots, stride kSave), FP64 in registers.
+    // pencil has updated those cells.  In shared memory: the kernel's per-thread
+    // slots, kSave values each.
     float *wsave;
     static constexpr int kSave = EXT == 2 ? 7 : 6;   // r, u, p, t1, t2, c (and eps with dual energy)
-    // FP32 march with the plain guess: the raw FP64 values (rho, m_n, m_t1,
+    // March with the plain guess: the raw FP64 values (rho, m_n, m_t1,
     // m_t2, E, and ge with dual energy) of the last kRingSlots positions, in
     // shared memory ([slot][field] x blockDim.x, this thread's column), so the
     // update of a cell four steps after its load and the fallback test read
@@ -1651,18 +1651,12 @@ struct Marcher {
     // Fallback mode 2 (EXT kernels): does the Godunov update of cell s with face
     // fluxes Fm, Fp leave rho <= 0 or a non-positive internal energy (tested as
     // 2 rho E - |m|^2 <= 0)?  Decided in FP64 on the exact update the cell would
-    // get: the FP64 flux difference, or the FP32 path's widened increments.
-    template <bool RING = false>
-    __device__ __forceinline__ bool fails_full(int s, const R Fm[5], const R Fp[5], R dtdx, double dtdx64) const
+    // get (its raw values are in the ring).
+    __device__ __forceinline__ bool fails_full(int s, const R Fm[5], const R Fp[5], R dtdx) const
     {
-        const int64_t idx = pc.at(s);
-        const int map[5] = {0, 1 + DIR, 1 + A1, 1 + A2, 4};
         double u[5];
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
-        {
-            const double U = RING ? ring(s, v) : a.U[map[v]][idx];
-            u[v] = (U + f2d_exact((float)(dtdx * Fm[v]))) - f2d_exact((float)(dtdx * Fp[v]));
-        }
+            u[v] = (ring(s, v) + f2d_exact((float)(dtdx * Fm[v]))) - f2d_exact((float)(dtdx * Fp[v]));
         return fails_state(u);
     }
 
@@ -1680,10 +1674,9 @@ struct Marcher {
     // the cell then becomes the pending one, and the previous pending cell,
     // whose right neighbour this is, is resynchronised and written.
     template <bool RING = false>
-    __device__ __forceinline__ void update(int s, const R Fm[5], const R Fp[5], double dtdx64,
-                                           const double Gm[5], const double Gp[5], bool fb,
-                                           Counters &cnt, const GeFace *gm = nullptr,
-                                           const GeFace *gp = nullptr, R pz = (R)0, R dtdx = (R)0)
+    __device__ __forceinline__ void update(int s, const double Gm[5], const double Gp[5], bool fb, Counters &cnt,
+                                           const GeFace *gm = nullptr, const GeFace *gp = nullptr, R pz = (R)0,
+                                           R dtdx = (R)0)
     {
         const int64_t idx = pc.at(s);
         double u[5];
@@ -1766,20 +1759,20 @@ struct Marcher {
     // One pencil with the plain guess: a sliding window over the zones; march
     // step kk loads zone kk and solves interface (kk-3)+1/2.
     template <class GS>
-    __device__ void run(R dtdx, double dtdx64, const MethodParams &mp, Counters &cnt, GS &guess)
+    __device__ void run(R dtdx, const MethodParams &mp, Counters &cnt, GS &guess)
     {
         constexpr bool RING = true;             // the shared-memory ring of raw values
         const int L = pc.L;
         const bool fb = mp.fallback != 0;
         Zone<R> zm2, zm1, z0;                 // zones k-2, k-1, k
         R dprev[5], qfprev[5], sLprev[5];
-        R Fgprev[5], Fuprev2[5];
-        double Gprev2[5];                     // FP32 path: widened face term of Fuprev2
+        R Fgprev[5];
+        double Gprev2[5];                     // widened flux of the face before last
         R rho3 = (R)0, rho2 = (R)0, rho1 = (R)0, rho0 = (R)0;   // FP32: raw densities of cells k-3..k
         bool badprev = false;
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
         {
-            dprev[v] = qfprev[v] = sLprev[v] = Fgprev[v] = Fuprev2[v] = (R)0;
+            dprev[v] = qfprev[v] = sLprev[v] = Fgprev[v] = (R)0;
             Gprev2[v] = 0.0;
         }
         z0 = zm1 = zm2 = Zone<R>{};
@@ -1914,7 +1907,7 @@ struct Marcher {
                                     // (always with dual energy: the zone pressure may come
                                     // from the gas energy, not from E)
                                     bad = (dual || !clearly_ok<R>(k, zm3, Fgprev, Fg, dtdx))
-                                              ? fails_full<RING>(c, Fgprev, Fg, dtdx, dtdx64) : false;
+                                              ? fails_full(c, Fgprev, Fg, dtdx) : false;
                                 } else {
                                     // FP32 screen; cells near zero are decided in FP64
                                     const R rt = rho3 + dtdx * (Fgprev[0] - Fg[0]);
@@ -1939,14 +1932,10 @@ struct Marcher {
                                 record(kk - 6, G1, f2d_exact((float)(dtdx * gfin.F)));
                             else record(kk - 6, G1);
                             if (kk >= 7)
-                                update<RING>(kk - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt,
+                                update<RING>(kk - 4, Gprev2, G1, fb, cnt,
                                              dual ? &gfin2 : nullptr, &gfin, p4, dtdx);
                             gfin2 = gfin;
-                            _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                            {
-                                Fuprev2[v] = Fu1[v];
-                                Gprev2[v] = G1[v];
-                            }
+                            _Pragma("unroll") for (int v = 0; v < 5; ++v) Gprev2[v] = G1[v];
                             badprev = bad;
                         }
                         _Pragma("unroll") for (int v = 0; v < 5; ++v) Fgprev[v] = Fg[v];
@@ -1975,7 +1964,7 @@ struct Marcher {
             record(pc.n, G1, f2d_exact((float)(dtdx * gfin.F)));
         else record(pc.n, G1);
         // the pressure of zone L-4 is the last window's zone k-3
-        update<RING>(L - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt, dual ? &gfin2 : nullptr, &gfin, zm3.p, dtdx);
+        update<RING>(L - 4, Gprev2, G1, fb, cnt, dual ? &gfin2 : nullptr, &gfin, zm3.p, dtdx);
         if (dual) ge_commit(Eghost_right);
     }
 
@@ -2005,7 +1994,7 @@ struct Marcher {
     // steps in a shared-memory ring while the tensor core evaluates the
     // network, and the pencil takes D extra drain steps).
     template <class GS>
-    __device__ void run_piped(R dtdx, double dtdx64, const MethodParams &mp, Counters &cnt, GS &guess)
+    __device__ void run_piped(R dtdx, const MethodParams &mp, Counters &cnt, GS &guess)
     {
         constexpr int D = GS::kDepth;
         static_assert(D == 2, "the state ring holds two steps");
@@ -2021,14 +2010,14 @@ struct Marcher {
         const bool fb = mp.fallback != 0;
         Zone<R> zm2, zm1, z0;                 // zones k-2, k-1, k
         R dprev[5], qfprev[5], sLprev[5];
-        R Fgprev[5], Fuprev2[5];
-        double Gprev2[5];                     // FP32 path: widened face term of Fuprev2
+        R Fgprev[5];
+        double Gprev2[5];                     // widened flux of the face before last
         R rh[6];                              // FP32: raw densities of cells kk..kk-5
         bool qh1 = false, qh2 = false;        // the ring slots hold states of interfaces 1 / 2 steps back
         bool badprev = false;
         _Pragma("unroll") for (int v = 0; v < 5; ++v)
         {
-            dprev[v] = qfprev[v] = sLprev[v] = Fgprev[v] = Fuprev2[v] = (R)0;
+            dprev[v] = qfprev[v] = sLprev[v] = Fgprev[v] = (R)0;
             Gprev2[v] = 0.0;
         }
         _Pragma("unroll") for (int i = 0; i < 6; ++i) rh[i] = (R)0;
@@ -2145,12 +2134,8 @@ struct Marcher {
                 double G1[5];
                 widen(Fu1, dtdx, G1);
                 record(jj - 6, G1);
-                if (jj >= 7) update(jj - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt);
-                _Pragma("unroll") for (int v = 0; v < 5; ++v)
-                {
-                    Fuprev2[v] = Fu1[v];
-                    Gprev2[v] = G1[v];
-                }
+                if (jj >= 7) update(jj - 4, Gprev2, G1, fb, cnt);
+                _Pragma("unroll") for (int v = 0; v < 5; ++v) Gprev2[v] = G1[v];
                 badprev = bad;
             }
             _Pragma("unroll") for (int v = 0; v < 5; ++v) Fgprev[v] = Fg[v];
@@ -2168,7 +2153,7 @@ struct Marcher {
         double G1[5];
         widen(Fu1, dtdx, G1);
         record(pc.n, G1);
-        update(L - 4, Fuprev2, Fu1, dtdx64, Gprev2, G1, fb, cnt);
+        update(L - 4, Gprev2, G1, fb, cnt);
     }
 };
 
@@ -2198,8 +2183,8 @@ __host__ __device__ constexpr size_t learned_smem_bytes()
     return learned_ring_offset() + (DIR != 0 ? 3 * 5 * kSweepThreads * sizeof(double) : 0);
 }
 
-// Persistent sweep kernel: CTAs take (patch, 128-pencil tile) work items from a
-// device counter until the batch is exhausted.  DIR is the sweep axis.
+// Persistent sweep kernel: CTAs take (patch, tile of THREADS pencils) work items
+// from a device counter until the batch is exhausted.  DIR is the sweep axis.
 #ifndef ENZO_SWEEP_MIN_BLOCKS_FP32
 #define ENZO_SWEEP_MIN_BLOCKS_FP32 4   // 128 registers per thread: 16 warps per SM
 #endif
@@ -2220,12 +2205,13 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (EXT ==
 {
     constexpr int A1 = DIR == 0 ? 1 : 0, A2 = DIR == 2 ? 1 : 2;
     __shared__ int s_tile;
-    // FP32: per-thread slots for the wrapped pencils' first three cells
+    // per-thread slots for the wrapped pencils' first three cells
     __shared__ float s_wrap[3 * (EXT == 2 ? 7 : 6) * THREADS];
     extern __shared__ __align__(16) unsigned char dsmem[];
-    // plain FP32 default kernels: the ring of raw values in dynamic shared memory
+    // dynamic shared memory: the ring of raw values; learned, the network and then
+    // (y and z) the staged loads
     double *uring = nullptr;
-    if constexpr (ring_bytes<R, THREADS, EXT, DIR>() > 0 && !LEARNED) uring = reinterpret_cast<double *>(dsmem) + threadIdx.x;
+    if constexpr (!LEARNED) uring = reinterpret_cast<double *>(dsmem) + threadIdx.x;
     if constexpr (LEARNED && DIR != 0) uring = reinterpret_cast<double *>(dsmem + learned_ring_offset()) + threadIdx.x;
     Counters cnt;
     cnt.st = a.status;
@@ -2260,8 +2246,7 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (EXT ==
         pc.L = P.n[DIR] + 2 * P.ng;
         pc.ng = P.ng;
         pc.n = P.n[DIR];
-        const double dtdx64 = x64::div(dt, P.dx[DIR]);   // off the FP64 pipe
-        const R dtdx = (R)dtdx64;
+        const R dtdx = (R)x64::div(dt, P.dx[DIR]);   // off the FP64 pipe
         if (valid) interfaces += (unsigned long long)(P.n[DIR] + 1);
         const unsigned key = (unsigned)lo * 7919u + (unsigned)pe;
         // flux register rows of this pencil (active transverse position only)
@@ -2287,12 +2272,12 @@ __global__ void __launch_bounds__(THREADS, LEARNED ? ENZO_LEARNED_CTAS : (EXT ==
         cnt.st = valid ? a.status : nullptr;
         if (P.flags & ENZO_PATCH_PERIODIC) {
             Marcher<R, true, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, s_wrap + threadIdx.x, uring};
-            if constexpr (LEARNED) m.run_piped(dtdx, dtdx64, a.mp, cnt, guess);
-            else m.run(dtdx, dtdx64, a.mp, cnt, guess);
+            if constexpr (LEARNED) m.run_piped(dtdx, a.mp, cnt, guess);
+            else m.run(dtdx, a.mp, cnt, guess);
         } else {
             Marcher<R, false, DIR, REG, EXT> m{a, pc, k, valid, key, reg_all, reg_bnd, s_wrap + threadIdx.x, uring};
-            if constexpr (LEARNED) m.run_piped(dtdx, dtdx64, a.mp, cnt, guess);
-            else m.run(dtdx, dtdx64, a.mp, cnt, guess);
+            if constexpr (LEARNED) m.run_piped(dtdx, a.mp, cnt, guess);
+            else m.run(dtdx, a.mp, cnt, guess);
         }
     }
     if constexpr (LEARNED) {
@@ -2458,7 +2443,6 @@ template <class R, int DIR, int THREADS, bool REG, int EXT = 0>
 cudaError_t ring_prepare(int dev)
 {
     constexpr int bytes = ring_bytes<R, THREADS, EXT, DIR>();
-    if (bytes == 0) return cudaSuccess;
     static bool done[64] = {false};
     if (dev < 0 || dev >= 64) dev = 0;
     if (done[dev]) return cudaSuccess;

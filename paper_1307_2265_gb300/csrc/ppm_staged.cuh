@@ -61,6 +61,7 @@ struct Staged {
     using Smem = StagedSmem<R, THREADS, EXT>;
     static constexpr int NV = Smem::NV;
     static constexpr bool dual = EXT == 2;
+    static_assert(!dual || sizeof(R) == 8, "FP32 dual-energy sweeps march");
     const SweepArgs &a;
     const enzo_patch &P;
     Smem &S;
@@ -107,7 +108,7 @@ struct Staged {
         return Zone<R>{S.q[0][z], S.q[1][z], S.q[2][z], S.q[3][z], S.q[4][z], S.q[5][z]};
     }
 
-    __device__ __forceinline__ double widen1(R F) const
+    __device__ __forceinline__ double widen(R F) const
     {
         return sizeof(R) == 8 ? (double)F : f2d_exact((float)(dtdx * F));
     }
@@ -120,12 +121,6 @@ struct Staged {
         if (x64::less(emax, E)) emax = E;
         if (x64::less(emax, Er)) emax = Er;
         return ok && x64::less(0.1 * emax, e) ? e : g;
-    }
-
-    __device__ __forceinline__ void widen(const R F[5], double G[5]) const
-    {
-        _Pragma("unroll") for (int v = 0; v < 5; ++v)
-            G[v] = sizeof(R) == 8 ? (double)F[v] : f2d_exact((float)(dtdx * F[v]));
     }
 
     // Flux registers of face f (left of active cell f) of pencil p, as the
@@ -152,7 +147,7 @@ struct Staged {
         if (P.freg_bnd >= 0 && (f == 0 || f == n)) {
             double *o = a.freg + P.freg_bnd + obnd + (row * 2 + (f == 0 ? 0 : 1)) * NV;
             _Pragma("unroll") for (int v = 0; v < 5; ++v) o[v] = o[v] + (sizeof(R) == 8 ? dt64 * G[v] : G[v]);
-            if constexpr (dual) o[5] = o[5] + (sizeof(R) == 8 ? dt64 * gG : gG);
+            if constexpr (dual) o[5] = o[5] + dt64 * gG;
         }
     }
 
@@ -358,19 +353,18 @@ struct Staged {
                 bool bad = false;
                 if (EXT && a.mp.fallback == 2) {
                     // FP32: a screen on the zone's own primitives with wide margins; unclear
-                    // cells (with dual energy all) take the exact test on the update they
-                    // would get
+                    // cells take the exact test on the update they would get
                     R Fm[5], Fp[5];
                     _Pragma("unroll") for (int v = 0; v < 5; ++v)
                     {
                         Fm[v] = S.B[v][z - e];
                         Fp[v] = S.B[v][z];
                     }
-                    if (sizeof(R) == 8 || dual || !clearly_ok<R>(k, zone(z), Fm, Fp, dtdx)) {
+                    if (sizeof(R) == 8 || !clearly_ok<R>(k, zone(z), Fm, Fp, dtdx)) {
                         double u[5];
                         _Pragma("unroll") for (int v = 0; v < 5; ++v)
                             u[v] = sizeof(R) == 8 ? cell_update(S.U[v][z], dtdx64, (double)Fm[v], (double)Fp[v])
-                                                  : (S.U[v][z] + widen1(Fm[v])) - widen1(Fp[v]);
+                                                  : (S.U[v][z] + widen(Fm[v])) - widen(Fp[v]);
                         bad = fails_state(u);
                     }
                 } else if (sizeof(R) == 8) {
@@ -430,10 +424,10 @@ struct Staged {
             }
             _Pragma("unroll") for (int v = 0; v < 5; ++v)
             {
-                Gm[v] = widen1(Fm[v]);
-                Gp[v] = widen1(Fp[v]);
+                Gm[v] = widen(Fm[v]);
+                Gp[v] = widen(Fp[v]);
             }
-            const double ggm = dual ? widen1(gm) : 0.0, ggp = dual ? widen1(gp) : 0.0;
+            const double ggm = (double)gm, ggp = (double)gp;
             if (REG) {
                 record(p, s - ng, Gm, ggm);
                 if (s == L - ng - 1) record(p, n, Gp, ggp);
@@ -446,18 +440,9 @@ struct Staged {
             if constexpr (dual) {
                 const double g0 = S.ge[z];
                 const R pz = S.q[2][z];
-                if (sizeof(R) == 8)
-                    gnew = (g0 + dtdx64 * (ggm - ggp)) - dtdx64 * (double)pz * ((double)up - (double)um);
-                else gnew = ((g0 + ggm) - ggp) - f2d_exact((float)(dtdx * pz * (up - um)));
+                gnew = (g0 + dtdx64 * (ggm - ggp)) - dtdx64 * (double)pz * ((double)up - (double)um);
                 ok = x64::gt0(u[0]);
-                if (ok) {
-                    if (sizeof(R) == 8) {
-                        enew = u[4] - x64::div<-1>((u[1] * u[1] + u[2] * u[2]) + u[3] * u[3], u[0], x64::recip(u[0]));
-                    } else {
-                        const float r = d2f_rz(u[0]), m0 = d2f_rz(u[1]), m1 = d2f_rz(u[2]), m2 = d2f_rz(u[3]);
-                        enew = u[4] - f2d_exact((R)0.5 * ((m0 * m0 + m1 * m1) + m2 * m2) / r);
-                    }
-                }
+                if (ok) enew = u[4] - x64::div<-1>((u[1] * u[1] + u[2] * u[2]) + u[3] * u[3], u[0], x64::recip(u[0]));
             }
             if (fb && (EXT && a.mp.fallback == 2 ? fails_state(u) : !x64::gt0(u[0]))) cnt.rare(ENZO_ST_NEG_AFTER);
             if (x64::is_nan(u[0]) || x64::is_nan(u[4])) cnt.rare(ENZO_ST_NAN);
