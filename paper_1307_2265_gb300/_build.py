@@ -1,7 +1,7 @@
 """Build of libenzo_ppm.so for sm_103a with nvcc (in-tree, no cmake).
 
 Translation units and their flags:
-  abi.cu        host entry points, work lists, ghost fill, CFL finalisation
+  abi.cu        host entry points, work lists, ghost fill, packing
   fp64_path.cu  FP64 sweep/CFL/Riemann: --fmad=false, IEEE div and sqrt
   fp32_path.cu  FP32 sweep/CFL/Riemann: -use_fast_math (FMA, fast rcp/sqrt)
   noalloc.cu    sweep entry point whose scratch is a library-owned device array

@@ -1462,7 +1462,8 @@ struct Marcher {
     // k+kStage at step k.  The option and dual-energy kernels, which loaded
     // each zone when they needed it and again for its update, took 10.0 and
     // 14.3 ms a step of a 1000-patch level; with the ring 8.7 and 12.4, and
-    // their spills fell from 72..88 to 16..28 B.
+    // their spill stores fell from 72..88 B to 12..28 (28..56 in the option
+    // kernels with flux registers).
     double *uring;
     static constexpr int kRingSlots = DIR == 0 ? 5 : 8;
     static constexpr int kStage = 3;
