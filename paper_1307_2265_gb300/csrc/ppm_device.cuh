@@ -50,7 +50,9 @@ namespace enzo {
 // sum it fuses) can differ from kernel to kernel.  The functions below that
 // take PIN state the choice when it is true: the one the marching kernels are
 // compiled to, found by comparing results, so that the staged kernels give
-// the march's values bit for bit.
+// the march's values bit for bit.  (The march's own forms stay the compiler's:
+// stated there too they give the same values, but a step of the 4000-patch level
+// takes 31.3 ms instead of 29.7.)
 //
 // a b + c d: OPT 0 rounds c d, 1 rounds a b, 2 rounds both products.
 template <int OPT>
