@@ -116,8 +116,8 @@ struct InterpArgs {
 // was formed up to eight times.  gridDim.y blocks share a box, so that a level
 // of few boxes still fills the chip.  Latency-bound; on a 64^3 root with three
 // levels (about 250 boxes per launch) a launch took 269 us with one thread per
-// child and one CTA per box, 83 us by parent cell, and about 45 us with the
-// boxes spread; the ghost fills of a root step now take 3.6 ms.
+// child and one CTA per box, 83 us by parent cell, and 42 us with the boxes
+// spread.
 template <class T>
 __global__ void __launch_bounds__(128) interp_ghosts_kernel(const __grid_constant__ InterpArgs a)
 {
